@@ -9,6 +9,7 @@ picks (TF32 tensor cores or FP32).
 from __future__ import annotations
 
 import math
+import weakref
 
 import torch
 
@@ -199,8 +200,8 @@ class _Layer:
 
     def __init__(self, L, gen, dev, stream, pointwise_out=0):
         N, Ci, H, W, Co, k, s, p, d, g = L
-        self.desc = None
         self.desc = gconv.gconv_desc_create_2d(N, Ci, H, W, Co, k[0], k[1], s[0], s[1], p[0], p[1], d[0], d[1], g)
+        weakref.finalize(self, gconv.gconv_desc_destroy, self.desc)
         Ho, Wo = gconv.gconv_out_shape(self.desc)
         w = torch.randn((Co, Ci // g, k[0], k[1]), generator=gen, device=dev).mul_(math.sqrt(2.0 / (Ci // g * k[0] * k[1])))
         self.c2 = pointwise_out
@@ -213,10 +214,6 @@ class _Layer:
             gconv.gconv_pack_weights(self.desc, w, self.wp, stream)
             self.workspace = attach_workspace(self.desc, dev)
         self.y = torch.empty((N, self.c2 or Co, Ho, Wo), device=dev)
-
-    def __del__(self):
-        if self.desc is not None:
-            gconv.gconv_desc_destroy(self.desc)
 
 
 def prepare(case, seed):
