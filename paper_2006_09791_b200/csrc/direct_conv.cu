@@ -1,0 +1,448 @@
+// FP32 direct grouped convolution for any filter size, stride, padding and dilation (DIRECT_GENERIC, and the 3x3 layers of
+// DIRECT_TILED that neither the depthwise nor the narrow-group kernel takes).
+//
+// What bounds these layers is the FP32 pipe (a group's filters times its taps are done on every staged pixel), so the
+// kernel is built to keep it fed.  A CTA owns a tile of output pixels (NI images x TH rows x TW columns) and BM filters
+// of one group; it stages the input patch of CC channels and their weights in shared memory (cp.async, two buffers, zero
+// fill outside the image), and every thread accumulates TM filters x TN pixels in registers:
+//   * a warp's 32 lanes are 32 consecutive pixels of the tile, so an input value is one conflict-free LDS.32 whatever the
+//     tap (with a column stride the patch's columns are stored phase by phase: lanes stay one float apart), and the TM
+//     weights of a tap are a broadcast LDS.128 of TM/4 vectors;
+//   * two filters share one fma.rn.f32x2 (each half is an ordinary FP32 FMA): TM x TN = 64 products are 32 issue slots, 8
+//     shared-memory loads and 4 register pairings, so the pipe, not instruction issue, is the limit;
+//   * the taps of a chunk are one flat loop over (channel, row, column) with a table of patch offsets: any filter shape
+//     runs the same loop.
+// Where the tiles do not fill the chip (small planes, small batches, many channels) the channels are split over the CTAs
+// of a cluster; each leaves its partial sums in its own shared memory and every CTA adds up one slice over distributed
+// shared memory, in rank order (deterministic, no workspace).
+//
+// Measured against the kernels it replaced (one thread per output; a fixed 4-pixel tile for 3x3), N = 16: 3 -> 64 @224x224
+// 7x7 stride 2 1310 -> 113 us (34 TFLOP/s, 45 % of the FP32 peak), 64 -> 64 @56x56 dilation 2, 4 groups 461 -> 39 us,
+// 64 -> 128 @28x28 5x5 stride 2, 4 groups 138 -> 29 us, 3 -> 32 @224x224 3x3 stride 2 32 -> 23 us; 512 -> 512 @4x4 3x3 (N = 6)
+// 3197 -> 37 us.  What is left on the large ones: the FP32 pipe is active 72 % of the time (the packed FMAs, and as many
+// moves that pair their operands as shared-memory loads), and the last wave of CTAs is partly empty.
+#include <cooperative_groups.h>
+#include <math.h>
+
+#include "gconv_internal.h"
+
+namespace gconv {
+
+namespace {
+
+namespace cg = cooperative_groups;
+
+constexpr int kMaxTapTable = 1024;      // entries of the patch-offset table (channels of a chunk x taps), at most
+
+__device__ __forceinline__ void cp_async4(uint32_t dst, const float* src, bool ok) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(ok ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const float* src, bool ok) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+// Two FP32 multiply-adds in one instruction.  (Packed accumulators in 64-bit variables measured 17 % slower than this form on
+// 64 -> 64 channels @512x512, plain fmaf 16 % slower: the register pairs the compiler picks decide.)
+__device__ __forceinline__ void ffma2(float2& d, float2 a, float2 b) {
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rd, {%0, %1};\n\t"
+        "fma.rn.f32x2 rd, ra, rb, rd;\n\t"
+        "mov.b64 {%0, %1}, rd;\n\t}"
+        : "+f"(d.x), "+f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+}
+
+template <int TM, int TN>
+__global__ void __launch_bounds__(256, TM * TN > 64 ? 1 : 2)
+direct_conv_kernel(const Shape s, const ConvCfg c, const float* __restrict__ x, const uint32_t* __restrict__ packed,
+                   float* __restrict__ y, Status* status, uint32_t tag) {
+    extern __shared__ __align__(16) float conv_smem[];
+    if (__ldg(packed) != tag) {                           // uniform across the grid
+        if (threadIdx.x == 0) record_status(status, GCONV_ERR_PACK_MISMATCH, (int)blockIdx.x);
+        return;
+    }
+    const float* __restrict__ wpk = reinterpret_cast<const float*>(packed + kHeaderBytes / 4);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, threads = (int)blockDim.x;
+    const int wn = warp / c.WM, wm = warp - wn * c.WM;
+    const int BM = c.WM * TM, BN = c.WN * TN * 32;
+
+    // ---- which tile: filter block fastest (the CTAs that read the same patch run together), then group, column, row, image
+    uint32_t b = blockIdx.x, rank = 0, kb, g, tx, ty;
+    if (c.split > 1) {
+        rank = b % (uint32_t)c.split;
+        b /= (uint32_t)c.split;
+    }
+    kb = b % (uint32_t)c.kblocks; b /= (uint32_t)c.kblocks;
+    g = b % (uint32_t)s.groups;   b /= (uint32_t)s.groups;
+    tx = b % (uint32_t)c.tiles_x; b /= (uint32_t)c.tiles_x;
+    ty = b % (uint32_t)c.tiles_y; b /= (uint32_t)c.tiles_y;
+    const int n0 = (int)b * c.NI, p0 = (int)ty * c.TH, q0 = (int)tx * c.TW, kb0 = (int)kb * BM;
+    const int in_y0 = p0 * s.stride - s.pad, in_x0 = q0 * s.stride_w - s.pad_w;
+    // rows are staged from a multiple of four columns on where whole 16-byte vectors can be copied
+    const int shift = c.vec ? (in_x0 & 3) : 0;
+    const int col0 = in_x0 - shift;
+
+    float* const s_in = conv_smem;                                       // [stages][NI][CC][PH][pitch]
+    float* const s_w = conv_smem + c.stages * c.in_floats;               // [stages][CC * taps][BM]
+    int* const s_off = reinterpret_cast<int*>(s_w + c.stages * c.w_floats);   // [CC * taps] patch offset of a tap
+
+    const int taps = s.KH * s.KW;
+    for (int i = tid; i < c.CC * taps; i += threads) {
+        const int ch = i / taps, rs = i - ch * taps;
+        const int r = rs / s.KW, v = (rs - r * s.KW) * s.dilation_w;
+        s_off[i] = ch * c.plane + r * s.dilation * c.pitch + (v % s.stride_w) * c.phase + v / s.stride_w;
+    }
+
+    // ---- staging ---------------------------------------------------------------------------------------------------
+    const size_t HW = (size_t)s.H * s.W;
+    const float* const xg = x + ((size_t)n0 * s.C_in + (size_t)g * s.Cg) * HW;
+    const float* const wg = wpk + (size_t)g * s.Cg * taps * s.Kg + kb0;
+    const int row_first = tid / c.lpr, row_step = threads / c.lpr, row_lane = tid % c.lpr;
+    auto load = [&](int chunk, int buf) {
+        const int c0 = chunk * c.CC, cc = min(c.CC, s.Cg - c0);
+        const uint32_t in_dst = (uint32_t)__cvta_generic_to_shared(s_in + buf * c.in_floats);
+        for (int row = row_first; row < c.NI * c.CC * c.PH; row += row_step) {
+            uint32_t t, ih, ni, ch;
+            c.div_ph.divmod((uint32_t)row, t, ih);
+            c.div_cc.divmod(t, ni, ch);
+            if ((int)ch >= cc) continue;
+            const int h = in_y0 + (int)ih;
+            const bool row_ok = h >= 0 && h < s.H && n0 + (int)ni < s.N;
+            const float* src = row_ok ? xg + ((size_t)ni * s.C_in + (size_t)(c0 + (int)ch)) * HW + (size_t)h * s.W : x;
+            const uint32_t dst = in_dst + 4u * (t * (uint32_t)c.plane + ih * (uint32_t)c.pitch);
+            if (c.vec) {
+                for (int v = row_lane * 4; v < c.pitch; v += c.lpr * 4) {
+                    const bool ok = row_ok && col0 + v >= 0 && col0 + v < s.W;
+                    cp_async16(dst + 4u * (uint32_t)v, ok ? src + col0 + v : x, ok);
+                }
+            } else {
+                for (int v = row_lane; v < c.PW; v += c.lpr) {
+                    const bool ok = row_ok && col0 + v >= 0 && col0 + v < s.W;
+                    uint32_t vq, vr;
+                    c.div_sw.divmod((uint32_t)v, vq, vr);
+                    cp_async4(dst + 4u * (vr * (uint32_t)c.phase + vq), ok ? src + col0 + v : x, ok);
+                }
+            }
+        }
+        const uint32_t w_dst = (uint32_t)__cvta_generic_to_shared(s_w + buf * c.w_floats);
+        const float* wsrc = wg + (size_t)c0 * taps * s.Kg;
+        if (c.wvec) {
+            const int per = BM >> 2;
+            for (int e = tid; e < cc * taps * per; e += threads) {
+                uint32_t kk, k4;
+                c.div_bm.divmod((uint32_t)e, kk, k4);
+                const bool ok = kb0 + (int)k4 * 4 < s.Kg;
+                cp_async16(w_dst + 16u * (uint32_t)e, ok ? wsrc + (size_t)kk * s.Kg + k4 * 4 : wpk, ok);
+            }
+        } else {
+            for (int e = tid; e < cc * taps * BM; e += threads) {
+                uint32_t kk, k;
+                c.div_bm.divmod((uint32_t)e, kk, k);
+                const bool ok = kb0 + (int)k < s.Kg;
+                cp_async4(w_dst + 4u * (uint32_t)e, ok ? wsrc + (size_t)kk * s.Kg + k : wpk, ok);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
+    // ---- which pixels this thread owns -----------------------------------------------------------------------------
+    int base[TN];
+#pragma unroll
+    for (int j = 0; j < TN; ++j) {
+        uint32_t ni, rem, p, q;
+        c.div_tile.divmod((uint32_t)((wn * TN + j) * 32 + lane), ni, rem);
+        c.div_tw.divmod(rem, p, q);
+        base[j] = (int)ni < c.NI ? (int)ni * c.CC * c.plane + (int)p * s.stride * c.pitch + (int)q + shift : 0;
+    }
+
+    float2 acc[(TM + 1) / 2][TN];                          // filters 2k and 2k + 1 of pixel set j
+#pragma unroll
+    for (int k = 0; k < (TM + 1) / 2; ++k)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[k][j] = make_float2(0.f, 0.f);
+
+    const int first = (int)rank * c.per_split, last = min(first + c.per_split, c.chunks);
+    if (first < last) load(first, 0);
+    for (int chunk = first; chunk < last; ++chunk) {
+        const int buf = c.stages == 2 ? ((chunk - first) & 1) : 0;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();                                   // the chunk has landed, and everyone is done with the one before
+        if (chunk + 1 < last) load(chunk + 1, buf ^ 1);
+        const int kkn = min(c.CC, s.Cg - chunk * c.CC) * taps;
+        const float* __restrict__ in = s_in + buf * c.in_floats;
+        const float* __restrict__ wp = s_w + buf * c.w_floats + wm * TM;
+        auto tap = [&](int off, const float* __restrict__ w) {
+            float xv[TN];
+#pragma unroll
+            for (int j = 0; j < TN; ++j) xv[j] = in[base[j] + off];
+            if constexpr (TM == 1) {
+                const float wv = w[0];
+#pragma unroll
+                for (int j = 0; j < TN; ++j) acc[0][j].x = fmaf(xv[j], wv, acc[0][j].x);
+            } else {
+                float2 wv[TM / 2];
+                if constexpr (TM == 2) {
+                    wv[0] = *reinterpret_cast<const float2*>(w);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < TM / 4; ++k) {
+                        const float4 t = *reinterpret_cast<const float4*>(w + 4 * k);
+                        wv[2 * k] = make_float2(t.x, t.y);
+                        wv[2 * k + 1] = make_float2(t.z, t.w);
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < TN; ++j) {
+                    const float2 xx = make_float2(xv[j], xv[j]);
+#pragma unroll
+                    for (int k = 0; k < TM / 2; ++k) ffma2(acc[k][j], wv[k], xx);
+                }
+            }
+        };
+        int kk = 0;
+        for (; kk + 4 <= kkn; kk += 4, wp += 4 * BM) {
+            const int4 o = *reinterpret_cast<const int4*>(s_off + kk);
+            tap(o.x, wp);
+            tap(o.y, wp + BM);
+            tap(o.z, wp + 2 * BM);
+            tap(o.w, wp + 3 * BM);
+        }
+        for (; kk < kkn; ++kk, wp += BM) tap(s_off[kk], wp);
+    }
+
+    // ---- results ---------------------------------------------------------------------------------------------------
+    const size_t OHW = (size_t)s.H_out * s.W_out;
+    float* const yg = y + ((size_t)g * s.Kg + kb0) * OHW;
+    // tile pixel -> address of filter 0 of this block, nullptr for pixels outside the tile or the plane
+    auto place = [&](uint32_t pix) -> float* {
+        uint32_t ni, rem, p, q;
+        c.div_tile.divmod(pix, ni, rem);
+        c.div_tw.divmod(rem, p, q);
+        if ((int)ni >= c.NI || n0 + (int)ni >= s.N || p0 + (int)p >= s.H_out || q0 + (int)q >= s.W_out) return nullptr;
+        return yg + (size_t)(n0 + (int)ni) * s.C_out * OHW + (size_t)(p0 + (int)p) * s.W_out + (q0 + (int)q);
+    };
+    if (c.split == 1) {
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+            float* dst = place((uint32_t)((wn * TN + j) * 32 + lane));
+            if (dst == nullptr) continue;
+            dst += (size_t)(wm * TM) * OHW;
+#pragma unroll
+            for (int k = 0; k < TM; ++k) {
+                if (kb0 + wm * TM + k < s.Kg) *dst = (k & 1) ? acc[k / 2][j].y : acc[k / 2][j].x;
+                dst += OHW;
+            }
+        }
+        return;
+    }
+    cg::cluster_group cluster = cg::this_cluster();
+    __syncthreads();                                       // the partial sums reuse the staging buffers
+#pragma unroll
+    for (int j = 0; j < TN; ++j)
+#pragma unroll
+        for (int k = 0; k < TM; ++k)
+            conv_smem[(wm * TM + k) * BN + (wn * TN + j) * 32 + lane] = (k & 1) ? acc[k / 2][j].y : acc[k / 2][j].x;
+    cluster.sync();
+    const int slice = BM * BN / c.split;
+    for (int i = tid; i < slice; i += threads) {
+        const int e = (int)rank * slice + i;
+        float v = 0.f;
+        for (int r = 0; r < c.split; ++r) v += *cluster.map_shared_rank(conv_smem + e, (unsigned)r);
+        const int k = e / BN;
+        float* dst = place((uint32_t)(e - k * BN));
+        if (dst != nullptr && kb0 + k < s.Kg) dst[(size_t)k * OHW] = v;
+    }
+    cluster.sync();                                        // nobody leaves while its partial sums are still being read
+}
+
+constexpr int kSmemMax = 224 * 1024;
+
+// Fills geometry, staging and grid for one choice of (TM, TN, WM, WN, tile columns, split); false if it does not fit.
+bool conv_geometry(const Shape& s, ConvCfg& c, int TW) {
+    const int BM = c.TM * c.WM, BN = 32 * c.TN * c.WN, taps = s.KH * s.KW;
+    c.TW = TW;
+    c.TH = BN / TW < s.H_out ? BN / TW : s.H_out;
+    const int ty = (s.H_out + c.TH - 1) / c.TH;
+    c.TH = (s.H_out + ty - 1) / ty;                       // equal row blocks
+    c.NI = (c.TH == s.H_out && c.TW == s.W_out) ? BN / (c.TH * c.TW) : 1;
+    if (c.NI > s.N) c.NI = s.N;
+    c.tiles_x = (s.W_out + c.TW - 1) / c.TW;
+    c.tiles_y = ty;
+    c.tiles_n = (s.N + c.NI - 1) / c.NI;
+    c.kblocks = (s.Kg + BM - 1) / BM;
+    const long long ph = (long long)(c.TH - 1) * s.stride + (long long)(s.KH - 1) * s.dilation + 1;
+    const long long pw = (long long)(c.TW - 1) * s.stride_w + (long long)(s.KW - 1) * s.dilation_w + 1;
+    if (ph * pw > kSmemMax / 4) return false;
+    c.PH = (int)ph;
+    c.PW = (int)pw;
+    c.vec = (s.stride_w == 1 && s.W % 4 == 0) ? 1 : 0;
+    c.phase = c.vec ? ((c.PW + 3 + 3) & ~3) : (c.PW + s.stride_w - 1) / s.stride_w;
+    c.pitch = c.phase * s.stride_w;
+    c.plane = c.PH * c.pitch;
+    c.wvec = (s.Kg % 4 == 0 && BM % 4 == 0) ? 1 : 0;
+    const long long per_channel = 4LL * ((long long)c.NI * c.plane + (long long)taps * BM);
+    if (taps > kMaxTapTable) return false;
+    // a chunk of channels: two buffers of up to 48 KB (two CTAs per SM), or one that holds everything; large filters or
+    // patches take more, down to one CTA per SM
+    const int rank_channels = (s.Cg + c.split - 1) / c.split;
+    int cc = (int)(48 * 1024 / per_channel);
+    if (cc < 1 && 2 * per_channel + 8192 <= kSmemMax) cc = 1;
+    if (cc < 1 && s.Cg == 1 && per_channel + 8192 <= kSmemMax) cc = 1;
+    if (cc < 1) return false;
+    if (cc * taps > kMaxTapTable) cc = kMaxTapTable / taps;
+    if (cc >= rank_channels) {
+        c.CC = rank_channels;
+        c.per_split = 1;
+    } else {
+        c.per_split = (rank_channels + cc - 1) / cc;
+        c.CC = (rank_channels + c.per_split - 1) / c.per_split;
+    }
+    c.chunks = (s.Cg + c.CC - 1) / c.CC;
+    if ((c.split - 1) * c.per_split >= c.chunks) return false;   // every rank has work
+    c.stages = c.per_split > 1 ? 2 : 1;
+    c.in_floats = (c.NI * c.CC * c.plane + 3) & ~3;
+    c.w_floats = (c.CC * taps * BM + 3) & ~3;
+    const long long floats = (long long)c.stages * (c.in_floats + c.w_floats) + ((c.CC * taps + 3) & ~3);
+    const long long part = c.split > 1 ? (long long)BM * BN : 0;
+    const long long bytes = 4 * (floats > part ? floats : part);
+    if (bytes > kSmemMax) return false;
+    c.smem = (size_t)bytes;
+    int lpr = 1;
+    const int cols = c.vec ? c.pitch / 4 : c.PW;
+    while (lpr < cols && lpr < 32) lpr <<= 1;
+    c.lpr = lpr;
+    const long long ctas = (long long)c.tiles_x * c.tiles_y * c.tiles_n * s.groups * c.kblocks * c.split;
+    if (ctas > 0x7fffffffLL / 2) return false;
+    c.ctas = (uint32_t)ctas;
+    return true;
+}
+
+// Estimated time in SM clocks.  Per tap a warp spends FP32-pipe cycles, issue slots and shared-memory wavefronts (whichever is
+// the most dominates: a soft maximum), the staging loop and the epilogue come on top, the CTAs of an SM share it, and a CTA
+// has a critical path of its own.  The constants are a least-squares fit over 14 800 timed configurations of 18 shapes
+// (first layers on images, dilated, one-dimensional and 5x5 filters, tiny planes with 512 and 1024 channels): on those the
+// chosen configuration is at most 20 % (6 % on average) slower than the best of all.
+double conv_cost(const Shape& s, const ConvCfg& c, int sm_count) {
+    const int taps = s.KH * s.KW, warps = c.WM * c.WN, threads = 32 * warps;
+    const double BM = c.TM * c.WM, outputs = BM * c.TN * c.WN;             // outputs of the tile, in warps
+    const double ch = c.per_split * c.CC < s.Cg ? c.per_split * c.CC : s.Cg;
+    const double work = ch * taps * warps, products = c.TM * c.TN, tm4 = (c.TM + 3) / 4;
+    const double fma = work * 0.361 * products;
+    const double issue = work * 0.25 * ((c.TM == 1 ? 1.0 : 0.5) * products + 6.18 * c.TN + 2.46 * tm4 + 0.88);
+    const double lsu = work * (2.3 * c.TN + 1.45 * tm4 + 0.3);
+    const double compute = cbrt(fma * fma * fma + issue * issue * issue + lsu * lsu * lsu);
+    const int cols = c.vec ? c.pitch / 4 : c.PW;
+    const double in_copies = ch * c.NI * c.PH * ((cols + c.lpr - 1) / c.lpr) * c.lpr / 32.0;
+    const double w_copies = ch * taps * BM / (c.wvec ? 128.0 : 32.0);
+    const double load = 21.2 * in_copies + 8.1 * w_copies;
+    const double cta = compute + load + (c.split > 1 ? 33.7 : 6.2) * outputs;
+    const double path = 1320.0 + 113.0 * c.per_split + ch * taps * (0.5 * products * (c.TM == 1 ? 2.0 : 1.0) + 36.2) + 13.3 * load / warps +
+                        (c.split > 1 ? 8750.0 : 0.0);
+    int occ = (int)(227 * 1024 / (c.smem + 1024));
+    const int by_regs = (products > 64 ? 256 : 512) / threads;             // 255 or 128 registers per thread
+    if (occ > by_regs) occ = by_regs;
+    if (occ < 1) occ = 1;
+    const double slots = (double)sm_count * occ;
+    const double full = floor(c.ctas / slots), rest = c.ctas - full * slots;
+    auto wave = [&](double share) { return (share * cta > path ? share * cta : path) + 0.3 * path; };
+    return full * wave(occ) + (rest > 0 ? wave(ceil(rest / sm_count)) : 0.0);
+}
+
+}  // namespace
+
+bool conv_config(const Shape& s, int sm_count, ConvCfg& best) {
+    bool found = false;
+    double best_cost = 0.0;
+    int tm_max = 1;
+    while (tm_max < 16 && tm_max < s.Kg) tm_max *= 2;
+    const double pixels = (double)s.N * s.H_out * s.W_out / 32.0;
+    for (int tm = tm_max; tm >= 1 && 8 * tm >= tm_max; tm /= 2) {
+        if (tm == 1 && s.Kg > 1) break;
+        for (int tn = tm >= 8 ? 8 : 4; tn >= 1; tn /= 2)
+            for (int wm = 1; wm <= 8; ++wm) {
+                if (wm > 1 && (wm - 1) * tm >= s.Kg) break;
+                // (no choice can beat its own FP32 arithmetic: whole filter blocks, every pixel, all SMs busy)
+                const int kblocks = (s.Kg + wm * tm - 1) / (wm * tm);
+                const double least = 0.361 * tm * wm * kblocks * pixels * s.groups * s.Cg * s.KH * s.KW / sm_count;
+                if (found && least >= best_cost) continue;
+                for (int wn = 1; wn * wm <= 8; wn *= 2) {
+                    if (wm * wn < 2) continue;
+                    const int BN = 32 * tn * wn;
+                    if (wn > 1 && BN / 2 >= s.N * s.H_out * s.W_out) break;      // half of the tile would already hold everything
+                    ConvCfg c;
+                    c.TM = tm; c.TN = tn; c.WM = wm; c.WN = wn;
+                    int last_tw = 0;
+                    const int tx0 = (s.W_out + BN - 1) / BN;
+                    for (int tx = tx0; tx < tx0 + 4; ++tx) {
+                        const int tw = (s.W_out + tx - 1) / tx;
+                        if (tw > BN || tw == last_tw) continue;
+                        last_tw = tw;
+                        double here = 1e30;
+                        for (int split = 1; split <= 8 && split <= s.Cg; split *= 2) {
+                            c.split = split;
+                            if (!conv_geometry(s, c, tw)) continue;
+                            const double cost = conv_cost(s, c, sm_count);
+                            if (cost < here) here = cost;
+                            if (!found || cost < best_cost) {
+                                found = true;
+                                best_cost = cost;
+                                best = c;
+                            }
+                            if (cost > 1.3 * here || (long long)c.ctas >= 2LL * sm_count) break;   // no gain, or the grid fills the chip
+                        }
+                        if (found && here > 1.3 * best_cost) break;       // other column counts of this tile size are no better
+                    }
+                }
+            }
+    }
+    if (!found) return false;
+    best.div_ph = make_fastdiv((uint32_t)best.PH);
+    best.div_cc = make_fastdiv((uint32_t)best.CC);
+    best.div_sw = make_fastdiv((uint32_t)s.stride_w);
+    best.div_bm = make_fastdiv((uint32_t)(best.wvec ? best.TM * best.WM / 4 : best.TM * best.WM));
+    best.div_tile = make_fastdiv((uint32_t)(best.TH * best.TW));
+    best.div_tw = make_fastdiv((uint32_t)best.TW);
+    return true;
+}
+
+template <int TM, int TN>
+static cudaError_t launch_conv(const Shape& s, const ConvCfg& c, const float* x, const uint32_t* pk, float* y, Status* status,
+                               uint32_t tag, cudaStream_t st) {
+    auto kernel = direct_conv_kernel<TM, TN>;
+    static bool attr_set[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64 || !attr_set[dev]) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) attr_set[dev] = true;
+    }
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(c.ctas);
+    lc.blockDim = dim3((unsigned)(32 * c.WM * c.WN));
+    lc.dynamicSmemBytes = c.smem;
+    lc.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)c.split;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    lc.attrs = attr;
+    lc.numAttrs = c.split > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&lc, kernel, s, c, x, pk, y, status, tag);
+}
+
+cudaError_t conv_forward(const Shape& s, const ConvCfg& c, const float* x, const void* packed, float* y, Status* status, uint32_t tag,
+                         cudaStream_t st) {
+    const uint32_t* pk = reinterpret_cast<const uint32_t*>(packed);
+#define GCONV_CONV_CASE(M, T) \
+    if (c.TM == M && c.TN == T) return launch_conv<M, T>(s, c, x, pk, y, status, tag, st);
+#define GCONV_CONV_ROW(M) GCONV_CONV_CASE(M, 1) GCONV_CONV_CASE(M, 2) GCONV_CONV_CASE(M, 4)
+    GCONV_CONV_ROW(1) GCONV_CONV_ROW(2) GCONV_CONV_ROW(4) GCONV_CONV_ROW(8) GCONV_CONV_ROW(16)
+    GCONV_CONV_CASE(8, 8) GCONV_CONV_CASE(16, 8)
+#undef GCONV_CONV_ROW
+#undef GCONV_CONV_CASE
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace gconv

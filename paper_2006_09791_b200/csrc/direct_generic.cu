@@ -1,7 +1,8 @@
-// Variant DIRECT_GENERIC: FP32 FFMA direct grouped convolution, one thread per output element.
-// Handles every shape the descriptor accepts (any kernel size; stride, padding and dilation per axis); it is
-// the safety net of the selector, not a fast path.  Grouped convolution of Section II of the paper,
-// summed in the (c, r, s) order of the convolution stage of Algorithm 1.
+// Variant DIRECT_GENERIC: FP32 grouped convolution of any shape the descriptor accepts (any kernel size; stride, padding and
+// dilation per axis).  Nearly every shape runs on the staged kernel of direct_conv.cu; the kernel here, one thread per output
+// element straight from global memory, takes what no tile of that one holds (single-channel patches over 200 KB: filters
+// or dilations of hundreds of pixels).  Grouped convolution of Section II of the paper, summed in the (c, r, s) order of
+// the convolution stage of Algorithm 1.  Packed weights: [g][c][r][s][Kg], as for DIRECT_TILED.
 #include "gconv_internal.h"
 
 namespace gconv {
@@ -10,23 +11,12 @@ size_t generic_packed_bytes(const Shape& s) {
     return kHeaderBytes + sizeof(float) * (size_t)s.C_out * s.Cg * s.KH * s.KW;
 }
 
-__global__ void generic_pack_kernel(const float* __restrict__ w, uint32_t* __restrict__ packed, size_t n, uint32_t tag) {
-    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) {
-        packed[0] = tag;
-        for (int j = 1; j < kHeaderBytes / 4; ++j) packed[j] = 0;
-    }
-    float* dst = reinterpret_cast<float*>(packed + kHeaderBytes / 4);
-    for (; i < n; i += (size_t)gridDim.x * blockDim.x) dst[i] = w[i];
+cudaError_t generic_pack(const Shape& s, const float* w, void* packed, cudaStream_t st) {
+    return group_pack(s, w, packed, generic_tag(s), st);
 }
 
-cudaError_t generic_pack(const Shape& s, const float* w, void* packed, cudaStream_t st) {
-    size_t n = (size_t)s.C_out * s.Cg * s.KH * s.KW;
-    int blocks = (int)((n + 255) / 256 < 1184 ? (n + 255) / 256 : 1184);
-    generic_pack_kernel<<<blocks, 256, 0, st>>>(w, reinterpret_cast<uint32_t*>(packed), n,
-                                                pack_tag(s, GCONV_VARIANT_DIRECT_GENERIC));
-    return cudaGetLastError();
-}
+// The tag names the layout as well as the shape (a blob packed as a plain OIHW copy by an earlier build is refused).
+uint32_t generic_tag(const Shape& s) { return pack_tag(s, GCONV_VARIANT_DIRECT_GENERIC | (2 << 8)); }
 
 __global__ void __launch_bounds__(256)
 generic_forward_kernel(Shape s, const float* __restrict__ x, const uint32_t* __restrict__ packed,
@@ -46,7 +36,7 @@ generic_forward_kernel(Shape s, const float* __restrict__ x, const uint32_t* __r
         const int n = (int)(t / s.C_out);
         const int g = ko / s.Kg;
         const float* xg = x + ((size_t)n * s.C_in + (size_t)g * s.Cg) * s.H * s.W;
-        const float* wk = w + (size_t)ko * s.Cg * s.KH * s.KW;
+        const float* wk = w + (size_t)g * s.Cg * s.KH * s.KW * s.Kg + (ko - g * s.Kg);
         float acc = 0.f;
         for (int c = 0; c < s.Cg; ++c) {
             for (int r = 0; r < s.KH; ++r) {
@@ -55,7 +45,7 @@ generic_forward_kernel(Shape s, const float* __restrict__ x, const uint32_t* __r
                 for (int ss = 0; ss < s.KW; ++ss) {
                     const int v = q * s.stride_w + ss * s.dilation_w - s.pad_w;
                     if (v < 0 || v >= s.W) continue;
-                    acc = fmaf(__ldg(xg + ((size_t)c * s.H + h) * s.W + v), __ldg(wk + (c * s.KH + r) * s.KW + ss), acc);
+                    acc = fmaf(__ldg(xg + ((size_t)c * s.H + h) * s.W + v), __ldg(wk + (size_t)((c * s.KH + r) * s.KW + ss) * s.Kg), acc);
                 }
             }
         }
@@ -63,14 +53,14 @@ generic_forward_kernel(Shape s, const float* __restrict__ x, const uint32_t* __r
     }
 }
 
-cudaError_t generic_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status,
-                            int sm_count, cudaStream_t st) {
+cudaError_t generic_forward(const Shape& s, const ConvCfg* conv, const float* x, const void* packed, float* y, Status* status,
+                            int sm_count, uint32_t tag, cudaStream_t st) {
+    if (conv != nullptr) return conv_forward(s, *conv, x, packed, y, status, tag, st);
     const size_t total = (size_t)s.N * s.C_out * s.H_out * s.W_out;
     size_t want = (total + 255) / 256;
     size_t cap = (size_t)sm_count * 8 * 4;
     int blocks = (int)(want < cap ? want : cap);
-    generic_forward_kernel<<<blocks, 256, 0, st>>>(s, x, reinterpret_cast<const uint32_t*>(packed), y, status,
-                                                   pack_tag(s, GCONV_VARIANT_DIRECT_GENERIC));
+    generic_forward_kernel<<<blocks, 256, 0, st>>>(s, x, reinterpret_cast<const uint32_t*>(packed), y, status, tag);
     return cudaGetLastError();
 }
 

@@ -100,10 +100,10 @@ extern "C" int gconv_forward_host_static(gconv_desc_t d, const float* x_host, co
                 e = igemm_forward(s, x_stage, w_packed, y_stage, status, sm_count, st, ws, opts);
                 break;
             case GCONV_VARIANT_DIRECT_TILED:
-                e = tiled_forward(s, x_stage, w_packed, y_stage, status, sm_count, st);
+                e = tiled_forward(s, d->conv_plan(), x_stage, w_packed, y_stage, status, sm_count, st);
                 break;
             default:
-                e = generic_forward(s, x_stage, w_packed, y_stage, status, sm_count, st);
+                e = generic_forward(s, d->conv_plan(), x_stage, w_packed, y_stage, status, sm_count, generic_tag(s), st);
                 break;
         }
     }

@@ -38,6 +38,13 @@ int select_variant(const Shape& s) {
     return GCONV_VARIANT_DIRECT_GENERIC;
 }
 
+// What the descriptor's variant keeps from call to call: the staged FP32 kernel's tile (a search over a few hundred choices).
+void make_plan(gconv_desc* d) {
+    d->has_conv = false;
+    if (d->variant == GCONV_VARIANT_DIRECT_GENERIC || (d->variant == GCONV_VARIANT_DIRECT_TILED && tiled_takes_conv(d->s)))
+        d->has_conv = conv_config(d->s, 148, d->conv);
+}
+
 int fail_cuda(gconv_desc* d, cudaError_t e) {
     d->last_cuda_error = (int)e;
     (void)cudaGetLastError();  // clear the sticky-free error state
@@ -118,6 +125,7 @@ int gconv_desc_create_2d(gconv_desc_t* out, int N, int C_in, int H, int W, int C
     d->pack_epoch_seen = 0;
     d->wait_us = 0;
     d->dbg_skip = -1;
+    make_plan(d);
     *out = d;
     return GCONV_OK;
 }
@@ -172,12 +180,14 @@ int gconv_desc_set_variant(gconv_desc_t d, int variant) {
     if (variant == GCONV_VARIANT_AUTO) {
         d->variant = select_variant(d->s);
         d->forced = 0;
+        make_plan(d);
         return GCONV_OK;
     }
     if (variant < GCONV_VARIANT_DIRECT_GENERIC || variant > GCONV_VARIANT_IGEMM_TF32) return GCONV_ERR_INVALID_ARG;
     if (!variant_supported(d->s, variant)) return GCONV_ERR_UNSUPPORTED;
     d->variant = variant;
     d->forced = 1;
+    make_plan(d);
     return GCONV_OK;
 }
 
@@ -213,7 +223,7 @@ int gconv_forward(gconv_desc_t d, const float* x, const void* w_packed, float* y
     cudaError_t e;
     switch (d->variant) {
         case GCONV_VARIANT_DIRECT_TILED:
-            e = tiled_forward(d->s, x, w_packed, y, d->status_dev, d->sm_count, st);
+            e = tiled_forward(d->s, d->conv_plan(), x, w_packed, y, d->status_dev, d->sm_count, st);
             break;
         case GCONV_VARIANT_IGEMM_TF32: {
             const size_t need = igemm_scratch_bytes(d->s);
@@ -223,7 +233,7 @@ int gconv_forward(gconv_desc_t d, const float* x, const void* w_packed, float* y
         }
         case GCONV_VARIANT_DIRECT_GENERIC:
         default:
-            e = generic_forward(d->s, x, w_packed, y, d->status_dev, d->sm_count, st);
+            e = generic_forward(d->s, d->conv_plan(), x, w_packed, y, d->status_dev, d->sm_count, generic_tag(d->s), st);
             break;
     }
     return e == cudaSuccess ? GCONV_OK : fail_cuda(d, e);

@@ -14,6 +14,31 @@ struct Shape {
     int stride_w, pad_w, dilation_w;                                   // the column axis (S_w); equal to the row values on square problems
     __host__ __device__ bool square() const { return stride_w == stride && pad_w == pad && dilation_w == dilation; }
 };
+
+// Division by a run-time constant as multiply-high + shift; exact for numerators below 2^31.
+struct FastDiv {
+    uint32_t mul, shr, div;
+    __device__ __forceinline__ void divmod(uint32_t n, uint32_t& q, uint32_t& r) const {
+        const uint32_t qq = (div != 1) ? (__umulhi(n, mul) >> shr) : n;
+        r = n - qq * div;
+        q = qq;
+    }
+};
+FastDiv make_fastdiv(uint32_t d);
+
+// FP32 direct convolution of any filter shape (direct_conv.cu): tile, staging and launch geometry.
+struct ConvCfg {
+    int TM, TN, WM, WN;                    // filters and pixel sets (of 32) per thread, warps over filters and over pixels
+    int TH, TW, NI;                        // output tile of a CTA: images x rows x columns
+    int tiles_x, tiles_y, tiles_n, kblocks;
+    int PH, PW, phase, pitch, plane;       // staged patch of one channel: rows, columns, floats per column phase, per row, in all
+    int CC, chunks, per_split, split;      // channels per stage, stages, stages of one rank, CTAs (a cluster) sharing the channels
+    int stages, in_floats, w_floats;       // buffers, floats of a buffer's patch and weights
+    int vec, wvec, lpr;                    // 16-byte copies of the patch / of the weights, lanes per staged row
+    uint32_t ctas;
+    size_t smem;
+    FastDiv div_ph, div_cc, div_sw, div_bm, div_tile, div_tw;
+};
 }  // namespace gconv
 
 // The descriptor behind gconv_desc_t.
@@ -31,6 +56,9 @@ struct gconv_desc {
     unsigned long long pack_epoch_seen;   // value of the process-wide pack counter at this descriptor's last forward
     int wait_us;                 // time limit of one bounded wait inside a kernel, microseconds (0 = the default, one second)
     int dbg_skip;                // failure-path test hook: stage fill that CTA 0's producer leaves out (-1 = none)
+    gconv::ConvCfg conv;         // tile and launch geometry of the staged FP32 kernel, where the variant runs it (chosen once)
+    bool has_conv;
+    const gconv::ConvCfg* conv_plan() const { return has_conv ? &conv : nullptr; }
 };
 
 namespace gconv {
@@ -61,20 +89,14 @@ __device__ inline void record_status(Status* st, int code, int detail) {
 
 // ---- per-variant entry points (host side launchers) --------------------------------------------
 size_t generic_packed_bytes(const Shape& s);
+uint32_t generic_tag(const Shape& s);
 cudaError_t generic_pack(const Shape& s, const float* w, void* packed, cudaStream_t st);
-cudaError_t generic_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status,
-                            int sm_count, cudaStream_t st);
+cudaError_t generic_forward(const Shape& s, const ConvCfg* conv, const float* x, const void* packed, float* y, Status* status,
+                            int sm_count, uint32_t tag, cudaStream_t st);
 
-// Division by a run-time constant as multiply-high + shift; exact for numerators below 2^31.
-struct FastDiv {
-    uint32_t mul, shr, div;
-    __device__ __forceinline__ void divmod(uint32_t n, uint32_t& q, uint32_t& r) const {
-        const uint32_t qq = (div != 1) ? (__umulhi(n, mul) >> shr) : n;
-        r = n - qq * div;
-        q = qq;
-    }
-};
-FastDiv make_fastdiv(uint32_t d);
+bool conv_config(const Shape& s, int sm_count, ConvCfg& c);   // false: no tile fits (huge filters or dilations)
+cudaError_t conv_forward(const Shape& s, const ConvCfg& c, const float* x, const void* packed, float* y, Status* status, uint32_t tag,
+                         cudaStream_t st);
 
 // DIRECT_TILED, narrow groups (Kg in {1,2,4,8}): one thread per (image, group, row strip, 4-pixel chunk).
 struct RowsCfg {
@@ -107,19 +129,13 @@ DwCfg dw_config(const Shape& s, int sm_count);
 cudaError_t dw_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, int sm_count,
                        cudaStream_t st);
 
-// DIRECT_TILED: launch geometry chosen on the host from the shape.
-struct TiledCfg {
-    int TXT, TY, KQ, GB, KT, CCH;          // x threads, rows, filter slabs, groups per CTA, filters per thread, channel chunk
-    int IH, IW, IWP, LPR;                  // staged patch rows, columns, padded row pitch, lanes per staged row
-    int tiles_x, tiles_y, kblocks, gblocks;
-    int threads;
-    size_t smem;
-};
+// DIRECT_TILED
 bool tiled_supported(const Shape& s);
+bool tiled_takes_conv(const Shape& s);   // neither depthwise nor narrow groups: the staged kernel
 size_t tiled_packed_bytes(const Shape& s);
-TiledCfg tiled_config(const Shape& s, int sm_count);
+cudaError_t group_pack(const Shape& s, const float* w, void* packed, uint32_t tag, cudaStream_t st);
 cudaError_t tiled_pack(const Shape& s, const float* w, void* packed, cudaStream_t st);
-cudaError_t tiled_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, int sm_count,
+cudaError_t tiled_forward(const Shape& s, const ConvCfg* conv, const float* x, const void* packed, float* y, Status* status, int sm_count,
                           cudaStream_t st);
 
 // IGEMM_TF32: tile geometry of the tcgen05 implicit-GEMM kernel.
