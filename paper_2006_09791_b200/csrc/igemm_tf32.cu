@@ -1790,21 +1790,22 @@ static IgemmCfg igemm_config_c2(const Shape& s_any, int sm_count, int C2) {
     // Row boxes: for widths that do not divide 32 a tile can instead be RT whole rows of SR 32-pixel segments each
     // (the second segment of a row shifted left to end at column W).  Every vertical tap is then a whole number of
     // segments away, so one staged block (tile + a row above and below, one 5-D TMA box) serves all three taps, and
-    // each segment contains the horizontal neighbours of the columns it stores (no exchange between warps).  Used
-    // when it wastes at most a quarter more lanes than the flat tiling.
+    // each segment contains the horizontal neighbours of the columns it stores (no exchange between warps).  Taken
+    // however many lanes of a segment stay empty: the flat tiling copies every tap by itself, exchanges edge lanes between warps and
+    // runs the generic instantiation.  Flat -> row boxes: 64 -> 64 @40x40 N = 64 42.9 -> 20.0 us (g = 1), 38.2 -> 14.0 us (g = 8);
+    // 256 -> 256 @12x12 N = 64, 3/8 of the lanes in use, 74.0 -> 39.5 us (g = 1), 24.1 -> 10.9 us (g = 8); 128 -> 128 @9x8 N = 8, a
+    // quarter in use, g = 8 7.7 -> 3.0 us; pointwise 256 -> 256 @40x40 stride 2 81.3 -> 58.8 us.  Only stride 2 on 4- and 8-wide planes
+    // (no stride-2 row tiles there) is faster flat: 128 -> 256 @9x8 N = 64 g = 8 13.1 against 21.9 us.
     c.rowbox = 0;
     c.SR = 0;
-    if (!c.seg_mode && s.W <= 62) {
+    if (!c.seg_mode && s.W <= 62 && !(s.stride == 2 && s.W <= 8)) {
         const int sr = s.W <= 32 ? 1 : 2;
-        const double util_box = (double)s.W / (32.0 * sr), util_flat = (double)((128 / s.W) * s.W) / 128.0;
-        if (util_box >= 0.8 * util_flat) {
-            c.rowbox = 1;
-            c.SR = sr;
-            c.R = 4 / sr;                                // rows per tile
-            c.RB = (s.H + c.R - 1) / c.R;
-            c.MT = s.N * c.RB;
-            c.need_xchg = 0;
-        }
+        c.rowbox = 1;
+        c.SR = sr;
+        c.R = 4 / sr;                                // rows per tile
+        c.RB = (s.H + c.R - 1) / c.R;
+        c.MT = s.N * c.RB;
+        c.need_xchg = 0;
     }
     // Stride 2 on widths 17..62: a tile is four output rows of one 32-column segment.  Its stage holds the nine input
     // rows 2p-1 .. 2p+7 of that segment; the rows a vertical tap needs are every other one, so tap r is the view that
