@@ -74,6 +74,7 @@ struct __align__(8) SharedCtl {
     // epilogue group) into a second MMA that accumulates the pointwise output of the pixel tile over all groups (d2)
     unsigned long long a2_full[2], a2_free[2], d2_full[2], d2_free[2], w2_full;
     unsigned long long raw_full[4], raw_empty[4];   // gather producer: ring of raw input buffers (bulk copies in, copy warps out)
+    unsigned long long red_bar[2];   // split channels: every CTA of the cluster has left its partial sums (of the pair's tile e) in shared memory
     uint32_t tmem_base;
     int abort_flag;      // set by the first role whose wait ran out; every other role then leaves at its next wait
     uint32_t wait_us;    // time limit of one wait, in microseconds (read as abort_flag[1] by the wait helpers)
@@ -122,6 +123,33 @@ __device__ __forceinline__ uint64_t global_ns() {
     return t;
 }
 
+// Cluster helpers (split channels): the shared-memory address of another CTA, an arrival on its barrier that publishes this
+// warp's writes to it, a load from its shared memory, and the wait that makes the other CTAs' writes visible.
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+}
+__device__ __forceinline__ float ld_remote(uint32_t cluster_addr) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr));
+    return v;
+}
+__device__ __forceinline__ uint32_t mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok;
+}
+
 // Bounded wait: gives up after the CTA's time limit (one second by default).  Returns false if the wait ran out or
 // another role already gave up; the first role to run out records GCONV_ERR_TIMEOUT with `where` as the detail.
 //
@@ -129,12 +157,14 @@ __device__ __forceinline__ uint64_t global_ns() {
 // walking the other warp's stages, see there): a parity wait is only meaningful one phase at a time, so such a waiter must
 // never be away from the barrier for as long as two phase flips take (a refill is a microsecond or more away).  The clock
 // (a read of the global timer is slow) is therefore looked at only once every 128 polls.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, Status* status,
                                           int where) {
-    if (mbar_try_wait(bar, parity)) return true;
+    auto poll = [&]() { return CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity); };
+    if (poll()) return true;
     uint64_t limit_ns = 0, t0 = 0;
     for (uint32_t it = 0;; ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (poll()) return true;
         if (*abort_flag) return false;
         if ((it & 127u) == 127u) {
             if (it == 127u) {
@@ -305,9 +335,9 @@ __device__ __forceinline__ void gath_part(const Shape& s, const IgemmCfg& c, uin
 // instruction stream matters: the 8x8 layers of the WRN stack run 20 % faster on their family than on family 0.
 struct Family {
     int rowbox, seg_mode, nr, need_xchg, b_res, egroups, s2h, lbo_segs, stride, CK, chunks, Kt, Np, NT, nacc, issuers, padded,
-        nt_fast, wseg, nseg, SR, fast4, tapb, fuse, ball, soft, pw, pair;   // (pair: 0 where a row leaves it out)
+        nt_fast, wseg, nseg, SR, fast4, tapb, fuse, ball, soft, pw, pair, spl;   // (pair, spl: 0 where a row leaves them out)
 };
-constexpr int kFamilies = 31;
+constexpr int kFamilies = 39;
 __host__ __device__ constexpr Family family(int f) {
     //                 rowbox seg nr xchg bres egr s2h lbo str CK  ch  Kt  Np  NT acc iss pad ntf wseg nseg SR f4 tapb fuse ball soft pw
     return f == 1 ? Family{0,   1,  1,  0,   1,  1,  0,  1,  1, 32,  1, 32,  96,  1,  2,  2, -1,  0,  0,   4,  0, -1,  0,  0,  0,  0,  0}     // 16x16 / 8x8 planes, narrow groups
@@ -340,11 +370,20 @@ __host__ __device__ constexpr Family family(int f) {
          : f == 28 ? Family{0,   0,  3,  0,  -1,  2,  0,  1,  1, 16, -1, 64, 192, -1,  2,  2,  0, -1,  4,  12,  0, -1,  0,  0,  0,  1,  0,  0}     // gather producer, stride 1, wide groups (one CTA per SM, 29 warps)
          : f == 29 ? Family{0,   0,  3,  0,   0,  2,  0,  1,  2,  8, -1, 64, 192, -1,  1,  1,  0, -1,  8,  24,  0, -1,  0,  0,  0,  2,  0,  1}     // gather producer, stride 2, wide groups, 8-channel stages, streamed weights shared by a pair of pixel tiles
          : f == 30 ? Family{0,   0,  3,  0,   0,  2,  0,  1,  1, 16, -1, 64, 192, -1,  1,  1,  0, -1,  4,  12,  0, -1,  0,  0,  0,  1,  0,  1}     // gather producer, stride 1, wide groups, streamed weights shared by a pair of pixel tiles
+         // channels split over a cluster (few tiles, many channels), streamed weights
+         : f == 31 ? Family{0,   0,  3,  0,   0,  2,  0,  1,  1, 16, -1, 64, 192, -1,  1,  1,  0, -1,  4,  12,  0, -1,  0,  0,  0,  1,  0,  1,  1}     // gather producer, stride 1, pair tiles
+         : f == 32 ? Family{0,   0,  3,  0,   0,  2,  0,  1,  2,  8, -1, 64, 192, -1,  1,  1,  0, -1,  8,  24,  0, -1,  0,  0,  0,  2,  0,  1,  1}     // gather producer, stride 2, pair tiles
+         : f == 33 ? Family{1,   0,  3,  0,   0,  2,  0,  1,  1, -1, -1, -1,  -1, -1,  2,  2, -1, -1, -1,  -1, -1,  1,  0,  0,  0,  0,  0,  0,  1}     // row boxes
+         : f == 34 ? Family{1,   0,  3,  0,   0,  2,  1,  2,  2, -1, -1, -1,  -1, -1,  2,  2, -1, -1,  1,   9, -1,  1,  0,  0,  0,  0,  0,  0,  1}     // stride-2 row tiles
+         : f == 35 ? Family{0,   1,  1,  0,   0,  2,  0,  1, -1, -1, -1, -1,  -1, -1,  2,  2, -1, -1,  0,   4,  0, -1,  0,  0,  0,  0,  0,  0,  1}     // segment tilings, a stage per tap
+         : f == 36 ? Family{0,   1,  3,  0,   0,  2,  0,  1,  1, -1, -1, -1,  -1, -1,  2,  2, -1, -1,  1,   6,  0,  2,  0,  0,  0,  0,  0,  0,  1}     // 32-wide planes with halo stages
+         : f == 37 ? Family{0,   0,  3,  0,   0,  2,  0,  1,  1, 16, -1, 64, 192, -1,  2,  2,  0, -1,  4,  12,  0, -1,  0,  0,  0,  1,  0,  0,  1}     // gather producer, stride 1
+         : f == 38 ? Family{0,   0,  3,  0,   0,  2,  0,  1,  2, 16, -1, 64, 192, -1,  2,  2,  0, -1,  8,  24,  0, -1,  0,  0,  0,  2,  0,  0,  1}     // gather producer, stride 2
                   : Family{-1, -1, -1, -1,  -1, -1, -1, -1, -1, -1, -1, -1,  -1, -1, -1, -1, -1, -1, -1,  -1, -1, -1, -1, -1, -1, -1, -1, -1};
 }
 #define GCONV_FAMILY_FIELDS(X) \
     X(rowbox) X(seg_mode) X(nr) X(need_xchg) X(b_res) X(egroups) X(s2h) X(lbo_segs) X(CK) X(chunks) X(Kt) X(Np) X(NT) X(nacc) X(issuers) \
-    X(padded) X(nt_fast) X(wseg) X(nseg) X(SR) X(fast4) X(tapb) X(fuse) X(ball) X(soft) X(pw) X(pair)
+    X(padded) X(nt_fast) X(wseg) X(nseg) X(SR) X(fast4) X(tapb) X(fuse) X(ball) X(soft) X(pw) X(pair) X(spl)
 
 static bool family_matches(int f, const Shape& s, const IgemmCfg& c) {
     const Family fam = family(f);
@@ -406,7 +445,8 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
             n = (w8 >= (int)offsetof(SharedCtl, b_free) && w8 < (int)offsetof(SharedCtl, a2_full)) ? (uint32_t)c.issuers : n;
             n = (w8 >= (int)offsetof(SharedCtl, a2_full) && w8 < (int)offsetof(SharedCtl, a2_free)) ? (uint32_t)kEpiWarps : n;
             n = (w8 >= (int)offsetof(SharedCtl, d2_free) && w8 < (int)offsetof(SharedCtl, w2_full)) ? (uint32_t)kEpiWarps : n;
-            n = (w8 >= (int)offsetof(SharedCtl, raw_empty) && w8 < (int)offsetof(SharedCtl, tmem_base)) ? n_copy : n;
+            n = (w8 >= (int)offsetof(SharedCtl, raw_empty) && w8 < (int)offsetof(SharedCtl, red_bar)) ? n_copy : n;
+            n = w8 >= (int)offsetof(SharedCtl, red_bar) ? (uint32_t)(kEpiWarps * (c.spl ? c.split : 1)) : n;
             if (t < kBarriers) mbar_init(smem_u32(&ctl) + (uint32_t)w8, n);
         }
         if (lane == 0) {
@@ -431,11 +471,22 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
         tc_fence_after();
     }
     const uint32_t tmem_base = warp == 0 ? 0u : ctl.tmem_base;   // (the producer never touches tensor memory)
+    // Split channels: the CTAs of a cluster work on one tile, rank r on channel chunks r * csplit ...; the first phase of the
+    // hardware cluster barrier says that every CTA has started and initialised its barriers.
+    // (the barrier counts warps: every arrival and wait is made by a converged warp)
+    const int rank = c.spl ? (int)(blockIdx.x % (uint32_t)c.split) : 0, bid = c.spl ? (int)(blockIdx.x / (uint32_t)c.split) : (int)blockIdx.x;
+    const int chunk0 = c.spl ? rank * c.csplit : 0;
+    const int chunks = c.spl ? min(c.csplit, c.chunks - chunk0) : c.chunks;
+    bool cluster_seen = false;
+    if (c.spl) {
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    }
     const bool tag_ok = (tag_seen == tag);   // uniform across the CTA
     // Tiles of this CTA: every gridDim.x-th tile, or -- with resident weights and several (group, filter tile) pairs --
     // the CTAs split into one set per pair, each set striding over that pair's pixel tiles: no CTA ever switches
     // weights, and the CTAs of a set still read neighbouring pixels at the same time.
-    int tile_first = (int)blockIdx.x, tile_end = c.num_tiles, tile_step = (int)gridDim.x;
+    int tile_first = bid, tile_end = c.num_tiles, tile_step = c.spl ? c.num_tiles : (int)gridDim.x;
     if (c.fuse) tile_first = (int)blockIdx.x * c.n_gn;    // tile = pixel tile * n_gn + group; see tile_next
     // next tile of this CTA: every gridDim.x-th tile, or (fused block) the next group of the pixel tile and, after
     // its last group, the first group of the pixel tile gridDim.x further on
@@ -456,7 +507,8 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
     // segments of one vertical tap (nr = 1, stages run chunk-major, tap-minor), or the tile plus its
     // row halo (nr = 3: the three taps are views of the same stage, shifted by whole segments).
     const int vt = c.pw ? 1 : 3;                 // vertical taps (a pointwise layer has one tap, no neighbours)
-    const int kstages = (vt / c.nr) * c.chunks;
+    const int kstages = (vt / c.nr) * chunks;
+    const int ks0 = (vt / c.nr) * chunk0;        // first stage of this CTA in the packed weights
     const uint32_t seg_bytes = (uint32_t)c.CK * 128u;
     const uint32_t a_bytes = (uint32_t)c.nseg * seg_bytes;
     const uint32_t a_all = c.pair ? 2u * a_bytes : a_bytes;   // pair tiles: the second tile's input sits behind the first's
@@ -571,7 +623,7 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
                     if (ruse > 0 && !mbar_wait_warp(smem_u32(&ctl.raw_empty[rs]), (ruse - 1) & 1u, abort_flag, status, 150 + (int)rs)) { ok = false; break; }
                     const uint32_t rbar = smem_u32(&ctl.raw_full[rs]);
                     const uint32_t rdst = smem_base + c.raw_off + rs * c.raw_bytes;
-                    const int chan = g * c.Cg + ks * c.CK;
+                    const int chan = g * c.Cg + (chunk0 + ks) * c.CK;
                     if (dep_pending) {
                         asm volatile("griddepcontrol.wait;" ::: "memory");   // the input may be the previous kernel's output
                         dep_pending = false;
@@ -608,7 +660,7 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
                         const uint32_t full = smem_u32(&ctl.full[stage]);
                         if (lane == 0) {
                             mbar_arrive_expect_tx(full, nb);
-                            bulk_load_1d(stage_base + (uint32_t)stage * c.stage_bytes + a_all, wtile + (size_t)ks * nb, nb, full);
+                            bulk_load_1d(stage_base + (uint32_t)stage * c.stage_bytes + a_all, wtile + (size_t)(ks0 + ks) * nb, nb, full);
                         }
                     }
                     if (++stage == c.stages) { stage = 0; ph ^= 1; }
@@ -654,7 +706,7 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
                 const uint32_t full = smem_u32(&ctl.full[stage]);
                 const uint32_t a_dst = stage_base + (uint32_t)stage * c.stage_bytes;
                 const uint32_t nb = c.b_res ? 0u : (uint32_t)c.nr * blk_bytes;
-                const int chan = g * c.Cg + ch * c.CK;
+                const int chan = g * c.Cg + (chunk0 + ch) * c.CK;
                 // Failure-path test hook (gconv_desc_set_debug): CTA 0 leaves out one stage fill entirely -- no copy is
                 // issued and the barrier is not armed -- so the consumer's bounded wait on that stage runs out.
                 const bool skip_fill = !pf && (int)it == c.dbg_skip && blockIdx.x == 0;
@@ -682,7 +734,7 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
                         else if (c.fast4 == 2) tma_load_4d(a_dst, &xmap4, 0, chan, lo >> 5, tile_n, full);   // segments outside the plane read as zeros
                         else tma_load_4d(a_dst, &xmap4, lo, chan, 0, tile_n, full);
                     }
-                    if (nb) bulk_load_1d(a_dst + a_all, wtile + (size_t)ks * nb, nb, full);
+                    if (nb) bulk_load_1d(a_dst + a_all, wtile + (size_t)(ks0 + ks) * nb, nb, full);
                 }
                 if (!box && !skip_fill) {
                     if (!have_lane_coords) {
@@ -992,6 +1044,8 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
             const uint32_t blk16 = blk_bytes >> 4;
             const uint32_t bk16 = b_kstep >> 4;
             const uint32_t b_in_stage16 = a_all >> 4;
+            // (in a cluster a shared-memory address carries the CTA's rank from bit 24 on: a descriptor holds the offset in the CTA)
+            const uint32_t stage_window = c.spl ? stage_base & 0xFFFFFFu : stage_base;
             const uint32_t a_pair16 = a_bytes >> 4;   // pair tiles: the second tile's input inside the stage
             uint32_t tcount = 0, switches = 0;
             int stage = 0;
@@ -1046,7 +1100,7 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
                 uint32_t acc = 0;
                 for (int ks = 0; ks < kstages; ++ks) {
                     // (the descriptors of the stage are worked out before the wait: what follows the arrival of the data is the MMAs)
-                    const uint32_t a16 = (stage_base + (uint32_t)stage * c.stage_bytes) >> 4;
+                    const uint32_t a16 = (stage_window + (uint32_t)stage * c.stage_bytes) >> 4;
                     // weights of this stage: (chunk, tap) blocks of the resident bank, or the blocks staged behind A
                     const uint32_t b16 = c.b_res ? (bres_addr >> 4) + (uint32_t)(c.nr == 3 ? ks * 3 : ks) * blk16 : a16 + b_in_stage16;
                     uint32_t alo = a_lo0 + a16, blo = b_lo0 + b16;
@@ -1102,6 +1156,44 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
         bool pend = false, pend_valid = false;
         uint32_t pend_p = 0;
         float* pend_y2 = nullptr;
+        // Split channels, second half of the epilogue: the partial sums of the tile are in the shared memory of every CTA of the
+        // cluster ([filter][128 pixels], over the input stages: this CTA's MMAs are done with them); this CTA adds up its
+        // filters' slices, rank by rank, and stores them.
+        auto reduce_ranks = [&](const uint32_t part, const uint32_t e, float* y_tile, const bool v) -> bool {
+            __syncwarp();
+            if (!cluster_seen) {
+                asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // every CTA's barriers are initialised
+                cluster_seen = true;
+            }
+            const uint32_t bar = smem_u32(&ctl.red_bar[e]);
+            if (lane < c.split) mbar_arrive_remote(map_rank(bar, (uint32_t)lane));
+            if (!__all_sync(0xffffffffu, mbar_wait<true>(bar, 0, abort_flag, status, 450 + (int)e) ? 1 : 0)) return false;
+            // this CTA stores `per` filters, the two warps of a quarter alternate ones; kGroup filters' loads are in flight at a
+            // time (one filter at a time cost a remote round trip each, 0.27 us; all at once spilled registers)
+            constexpr int kGroup = 4;
+            const int per = (Kt + c.split - 1) / c.split;
+            const int mine = min(per, Kt - rank * per);
+            uint32_t at = part + (uint32_t)((rank * per + half) * 128 + l) * 4u;
+            float* dst = y_tile + (size_t)(rank * per + half) * OHW;
+            for (int k = half; k < mine; k += 2 * kGroup, at += 1024u * kGroup) {
+                float sum[kGroup] = {};
+#pragma unroll
+                for (int r = 0; r < 8; ++r) {
+                    if (r < c.split) {                             // in rank order
+                        const uint32_t from = map_rank(at, (uint32_t)r);
+#pragma unroll
+                        for (int j = 0; j < kGroup; ++j)
+                            if (k + 2 * j < mine) sum[j] += ld_remote(from + (uint32_t)j * 1024u);
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < kGroup; ++j) {
+                    if (v && k + 2 * j < mine) *dst = sum[j];
+                    dst += 2 * OHW;
+                }
+            }
+            return true;
+        };
         const int c2h = ((c.C2 / 2) + 7) & ~7;
         const int c2beg = half == 0 ? 0 : c2h, c2end = half == 0 ? c2h : c.C2;
         auto epilogue2 = [&](uint32_t db, uint32_t parity, float* y2, bool v) -> bool {
@@ -1257,6 +1349,14 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&ctl.tmem_empty[buf]));
+                if (c.spl) {
+                    const uint32_t part_off = stage_base - smem_base + egroup * (uint32_t)Kt * 512u;
+                    float* part = reinterpret_cast<float*>(smem + part_off) + kbeg * 128 + l;
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) part[j * 128] = v[j];
+                    if (!reduce_ranks(smem_base + part_off, egroup, yk - (size_t)kbeg * OHW, valid)) break;
+                    continue;
+                }
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
                     if (valid) *yk = v[j];
@@ -1296,11 +1396,18 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
                     if (c.fuse) {
                         const int k = k0 + j;
                         *reinterpret_cast<float*>(a2p + (size_t)k * 128u + (size_t)((((uint32_t)lane >> 3) ^ ((uint32_t)k & 3u)) << 5)) = v;
+                    } else if (c.spl) {
+                        reinterpret_cast<float*>(smem + (stage_base - smem_base))[(k0 + j) * 128 + l] = v;
                     } else {
                         if (valid) *yk = v;
                         yk += OHW;
                     }
                 }
+            }
+            if (c.spl) {
+                tc_fence_before();
+                if (!reduce_ranks(stage_base, 0u, yk - (size_t)kbeg * OHW, valid)) break;
+                continue;
             }
             if (c.fuse) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor core reads A2 through the async proxy
             tc_fence_before();
@@ -1339,6 +1446,14 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
         if (c.fuse && pend && !*abort_flag) epilogue2(pend_p & 1u, (pend_p >> 1) & 1u, pend_y2, pend_valid);
     }
 
+    if (c.spl) {
+        // nobody leaves while another CTA of the cluster may still read its partial sums or arrive on its barrier
+        // (single-lane roles come back to their warps first)
+        __syncwarp();
+        if (!cluster_seen) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1357,7 +1472,8 @@ igemm_tf32_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constan
                   const float* __restrict__ x) {
     if constexpr (F == 0) {
         IgemmCfg c = c_in;
-        c.pair = 0;     // pair tiles always run on their own instantiation (the host refuses anything else)
+        c.pair = 0;     // pair tiles and split channels always run on their own instantiations (the host refuses anything else)
+        c.spl = 0;
         igemm_tf32_body(xmap, xmap4, s_in, c, packed, y, status, tag, x);
     } else {
         constexpr Family fam = family(F);
@@ -1577,10 +1693,41 @@ size_t igemm_scratch_bytes(const Shape& s_any) {
 }
 
 
+// Split channels.  Wide groups on few pixels (small batches, small planes) give fewer tiles than SMs, and a tile is a serial
+// walk over all channels (512 channels on 7x7 planes, N = 13, g = 2: 32 CTAs of 64 stages, 25 us).  A cluster of `split` CTAs
+// then shares the tile, each takes a range of channel chunks, and the partial sums meet in distributed shared memory.
+// Taken while all clusters of the grid run at once: a cluster of one-CTA-per-SM blocks stays inside a GPC, and the 148 SMs hold
+// 74, 45, 33, 26, 22, 15 and 15 clusters of 2 ... 8 (the runtime's occupancy query); a second wave would cost what the split saves.
+// The exchange costs 3 us: measured (whole tiles -> split) 768 -> 768 @5x5 N = 4 54.9 -> 14.0 us, 512 -> 512 @7x7 N = 1 35.0 -> 10.6,
+// 512 -> 512 @7x7 N = 13 g = 2 25.2 -> 14.4, 384 -> 768 @10x10 stride 2 N = 4 19.8 -> 11.5 (no padded copy any more), 256 -> 256 @8x8 N = 1
+// 12.7 -> 6.7, 256 -> 256 @13x13 N = 13 g = 2 14.2 -> 12.9; but 64 -> 64 @14x14 N = 1 (48 channels spared) 5.9 -> 6.4 and, on row boxes,
+// whose stages are the quickest, 128 -> 128 @20x20 N = 2 (96 spared) 6.6 -> 7.4 against 256 -> 256 @28x28 N = 1 (192 spared)
+// 10.1 -> 9.3: the lines lie between.  16x16 and 8x8 planes: 128 -> 128 @16x16 (96 spared) N = 1, 4 tiles, 6.8 -> 6.2, N = 6, 24 tiles, 7.1 -> 7.5.
+// Stride-2 row tiles gain at 32 channels already (64 -> 128 @56x56 N = 1 8.5 -> 6.2).
+static int max_split(int tiles) { return tiles <= 15 ? 8 : (tiles <= 22 ? 6 : (tiles <= 26 ? 5 : (tiles <= 33 ? 4 : (tiles <= 45 ? 3 : (tiles <= 74 ? 2 : 1))))); }
+static void split_channels(IgemmCfg& c) {
+    c.spl = 0;
+    c.split = 1;
+    c.csplit = c.chunks;
+    int S = max_split(c.num_tiles);
+    if (S > c.chunks) S = c.chunks;
+    if (S < 2) return;
+    const int per = (c.chunks + S - 1) / S;
+    S = (c.chunks + per - 1) / per;                  // every rank has work
+    // channels a CTA has to be spared, above (0: tilings whose whole tiles run the generic instantiation)
+    const bool s1 = !c.sub_h && !c.sub_w;
+    const int least = c.soft == 1 ? 96 : (s1 && c.Kt == 64 && c.rowbox ? 160 : (s1 && c.Kt == 64 && c.nr == 1 ? (c.num_tiles <= 15 ? 96 : 160) : 0));
+    if ((c.chunks - per) * c.CK * (c.pair ? 2 : 1) < least) return;
+    if (S < 2 || (uint32_t)c.stages * c.stage_bytes < (uint32_t)(c.pair ? 2 : 1) * (uint32_t)c.Kt * 512u) return;
+    c.spl = 1;
+    c.split = S;
+    c.csplit = per;
+}
+
 // Gather producer (see the copy warps in the kernel): planes whose rows the tiled bulk copies cannot deliver as operand
 // rows (width not a multiple of 4, up to 32) with stride 1, and stride-2 layers on such planes.  Narrow (merged) groups in
 // the two-CTA launch shape.  Fills every field of the configuration; returns false when the shape is not taken.
-static bool gather_config(IgemmCfg& out, const Shape& st, int sm_count) {
+static bool gather_config(IgemmCfg& out, const Shape& st, int sm_count, bool singles) {
     IgemmCfg c = out;                    // committed only when the shape is taken
     const int mode = st.stride == 2 ? 2 : 1;
     if (st.KH != 3 || st.W % 4 == 0 || st.W_out > 32 || st.W_out < 1) return false;
@@ -1606,9 +1753,6 @@ static bool gather_config(IgemmCfg& out, const Shape& st, int sm_count) {
     c.padded = 0;
     c.Hv = st.H;
     c.Wv = st.W;
-    c.CK = c.Cg % 16 == 0 ? 16 : 8;
-    if (heavy && mode == 2) c.CK = 8;            // two pixel tiles of six blocks each share a stage with the streamed weights (pair tiles, below)
-    c.chunks = c.Cg / c.CK;
     const int Wo = st.W_out, Ho = st.H_out, HW = st.H * st.W;
     c.rps = 32 / Wo;
     c.SPI = (Ho + c.rps - 1) / c.rps;
@@ -1622,6 +1766,12 @@ static bool gather_config(IgemmCfg& out, const Shape& st, int sm_count) {
         c.MT = (st.N + c.IPT - 1) / c.IPT;
     }
     c.MTr = c.MT;
+    // few tiles: the channels are split over clusters (below); where that fills the chip with single tiles they stay single (unless
+    // two stages of them do not fit: tall planes of odd width with stride 2)
+    const bool few = singles && heavy && max_split(c.groups * c.NT * c.MTr) == 8;
+    c.CK = c.Cg % 16 == 0 ? 16 : 8;
+    if (heavy && mode == 2 && !few) c.CK = 8;    // two pixel tiles of six blocks each share a stage with the streamed weights (pair tiles, below)
+    c.chunks = c.Cg / c.CK;
     // raw parts: the input rows a tile needs, as flat pixels from a multiple of 4 on
     c.raw_bulk = HW % 4 != 0 ? 1 : 0;
     int px;
@@ -1677,7 +1827,8 @@ static bool gather_config(IgemmCfg& out, const Shape& st, int sm_count) {
     // every weight block feeds two MMAs (two accumulators side by side, one buffer), the eight copy warps build one tile each
     // per four, and the two epilogue groups drain the two accumulators at the same time.
     if (heavy && mode == 2) c.b_res = 0;         // (its stages leave no room for a resident bank)
-    if (heavy && !c.b_res && c.MT >= 2 && 2u * a_stage + (uint32_t)c.nr * (uint32_t)c.Np * (uint32_t)c.CK * 4u <= 100u * 1024u) {
+    if (few) c.b_res = 0;
+    if (heavy && !c.b_res && !few && c.MT >= 2 && 2u * a_stage + (uint32_t)c.nr * (uint32_t)c.Np * (uint32_t)c.CK * 4u <= 100u * 1024u) {
         c.pair = 1;
         c.MT = (c.MTr + 1) / 2;
         c.nacc = 1;
@@ -1700,12 +1851,13 @@ static bool gather_config(IgemmCfg& out, const Shape& st, int sm_count) {
         if (c.stages < max_ring && used + c.stage_bytes <= total) { ++c.stages; continue; }
         break;
     }
-    if (heavy && (c.stages < 2 || (mode == 2 && !c.pair))) return false;
+    if (heavy && !c.b_res) split_channels(c);
+    if (heavy && (c.stages < 2 || (mode == 2 && !c.pair && !c.spl))) return false;
     c.raw_off = bank + (uint32_t)c.stages * c.stage_bytes;
     c.xchg_off = c.raw_off + (uint32_t)c.raw_stages * c.raw_bytes;
     c.smem_bytes = (size_t)c.xchg_off + 1024;
     const int ctas = heavy ? sm_count : 2 * sm_count;
-    c.grid = c.num_tiles < ctas ? c.num_tiles : ctas;
+    c.grid = c.spl ? c.num_tiles * c.split : (c.num_tiles < ctas ? c.num_tiles : ctas);
     c.cps = 0;
     c.fuse = 0;
     c.ball = 0;
@@ -1728,6 +1880,9 @@ static bool gather_config(IgemmCfg& out, const Shape& st, int sm_count) {
 static IgemmCfg igemm_config_c2(const Shape& s_any, int sm_count, int C2) {
     const Shape s_true = as_3x3(s_any);
     IgemmCfg c;
+    c.spl = 0;
+    c.split = 1;
+    c.csplit = 0;
     c.wait_us = kDefaultWaitUs;
     c.dbg_skip = -1;
     // Pointwise: one vertical tap (a third of the stages and MMAs), one accumulator per filter (N = Kt), filter tiles of
@@ -1766,7 +1921,7 @@ static IgemmCfg igemm_config_c2(const Shape& s_any, int sm_count, int C2) {
     c.rps = c.IPT = c.boxpx = c.pieces = c.raw_whole = c.raw_bulk = c.raw_stages = 0;
     c.raw_off = c.raw_bytes = 0;
     c.div_boxpx = make_fastdiv(1);
-    if (!fuse && gather_config(c, s_true, sm_count)) return c;
+    if (!fuse && (gather_config(c, s_true, sm_count, true) || gather_config(c, s_true, sm_count, false))) return c;
     const int HW = s.H * s.W;
     c.seg_mode = (32 % s.W == 0) && (HW % 32 == 0);
     c.seg_fstep = 32;
@@ -1992,6 +2147,14 @@ static IgemmCfg igemm_config_c2(const Shape& s_any, int sm_count, int C2) {
         const int ctas = c.egroups == 1 ? 2 * sm_count : sm_count;
         c.grid = c.MT < ctas ? c.MT : ctas;                // a CTA takes whole pixel tiles (all groups of each)
     }
+    if (!fuse && !c.pw && !c.pair && !c.tapb && !c.need_xchg && s.dilation == 1 && c.egroups == 2 && c.b_res == 0) {
+        // (two accumulators, as the split instantiations have: a CTA has one tile)
+        split_channels(c);
+        if (c.spl) {
+            c.nacc = c.issuers = 2;
+            c.grid = c.num_tiles * c.split;
+        }
+    }
     {
         const int n_gn = c.groups * c.NT;
         if (!fuse && c.b_res == 1 && n_gn > 1 && c.grid >= n_gn) {
@@ -2196,10 +2359,13 @@ static cudaError_t igemm_launch(const Shape& s_true, int C2, const float* x_in, 
                                                 igemm_tf32_kernel<14>, igemm_tf32_kernel<15>, igemm_tf32_kernel<16>,
                                                 igemm_tf32_kernel<17>, igemm_tf32_kernel<18>, igemm_tf32_kernel<19>, igemm_tf32_kernel<20>,
                                                 igemm_tf32_kernel<21>, igemm_tf32_kernel<22>, igemm_tf32_kernel<23>,
-                                                igemm_tf32_kernel<24>, igemm_tf32_kernel<25>, igemm_tf32_kernel<26>, igemm_tf32_kernel<27>, igemm_tf32_kernel<28>, igemm_tf32_kernel<29>, igemm_tf32_kernel<30>};
+                                                igemm_tf32_kernel<24>, igemm_tf32_kernel<25>, igemm_tf32_kernel<26>, igemm_tf32_kernel<27>, igemm_tf32_kernel<28>, igemm_tf32_kernel<29>, igemm_tf32_kernel<30>,
+                                                igemm_tf32_kernel<31>, igemm_tf32_kernel<32>, igemm_tf32_kernel<33>, igemm_tf32_kernel<34>,
+                                                igemm_tf32_kernel<35>, igemm_tf32_kernel<36>, igemm_tf32_kernel<37>, igemm_tf32_kernel<38>};
     int fam = 0;
     for (int f = 1; f < kFamilies && fam == 0; ++f)
         if (family_matches(f, s, cfg)) fam = f;
+    if (cfg.spl && family(fam).spl != 1) return cudaErrorInvalidValue;     // nor split-channel code
     if (cfg.pair && family(fam).pair != 1) return cudaErrorInvalidValue;   // the generic instantiation has no pair-tile code
     if (cfg.soft && cfg.egroups == 2 && family(fam).soft != cfg.soft) return cudaErrorInvalidValue;   // 29 warps: only the wide-group gather instantiations take them
     static bool attr_set[64][kFamilies] = {};
@@ -2215,14 +2381,17 @@ static cudaError_t igemm_launch(const Shape& s_true, int C2, const float* x_in, 
     lc.blockDim = dim3((unsigned)c.threads);
     lc.dynamicSmemBytes = c.smem_bytes;
     lc.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = opts.pdl ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)c.split;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     lc.attrs = attr;
     // Without the attribute the kernel starts only after everything before it in the stream has completed and is
     // visible (griddepcontrol.* are then no-ops): used for the first forward after any weight packing, because the
     // kernel reads the packed weights before its dependency wait.
-    lc.numAttrs = opts.pdl ? 1 : 0;
+    lc.numAttrs = c.spl ? 2 : (opts.pdl ? 1 : 0);
     return cudaLaunchKernelEx(&lc, kernels[fam], xmap, xmap4, s, cfg, reinterpret_cast<const uint32_t*>(packed), y, status,
                               C2 > 0 ? block_tag(s_true, c, C2) : igemm_tag(s_true, c), x);
 }

@@ -1,0 +1,67 @@
+"""GPU parity of the tensor-core variant where a tile's channels are split over a cluster of thread blocks (wide groups on few
+pixels): every tiling it is taken on, even and uneven splits, full and short last tiles, against the fp64 oracle."""
+import pytest
+import torch
+
+from paper_2006_09791_b200 import build as gbuild
+from paper_2006_09791_b200 import gconv
+from paper_2006_09791_b200.workloads import Layer
+
+from gpu_util import check_layer
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    gbuild.build()
+
+
+CASES = [  # N, C_in, H, W, C_out, stride, groups
+    # widths that are not a multiple of 4: pairs of pixel tiles (odd and even counts), single tiles, one image, stride 2
+    (13, 512, 7, 7, 512, 1, 2), (13, 256, 13, 13, 256, 1, 2), (12, 512, 7, 7, 512, 1, 2), (4, 384, 10, 10, 384, 1, 1),
+    (1, 768, 5, 5, 768, 1, 1), (1, 320, 30, 30, 64, 1, 1), (13, 256, 13, 13, 512, 2, 2), (4, 384, 10, 10, 768, 2, 1),
+    (1, 128, 14, 14, 256, 2, 1), (9, 144, 7, 7, 64, 1, 1),
+    # (a split of 3 and of 5: slices of 22 and 13 filters, the last one short)
+    (5, 256, 13, 13, 256, 1, 1), (3, 256, 13, 13, 256, 1, 1),
+    # row boxes of one and two segments, filter tiles of 64 and 48, 16- and 32-channel stages, a padded width
+    (1, 192, 20, 20, 192, 1, 1), (1, 96, 40, 40, 96, 1, 1), (1, 256, 28, 28, 256, 1, 1), (2, 80, 24, 20, 80, 1, 1), (1, 256, 22, 54, 64, 1, 1),
+    # stride-2 row tiles, segment tilings with a stage per tap (both strides), 32-wide planes with halo stages
+    (4, 192, 20, 20, 384, 2, 1), (1, 96, 40, 40, 192, 2, 1), (6, 256, 8, 8, 256, 1, 1), (2, 128, 16, 16, 128, 1, 1),
+    (6, 256, 8, 8, 512, 2, 1), (1, 64, 32, 32, 64, 1, 1), (2, 160, 32, 32, 160, 1, 1), (1, 1024, 8, 8, 64, 1, 1),
+]
+
+
+@pytest.mark.parametrize("cfg", CASES)
+def test_split_channels(cfg):
+    N, Ci, H, W, Co, stride, g = cfg
+    L = Layer("split", N, Ci, H, W, Co, stride=stride, groups=g)
+    err, used = check_layer(L, seed=77)
+    assert used == gconv.GCONV_VARIANT_IGEMM_TF32
+
+
+def test_split_channels_back_to_back():
+    """Dependent launches: the next kernel's clusters start while this one's still exchange partial sums."""
+    L = Layer("chain", 2, 256, 13, 13, 256)
+    dev = torch.device("cuda:0")
+    d = gconv.gconv_desc_create(*L.desc_args())
+    try:
+        gen = torch.Generator(device=dev)
+        gen.manual_seed(5)
+        w = torch.randn((256, 256, 3, 3), generator=gen, device=dev) * (1.0 / 48.0)
+        wp = torch.empty(gconv.gconv_packed_bytes(d) // 4, device=dev)
+        gconv.gconv_pack_weights(d, w, wp)
+        runs = []
+        for _ in range(2):
+            bufs = [torch.randn((2, 256, 13, 13), generator=gen.manual_seed(6), device=dev)]
+            for _ in range(12):
+                bufs.append(torch.full_like(bufs[0], float("nan")))
+                gconv.gconv_forward(d, bufs[-2], wp, bufs[-1])
+            assert gconv.gconv_last_status(d) == gconv.GCONV_OK
+            runs.append(bufs[-1].clone())
+        assert bool(torch.isfinite(runs[0]).all()) and torch.equal(runs[0], runs[1])   # deterministic
+        one = torch.empty_like(runs[0])
+        gconv.gconv_forward(d, bufs[-2], wp, one)
+        assert gconv.gconv_last_status(d) == gconv.GCONV_OK and torch.equal(one, runs[1])
+    finally:
+        gconv.gconv_desc_destroy(d)
