@@ -1,14 +1,17 @@
-"""Builds libgconv.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds libgconv.so with nvcc for sm_100a (cross-compiles without a GPU) and the Python call module, both in-tree."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libgconv.so")
+CALLS = os.path.join(PKG, "_calls.so")
+CALLS_SRC = os.path.join(CSRC, "python_calls.c")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-shared",
               "-Xcompiler", "-fPIC", "--use_fast_math=false"]
@@ -27,7 +30,18 @@ def _stale() -> bool:
     return any(os.path.getmtime(p) > t for p in deps)
 
 
+def build_calls(force: bool = False) -> str:
+    """The C module behind gconv.gconv_forward and its like (argument marshalling; no CUDA in it)."""
+    if force or not os.path.exists(CALLS) or os.path.getmtime(CALLS_SRC) > os.path.getmtime(CALLS):
+        tmp = CALLS + ".tmp.%d" % os.getpid()
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"],
+                               "-o", tmp, CALLS_SRC])
+        os.replace(tmp, CALLS)
+    return CALLS
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_calls(force)
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -96,9 +96,11 @@ extern "C" int gconv_forward_host_static(gconv_desc_t d, const float* x_host, co
         opts.wait_us = (uint32_t)d->wait_us;
         opts.dbg_skip = d->dbg_skip;
         switch (d->variant) {
-            case GCONV_VARIANT_IGEMM_TF32:
-                e = igemm_forward(s, x_stage, w_packed, y_stage, status, sm_count, st, ws, opts);
+            case GCONV_VARIANT_IGEMM_TF32: {
+                const IgemmPlan* plan = igemm_plan(d->plans, s, 0, dev, sm_count, x_stage, &e);
+                if (plan != nullptr) e = igemm_run(plan, x_stage, w_packed, y_stage, status, st, ws, opts);
                 break;
+            }
             case GCONV_VARIANT_DIRECT_TILED:
                 e = tiled_forward(s, d->conv_plan(), x_stage, w_packed, y_stage, status, sm_count, st);
                 break;

@@ -39,7 +39,7 @@ int select_variant(const Shape& s) {
 }
 
 // What the descriptor's variant keeps from call to call: the staged FP32 kernel's tile (a search over a few hundred choices).
-void make_plan(gconv_desc* d) {
+void choose_tile(gconv_desc* d) {
     d->has_conv = false;
     if (d->variant == GCONV_VARIANT_DIRECT_GENERIC || (d->variant == GCONV_VARIANT_DIRECT_TILED && tiled_takes_conv(d->s)))
         d->has_conv = conv_config(d->s, 148, d->conv);
@@ -125,7 +125,8 @@ int gconv_desc_create_2d(gconv_desc_t* out, int N, int C_in, int H, int W, int C
     d->pack_epoch_seen = 0;
     d->wait_us = 0;
     d->dbg_skip = -1;
-    make_plan(d);
+    d->plans.store(nullptr);
+    choose_tile(d);
     *out = d;
     return GCONV_OK;
 }
@@ -138,6 +139,7 @@ int gconv_desc_create(gconv_desc_t* out, int N, int C_in, int H, int W, int C_ou
 int gconv_desc_destroy(gconv_desc_t d) {
     if (d == nullptr) return GCONV_OK;
     if (d->status_dev != nullptr) cudaFree(d->status_dev);
+    igemm_free_plans(d->plans);
     delete d;
     return GCONV_OK;
 }
@@ -180,14 +182,14 @@ int gconv_desc_set_variant(gconv_desc_t d, int variant) {
     if (variant == GCONV_VARIANT_AUTO) {
         d->variant = select_variant(d->s);
         d->forced = 0;
-        make_plan(d);
+        choose_tile(d);
         return GCONV_OK;
     }
     if (variant < GCONV_VARIANT_DIRECT_GENERIC || variant > GCONV_VARIANT_IGEMM_TF32) return GCONV_ERR_INVALID_ARG;
     if (!variant_supported(d->s, variant)) return GCONV_ERR_UNSUPPORTED;
     d->variant = variant;
     d->forced = 1;
-    make_plan(d);
+    choose_tile(d);
     return GCONV_OK;
 }
 
@@ -226,9 +228,11 @@ int gconv_forward(gconv_desc_t d, const float* x, const void* w_packed, float* y
             e = tiled_forward(d->s, d->conv_plan(), x, w_packed, y, d->status_dev, d->sm_count, st);
             break;
         case GCONV_VARIANT_IGEMM_TF32: {
-            const size_t need = igemm_scratch_bytes(d->s);
+            const IgemmPlan* plan = igemm_plan(d->plans, d->s, 0, d->device, d->sm_count, x, &e);
+            if (plan == nullptr) return fail_cuda(d, e);
+            const size_t need = igemm_plan_scratch(plan);
             if (need > 0 && (d->workspace == nullptr || d->workspace_bytes < need)) return GCONV_ERR_WORKSPACE;
-            e = igemm_forward(d->s, x, w_packed, y, d->status_dev, d->sm_count, st, need > 0 ? d->workspace : nullptr, launch_opts(d));
+            e = igemm_run(plan, x, w_packed, y, d->status_dev, st, need > 0 ? d->workspace : nullptr, launch_opts(d));
             break;
         }
         case GCONV_VARIANT_DIRECT_GENERIC:
@@ -276,11 +280,14 @@ int gconv_block_pack_weights(gconv_desc_t d, int C2, const float* w_ochw, const 
 int gconv_block_forward(gconv_desc_t d, int C2, const float* x, const void* w_packed, float* y2, void* stream) {
     if (d == nullptr || x == nullptr || w_packed == nullptr || y2 == nullptr) return GCONV_ERR_NULL;
     if (!aligned16(x) || !aligned16(w_packed) || !aligned16(y2)) return GCONV_ERR_ALIGNMENT;
-    if (!igemm_block_supported(d->s, C2)) return GCONV_ERR_UNSUPPORTED;
+    // (a plan exists for supported pairs only)
+    if (!igemm_has_plan(d->plans, C2) && !igemm_block_supported(d->s, C2)) return GCONV_ERR_UNSUPPORTED;
     int rc = ensure_device_state(d);
     if (rc != GCONV_OK) return rc;
-    const cudaError_t e = igemm_block_forward(d->s, C2, x, w_packed, y2, d->status_dev, d->sm_count, reinterpret_cast<cudaStream_t>(stream),
-                                              launch_opts(d));
+    cudaError_t e = cudaSuccess;
+    const IgemmPlan* plan = igemm_plan(d->plans, d->s, C2, d->device, d->sm_count, x, &e);
+    if (plan == nullptr) return fail_cuda(d, e);
+    e = igemm_run(plan, x, w_packed, y2, d->status_dev, reinterpret_cast<cudaStream_t>(stream), nullptr, launch_opts(d));
     return e == cudaSuccess ? GCONV_OK : fail_cuda(d, e);
 }
 

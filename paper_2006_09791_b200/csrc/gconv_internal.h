@@ -1,6 +1,7 @@
 // Internal declarations shared by the host API and the kernel translation units of libgconv.
 #pragma once
 #include <cuda_runtime.h>
+#include <atomic>
 #include <stddef.h>
 #include <stdint.h>
 
@@ -8,6 +9,7 @@
 
 namespace gconv {
 struct Status;
+struct IgemmPlan;
 struct Shape {
     int N, C_in, H, W, C_out, KH, KW, stride, pad, dilation, groups;   // stride, pad, dilation: the row axis (S_h of Algorithm 1)
     int Cg, Kg, H_out, W_out;
@@ -58,6 +60,9 @@ struct gconv_desc {
     int dbg_skip;                // failure-path test hook: stage fill that CTA 0's producer leaves out (-1 = none)
     gconv::ConvCfg conv;         // tile and launch geometry of the staged FP32 kernel, where the variant runs it (chosen once)
     bool has_conv;
+    // plans of the tensor-core variant, one per (pointwise outputs of a fused block, device): immutable once published, freed
+    // with the descriptor (calls of several threads may look them up and add to the list at the same time)
+    std::atomic<gconv::IgemmPlan*> plans;
     const gconv::ConvCfg* conv_plan() const { return has_conv ? &conv : nullptr; }
 };
 
@@ -202,10 +207,14 @@ cudaError_t igemm_pack(const Shape& s, const float* w, void* packed, cudaStream_
 bool igemm_block_supported(const Shape& s, int C2);
 size_t igemm_block_packed_bytes(const Shape& s, int C2);
 cudaError_t igemm_block_pack(const Shape& s, int C2, const float* w, const float* w2, void* packed, cudaStream_t st);
-cudaError_t igemm_block_forward(const Shape& s, int C2, const float* x, const void* packed, float* y2, Status* status, int sm_count,
-                                cudaStream_t st, const IgemmLaunchOpts& opts);
 size_t igemm_scratch_bytes(const Shape& s);   // device workspace the forward needs (padded copy of x), 0 for most shapes
-cudaError_t igemm_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, int sm_count,
-                          cudaStream_t st, float* scratch, const IgemmLaunchOpts& opts);
+// What a launch needs besides its pointers: configuration, instantiation, tag, tensor maps.  It follows the shape, C2 (0: the plain
+// convolution) and the device; `x` only has to be a valid 16-byte aligned address (the maps take each call's own).
+const IgemmPlan* igemm_plan(std::atomic<IgemmPlan*>& plans, const Shape& s, int C2, int device, int sm_count, const float* x, cudaError_t* err);
+void igemm_free_plans(std::atomic<IgemmPlan*>& plans);
+bool igemm_has_plan(const std::atomic<IgemmPlan*>& plans, int C2);
+size_t igemm_plan_scratch(const IgemmPlan* p);
+cudaError_t igemm_run(const IgemmPlan* plan, const float* x, const void* packed, float* y, Status* status, cudaStream_t st, float* scratch,
+                      const IgemmLaunchOpts& opts);
 
 }  // namespace gconv

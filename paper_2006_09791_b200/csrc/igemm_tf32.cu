@@ -40,6 +40,8 @@
 #include <cuda.h>
 #include <string.h>
 
+#include <new>
+
 #include "gconv_internal.h"
 
 namespace gconv {
@@ -2242,63 +2244,90 @@ cudaError_t igemm_pack(const Shape& s, const float* w, void* packed, cudaStream_
     return cudaGetLastError();
 }
 
-static cudaError_t igemm_launch(const Shape& s_true, int C2, const float* x_in, const void* packed, float* y, Status* status,
-                                int sm_count, cudaStream_t st, float* scratch, const IgemmLaunchOpts& opts);
-
-cudaError_t igemm_forward(const Shape& s_true, const float* x_in, const void* packed, float* y, Status* status, int sm_count,
-                          cudaStream_t st, float* scratch, const IgemmLaunchOpts& opts) {
-    return igemm_launch(s_true, 0, x_in, packed, y, status, sm_count, st, scratch, opts);
+namespace {
+typedef CUresult (*ReplaceAddressFn)(CUtensorMap*, void*);
+ReplaceAddressFn get_replace_fn() {
+    static ReplaceAddressFn fn = nullptr;
+    if (fn == nullptr) {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuTensorMapReplaceAddress", &p, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<ReplaceAddressFn>(p);
+    }
+    return fn;
 }
 
-cudaError_t igemm_block_forward(const Shape& s, int C2, const float* x, const void* packed, float* y2, Status* status, int sm_count,
-                                cudaStream_t st, const IgemmLaunchOpts& opts) {
-    return igemm_launch(s, C2, x, packed, y2, status, sm_count, st, nullptr, opts);
-}
+using KernelFn = void (*)(const CUtensorMap, const CUtensorMap, const Shape, const IgemmCfg, const uint32_t*, float*, Status*, uint32_t,
+                              const float*);
+const KernelFn kernels[kFamilies] = {igemm_tf32_kernel<0>, igemm_tf32_kernel<1>, igemm_tf32_kernel<2>,
+                                                igemm_tf32_kernel<3>, igemm_tf32_kernel<4>, igemm_tf32_kernel<5>,
+                                                igemm_tf32_kernel<6>, igemm_tf32_kernel<7>, igemm_tf32_kernel<8>,
+                                                igemm_tf32_kernel<9>, igemm_tf32_kernel<10>, igemm_tf32_kernel<11>,
+                                                igemm_tf32_kernel<12>, igemm_tf32_kernel<13>,
+                                                igemm_tf32_kernel<14>, igemm_tf32_kernel<15>, igemm_tf32_kernel<16>,
+                                                igemm_tf32_kernel<17>, igemm_tf32_kernel<18>, igemm_tf32_kernel<19>, igemm_tf32_kernel<20>,
+                                                igemm_tf32_kernel<21>, igemm_tf32_kernel<22>, igemm_tf32_kernel<23>,
+                                                igemm_tf32_kernel<24>, igemm_tf32_kernel<25>, igemm_tf32_kernel<26>, igemm_tf32_kernel<27>, igemm_tf32_kernel<28>, igemm_tf32_kernel<29>, igemm_tf32_kernel<30>,
+                                                igemm_tf32_kernel<31>, igemm_tf32_kernel<32>, igemm_tf32_kernel<33>, igemm_tf32_kernel<34>,
+                                                igemm_tf32_kernel<35>, igemm_tf32_kernel<36>, igemm_tf32_kernel<37>, igemm_tf32_kernel<38>};
+}  // namespace
 
-static cudaError_t igemm_launch(const Shape& s_true, int C2, const float* x_in, const void* packed, float* y, Status* status,
-                                int sm_count, cudaStream_t st, float* scratch, const IgemmLaunchOpts& opts) {
-    IgemmCfg c = igemm_config_c2(s_true, sm_count, C2);
-    if (opts.wait_us > 0) c.wait_us = opts.wait_us;
-    c.dbg_skip = opts.dbg_skip;
+struct IgemmPlan {
+    IgemmCfg cfg;
+    Shape s;                     // the problem as the kernel sees it (padded plane, re-cut pointwise plane)
+    KernelFn kernel;
+    uint32_t tag;
+    int C2, device;
+    bool use_map, use_map4;      // which tensor maps take the call's input address (an unused one is a copy of the other, or zeros)
+    CUtensorMap map, map4;
+    // zero-padded copy of x (widths no tiling addresses): the true plane and the launch that fills the copy
+    size_t scratch_bytes, pad_total, pad_planes;
+    int pad_blocks, pad_H, pad_W;
+    FastDiv pad_div_plane, pad_div_row;
+    IgemmPlan* next;
+};
+
+static cudaError_t make_plan(IgemmPlan& p, const Shape& s_true, int sm_count, const float* x) {
+    p.cfg = igemm_config_c2(s_true, sm_count, p.C2);
+    const IgemmCfg c = p.cfg;
+    p.tag = p.C2 > 0 ? block_tag(s_true, c, p.C2) : igemm_tag(s_true, c);
     Shape s = as_3x3(s_true);
-    const float* x = x_in;
+    p.scratch_bytes = 0;
     if (c.padded) {
-        if (scratch == nullptr) return cudaErrorInvalidValue;
         const IgemmGeom ge = igemm_geom(s);
-        const size_t planes = (size_t)s.N * s.C_in;
-        const size_t total = planes * ge.Hp * (ge.Wp / 4);
-        const int blocks = (int)((total + 255) / 256 < (size_t)sm_count * 16 ? (total + 255) / 256 : (size_t)sm_count * 16);
-        const FastDiv div_plane = make_fastdiv((uint32_t)(ge.Hp * (ge.Wp / 4))), div_row = make_fastdiv((uint32_t)(ge.Wp / 4));
-        if (total < (1ull << 32))
-            igemm_pad_kernel<uint32_t><<<blocks, 256, 0, st>>>(x_in, scratch, planes, s.H, s.W, ge.Hp, ge.Wp, div_plane, div_row);
-        else
-            igemm_pad_kernel<uint64_t><<<blocks, 256, 0, st>>>(x_in, scratch, planes, s.H, s.W, ge.Hp, ge.Wp, div_plane, div_row);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+        p.pad_H = s.H;
+        p.pad_W = s.W;
+        p.pad_planes = (size_t)s.N * s.C_in;
+        p.pad_total = p.pad_planes * ge.Hp * (ge.Wp / 4);
+        p.pad_blocks = (int)((p.pad_total + 255) / 256 < (size_t)sm_count * 16 ? (p.pad_total + 255) / 256 : (size_t)sm_count * 16);
+        p.pad_div_plane = make_fastdiv((uint32_t)(ge.Hp * (ge.Wp / 4)));
+        p.pad_div_row = make_fastdiv((uint32_t)(ge.Wp / 4));
         s.H = ge.Hp;
         s.W = ge.Wp;
-        x = scratch;
+        p.scratch_bytes = sizeof(float) * p.pad_planes * ge.Hp * ge.Wp;
     }
+    p.s = s;
     EncodeTiledFn encode = get_encode_fn();
-    if (encode == nullptr) return cudaErrorNotSupported;
-    CUtensorMap xmap;
+    if (encode == nullptr || get_replace_fn() == nullptr) return cudaErrorNotSupported;
+    CUtensorMap &xmap = p.map, &xmap4 = p.map4;
     const cuuint64_t HW = (cuuint64_t)s.H * s.W;
     const cuuint64_t dims[3] = {HW, (cuuint64_t)s.C_in, (cuuint64_t)s.N};
     const cuuint64_t strides[2] = {HW * 4, HW * 4 * (cuuint64_t)s.C_in};
     const cuuint32_t box[3] = {32, (cuuint32_t)c.CK, 1};
     const cuuint32_t estr[3] = {1, 1, 1};
-    if (c.soft) {
-        memset(&xmap, 0, sizeof(xmap));      // the gather producer uses no swizzled map (and odd planes cannot have one)
-    } else {
+    memset(&xmap, 0, sizeof(xmap));              // (the gather producer uses no swizzled map, and odd planes cannot have one)
+    p.use_map = !c.soft;
+    if (p.use_map) {
         const CUresult r = encode(&xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(x), dims, strides, box, estr,
                                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
     }
+    xmap4 = xmap;
     // 4-D view for whole-tile copies: (pixel, channel, 32-pixel segment, image); the segment axis re-walks the
     // pixel axis in steps of 128 bytes, so one box covers nseg consecutive segments.
-    IgemmCfg cfg = c;
-    CUtensorMap xmap4 = xmap;
+    IgemmCfg& cfg = p.cfg;
     cfg.fast4 = 0;
     if (c.soft) {
         // gather producer: raw boxes of (boxpx flat pixels, CK channels) of one image, unswizzled; planes that are not a
@@ -2349,52 +2378,89 @@ static cudaError_t igemm_launch(const Shape& s_true, int C2, const float* x_in, 
         else
             xmap4 = xmap;
     }
-    using KernelFn = void (*)(const CUtensorMap, const CUtensorMap, const Shape, const IgemmCfg, const uint32_t*, float*, Status*, uint32_t,
-                              const float*);
-    static const KernelFn kernels[kFamilies] = {igemm_tf32_kernel<0>, igemm_tf32_kernel<1>, igemm_tf32_kernel<2>,
-                                                igemm_tf32_kernel<3>, igemm_tf32_kernel<4>, igemm_tf32_kernel<5>,
-                                                igemm_tf32_kernel<6>, igemm_tf32_kernel<7>, igemm_tf32_kernel<8>,
-                                                igemm_tf32_kernel<9>, igemm_tf32_kernel<10>, igemm_tf32_kernel<11>,
-                                                igemm_tf32_kernel<12>, igemm_tf32_kernel<13>,
-                                                igemm_tf32_kernel<14>, igemm_tf32_kernel<15>, igemm_tf32_kernel<16>,
-                                                igemm_tf32_kernel<17>, igemm_tf32_kernel<18>, igemm_tf32_kernel<19>, igemm_tf32_kernel<20>,
-                                                igemm_tf32_kernel<21>, igemm_tf32_kernel<22>, igemm_tf32_kernel<23>,
-                                                igemm_tf32_kernel<24>, igemm_tf32_kernel<25>, igemm_tf32_kernel<26>, igemm_tf32_kernel<27>, igemm_tf32_kernel<28>, igemm_tf32_kernel<29>, igemm_tf32_kernel<30>,
-                                                igemm_tf32_kernel<31>, igemm_tf32_kernel<32>, igemm_tf32_kernel<33>, igemm_tf32_kernel<34>,
-                                                igemm_tf32_kernel<35>, igemm_tf32_kernel<36>, igemm_tf32_kernel<37>, igemm_tf32_kernel<38>};
+    p.use_map4 = cfg.fast4 != 0;
     int fam = 0;
     for (int f = 1; f < kFamilies && fam == 0; ++f)
         if (family_matches(f, s, cfg)) fam = f;
     if (cfg.spl && family(fam).spl != 1) return cudaErrorInvalidValue;     // nor split-channel code
     if (cfg.pair && family(fam).pair != 1) return cudaErrorInvalidValue;   // the generic instantiation has no pair-tile code
     if (cfg.soft && cfg.egroups == 2 && family(fam).soft != cfg.soft) return cudaErrorInvalidValue;   // 29 warps: only the wide-group gather instantiations take them
-    static bool attr_set[64][kFamilies] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || !attr_set[dev][fam]) {
-        cudaError_t e = cudaFuncSetAttribute(kernels[fam], cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) attr_set[dev][fam] = true;
+    p.kernel = kernels[fam];
+    return cudaFuncSetAttribute(p.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+}
+
+const IgemmPlan* igemm_plan(std::atomic<IgemmPlan*>& plans, const Shape& s, int C2, int device, int sm_count, const float* x, cudaError_t* err) {
+    IgemmPlan* head = plans.load(std::memory_order_acquire);
+    for (const IgemmPlan* p = head; p != nullptr; p = p->next)
+        if (p->C2 == C2 && p->device == device) return p;
+    IgemmPlan* p = new (std::nothrow) IgemmPlan();
+    if (p == nullptr) { *err = cudaErrorMemoryAllocation; return nullptr; }
+    p->C2 = C2;
+    p->device = device;
+    *err = make_plan(*p, s, sm_count, x);
+    if (*err != cudaSuccess) { delete p; return nullptr; }
+    p->next = head;
+    // (two threads that miss at the same time both add their plan: equal, one of them is simply never found)
+    while (!plans.compare_exchange_weak(p->next, p, std::memory_order_release, std::memory_order_relaxed)) {}
+    return p;
+}
+
+bool igemm_has_plan(const std::atomic<IgemmPlan*>& plans, int C2) {
+    for (const IgemmPlan* p = plans.load(std::memory_order_acquire); p != nullptr; p = p->next)
+        if (p->C2 == C2) return true;
+    return false;
+}
+
+void igemm_free_plans(std::atomic<IgemmPlan*>& plans) {
+    for (IgemmPlan* p = plans.exchange(nullptr); p != nullptr;) {
+        IgemmPlan* next = p->next;
+        delete p;
+        p = next;
     }
+}
+
+size_t igemm_plan_scratch(const IgemmPlan* p) { return p->scratch_bytes; }
+
+// A call takes its plan (a call used to work the configuration out twice and encode both tensor maps, 1 us of host time) and
+// puts its own input address into copies of the maps.
+cudaError_t igemm_run(const IgemmPlan* plan, const float* x, const void* packed, float* y, Status* status, cudaStream_t st, float* scratch,
+                      const IgemmLaunchOpts& opts) {
+    const IgemmPlan& p = *plan;
+    IgemmCfg cfg = p.cfg;
+    if (opts.wait_us > 0) cfg.wait_us = opts.wait_us;
+    cfg.dbg_skip = opts.dbg_skip;
+    if (p.scratch_bytes > 0) {
+        if (scratch == nullptr) return cudaErrorInvalidValue;
+        if (p.pad_total < (1ull << 32))
+            igemm_pad_kernel<uint32_t><<<p.pad_blocks, 256, 0, st>>>(x, scratch, p.pad_planes, p.pad_H, p.pad_W, p.s.H, p.s.W, p.pad_div_plane, p.pad_div_row);
+        else
+            igemm_pad_kernel<uint64_t><<<p.pad_blocks, 256, 0, st>>>(x, scratch, p.pad_planes, p.pad_H, p.pad_W, p.s.H, p.s.W, p.pad_div_plane, p.pad_div_row);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        x = scratch;
+    }
+    CUtensorMap xmap = p.map;
+    const ReplaceAddressFn replace = get_replace_fn();
+    if (p.use_map && replace(&xmap, const_cast<float*>(x)) != CUDA_SUCCESS) return cudaErrorInvalidValue;
+    CUtensorMap xmap4 = p.use_map4 ? p.map4 : xmap;
+    if (p.use_map4 && replace(&xmap4, const_cast<float*>(x)) != CUDA_SUCCESS) return cudaErrorInvalidValue;
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((unsigned)c.grid);
-    lc.blockDim = dim3((unsigned)c.threads);
-    lc.dynamicSmemBytes = c.smem_bytes;
+    lc.gridDim = dim3((unsigned)cfg.grid);
+    lc.blockDim = dim3((unsigned)cfg.threads);
+    lc.dynamicSmemBytes = cfg.smem_bytes;
     lc.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = opts.pdl ? 1 : 0;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)c.split;
+    attr[1].val.clusterDim.x = (unsigned)cfg.split;
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     lc.attrs = attr;
     // Without the attribute the kernel starts only after everything before it in the stream has completed and is
     // visible (griddepcontrol.* are then no-ops): used for the first forward after any weight packing, because the
     // kernel reads the packed weights before its dependency wait.
-    lc.numAttrs = c.spl ? 2 : (opts.pdl ? 1 : 0);
-    return cudaLaunchKernelEx(&lc, kernels[fam], xmap, xmap4, s, cfg, reinterpret_cast<const uint32_t*>(packed), y, status,
-                              C2 > 0 ? block_tag(s_true, c, C2) : igemm_tag(s_true, c), x);
+    lc.numAttrs = cfg.spl ? 2 : (opts.pdl ? 1 : 0);
+    return cudaLaunchKernelEx(&lc, p.kernel, xmap, xmap4, p.s, cfg, reinterpret_cast<const uint32_t*>(packed), y, status, p.tag, x);
 }
-
 
 }  // namespace gconv

@@ -1,5 +1,7 @@
 """ctypes binding of the libgconv C ABI (include/gconv.h): same names, argument marshalling only.
 
+The calls made per layer and pass (`gconv_forward`, `gconv_block_forward`, `gconv_forward_host`) are
+marshalled in C where the `_calls` module is built (paper_2006_09791_b200.build does), by ctypes otherwise.
 Every step of the convolution runs inside the CUDA library.  There is no fallback: if the shared
 library has not been built, importing a function from here raises.  torch is used by callers for
 device memory and streams; this module accepts raw integer pointers or anything with
@@ -9,6 +11,11 @@ from __future__ import annotations
 
 import ctypes
 import os
+
+try:
+    from . import _calls
+except ImportError:          # not built yet (a fresh checkout): the ctypes functions below are used as they are
+    _calls = None
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libgconv.so")
 _lib = None
@@ -64,6 +71,10 @@ _SIGNATURES = {
 }
 
 
+# bound in this order by _calls.bind
+_NATIVE_CALLS = ("gconv_forward", "gconv_block_forward", "gconv_forward_host")
+
+
 class GconvError(RuntimeError):
     def __init__(self, status: int, where: str):
         self.status = status
@@ -86,6 +97,8 @@ def load() -> ctypes.CDLL:
             fn = getattr(lib, name)
             fn.restype = res
             fn.argtypes = args
+        if _calls is not None:
+            _calls.bind(*(ctypes.cast(getattr(lib, name), _vp).value for name in _NATIVE_CALLS))
         _lib = lib
     return _lib
 
@@ -231,3 +244,10 @@ def gconv_last_cuda_error(desc) -> int:
 
 def gconv_last_status_detail(desc) -> int:
     return int(load().gconv_last_status_detail(desc))
+
+
+if _calls is not None:       # same names, arguments and results
+    _calls.setup(load, _check)
+    gconv_forward = _calls.gconv_forward
+    gconv_block_forward = _calls.gconv_block_forward
+    gconv_forward_host = _calls.gconv_forward_host
