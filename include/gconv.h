@@ -168,6 +168,8 @@ int gconv_desc_set_workspace(gconv_desc_t desc, void *workspace, size_t bytes);
 /*
  * gconv_forward_host -- the same operation (Section II) for callers whose activations live in host memory:
  * copies x to the device, runs gconv_forward and copies y back, all enqueued on `stream` in order.
+ * Batches of a few MB and more are cut into parts whose copies and kernels overlap on streams the library keeps; `stream`
+ * still orders the whole call (work before it is waited for, what follows it finds y_host complete).
  *   x_host    host, fp32 [N, C_in, H, W] (pinned memory makes the copies asynchronous).
  *   y_host    host, fp32 [N, C_out, H_out, W_out], written when the stream reaches that point.
  *   x_stage, y_stage   device staging buffers of the sizes of x and y, caller-owned.

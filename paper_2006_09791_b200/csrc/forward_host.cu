@@ -1,0 +1,258 @@
+// gconv_forward_host: grouped convolution on host buffers, copies and kernels of successive parts of the batch overlapped.
+//
+// What bounds it is the host link (PCIe), which carries both directions at once: copy-in, kernel and copy-out one after the
+// other leave half of it idle.  The batch is cut into up to kMaxParts runs of images; their copies in are enqueued on one side
+// stream, the kernels on the caller's stream as each part lands, the copies out on a second side stream.  The caller's stream
+// waits for the last copy out, so the call keeps its contract: everything happens in stream order, y_host is complete when the
+// stream gets there.  51 MB each way (64 channels @56x56, N = 64, g = 8): 1870 -> 1297 us; the link moves 84 GB/s both ways
+// together on this machine (1224 us), the rest is the first part's way in and the last one's way out.
+#include <new>
+
+#include "gconv_internal.h"
+
+using namespace gconv;
+
+namespace gconv {
+
+constexpr int kMaxParts = 5;                   // at most (the example above with 8 parts: 1320 us, with 16: 2000)
+constexpr size_t kPartBytes = 1024 * 1024;     // bytes a part moves in the smaller direction, at least: a part costs some 10 us of enqueueing and copy start-up
+constexpr int kMaxLanes = 4;
+
+// Side streams and events of a call in flight.  Creating them takes 200 us, as long as a small call, so they are kept for the next
+// call of any descriptor: at most kMaxLanes (a call that finds them all in flight runs in order), destroyed with the last
+// descriptor that uses them.
+struct Lane {
+    int device;
+    bool busy;                       // a thread is enqueueing on it
+    cudaStream_t last;               // the caller's stream of its last call
+    cudaStream_t in, out;
+    cudaEvent_t begin, end, landed[kMaxParts], done[kMaxParts];
+};
+static std::mutex g_lane_mutex;
+static Lane* g_lanes[kMaxLanes] = {};
+static int g_lane_users = 0;         // descriptors with a HostPipe
+
+// What a descriptor keeps: how its batch is cut.
+struct HostPipe {
+    int parts, images;               // parts the batch is cut into (0: not cut), images of each but the last
+    gconv_desc* part[2];             // descriptors of `images` images and of the last, shorter part
+};
+
+static void close_lane(Lane* l) {
+    for (int i = 0; i < kMaxParts; ++i) {
+        if (l->landed[i] != nullptr) cudaEventDestroy(l->landed[i]);
+        if (l->done[i] != nullptr) cudaEventDestroy(l->done[i]);
+    }
+    if (l->begin != nullptr) cudaEventDestroy(l->begin);
+    if (l->end != nullptr) cudaEventDestroy(l->end);
+    if (l->in != nullptr) cudaStreamDestroy(l->in);
+    if (l->out != nullptr) cudaStreamDestroy(l->out);
+    delete l;
+}
+
+static Lane* open_lane(int device) {
+    Lane* l = new (std::nothrow) Lane();
+    if (l == nullptr) return nullptr;
+    l->device = device;
+    cudaError_t e = cudaStreamCreateWithFlags(&l->in, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&l->out, cudaStreamNonBlocking);
+    auto event = [&](cudaEvent_t* v) {
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(v, cudaEventDisableTiming);
+    };
+    event(&l->begin);
+    event(&l->end);
+    for (int i = 0; i < kMaxParts; ++i) {
+        event(&l->landed[i]);
+        event(&l->done[i]);
+    }
+    if (e == cudaSuccess) return l;
+    (void)cudaGetLastError();
+    close_lane(l);
+    return nullptr;
+}
+
+// The lane of the last call on this stream (in stream order anyway), else one with nothing in flight (a call's side streams must
+// not wait for another caller's stream), else a new one; nullptr if there is none.
+static Lane* take_lane(int device, cudaStream_t st) {
+    std::lock_guard<std::mutex> lock(g_lane_mutex);
+    // (another thread may be capturing a stream: a query or a creation here is none of that capture's business)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    (void)cudaThreadExchangeStreamCaptureMode(&mode);
+    Lane* found = nullptr;
+    int empty = -1;
+    for (int i = 0; i < kMaxLanes; ++i) {
+        Lane* l = g_lanes[i];
+        if (l != nullptr && !l->busy && l->device == device && l->last == st) found = l;
+        if (l == nullptr && empty < 0) empty = i;
+    }
+    for (int i = 0; i < kMaxLanes && found == nullptr; ++i) {
+        Lane* l = g_lanes[i];
+        if (l == nullptr || l->busy || l->device != device) continue;
+        if (cudaEventQuery(l->end) == cudaSuccess) found = l;
+        else (void)cudaGetLastError();               // (cudaErrorNotReady)
+    }
+    if (found == nullptr && empty >= 0) found = g_lanes[empty] = open_lane(device);
+    if (found != nullptr) {
+        found->busy = true;
+        found->last = st;
+    }
+    (void)cudaThreadExchangeStreamCaptureMode(&mode);
+    return found;
+}
+static void give_back(Lane* l) {
+    std::lock_guard<std::mutex> lock(g_lane_mutex);
+    l->busy = false;
+}
+
+void free_host_pipe(gconv_desc* d) {
+    HostPipe* p = d->host_pipe;
+    if (p == nullptr) return;
+    for (int i = 0; i < 2; ++i)
+        if (p->part[i] != nullptr) gconv_desc_destroy(p->part[i]);
+    delete p;
+    d->host_pipe = nullptr;
+    std::lock_guard<std::mutex> lock(g_lane_mutex);
+    if (--g_lane_users > 0) return;
+    for (int i = 0; i < kMaxLanes; ++i) {
+        if (g_lanes[i] != nullptr && !g_lanes[i]->busy) {
+            close_lane(g_lanes[i]);  // (streams and events are released once their work has completed)
+            g_lanes[i] = nullptr;
+        }
+    }
+}
+
+// A descriptor of the same layer with n images that runs on weights packed for `d`, or nullptr.
+static gconv_desc* part_of(gconv_desc* d, int n) {
+    const Shape& s = d->s;
+    gconv_desc* c = nullptr;
+    if (gconv_desc_create_2d(&c, n, s.C_in, s.H, s.W, s.C_out, s.KH, s.KW, s.stride, s.stride_w, s.pad, s.pad_w, s.dilation, s.dilation_w,
+                             s.groups) != GCONV_OK)
+        return nullptr;
+    if (gconv_desc_set_variant(c, d->variant) != GCONV_OK ||
+        (d->variant == GCONV_VARIANT_IGEMM_TF32 && igemm_layout_tag(c->s) != igemm_layout_tag(s))) {
+        gconv_desc_destroy(c);
+        return nullptr;
+    }
+    return c;
+}
+
+// Cuts the batch: as many parts as the size allows, fewer where the packed layout of a shorter batch differs.
+static void cut(gconv_desc* d, HostPipe* p, size_t xb, size_t yb) {
+    const Shape& s = d->s;
+    const size_t most = (xb < yb ? xb : yb) / kPartBytes;
+    // parts start on 16-byte boundaries of x and y
+    const bool odd = ((size_t)s.C_in * s.H * s.W) % 4 != 0 || ((size_t)s.C_out * s.H_out * s.W_out) % 4 != 0;
+    for (int parts = most < (size_t)kMaxParts ? (int)most : kMaxParts; parts >= 2; --parts) {
+        int images = (s.N + parts - 1) / parts;
+        if (odd) images = (images + 3) & ~3;
+        const int count = (s.N + images - 1) / images;
+        if (count < 2) continue;
+        const int last = s.N - (count - 1) * images;
+        gconv_desc* a = part_of(d, images);
+        gconv_desc* b = a != nullptr && last != images ? part_of(d, last) : nullptr;
+        if (a == nullptr || (last != images && b == nullptr)) {
+            if (a != nullptr) gconv_desc_destroy(a);
+            continue;
+        }
+        p->parts = count;
+        p->images = images;
+        p->part[0] = a;
+        p->part[1] = b;
+        return;
+    }
+}
+
+}  // namespace gconv
+
+extern "C" int gconv_forward_host(gconv_desc_t d, const float* x_host, const void* w_packed, float* y_host, float* x_stage,
+                                  float* y_stage, void* stream) {
+    if (d == nullptr || x_host == nullptr || y_host == nullptr || x_stage == nullptr || y_stage == nullptr) return GCONV_ERR_NULL;
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    const Shape& s = d->s;
+    const size_t xi = sizeof(float) * (size_t)s.C_in * s.H * s.W, yi = sizeof(float) * (size_t)s.C_out * s.H_out * s.W_out;
+    const size_t xb = xi * s.N, yb = yi * s.N;
+    auto in_order = [&]() -> int {
+        cudaError_t e = cudaMemcpyAsync(x_stage, x_host, xb, cudaMemcpyHostToDevice, st);
+        if (e != cudaSuccess) return fail_cuda(d, e);
+        const int rc = gconv_forward(d, x_stage, w_packed, y_stage, stream);
+        if (rc != GCONV_OK) return rc;
+        e = cudaMemcpyAsync(y_host, y_stage, yb, cudaMemcpyDeviceToHost, st);
+        return e == cudaSuccess ? GCONV_OK : fail_cuda(d, e);
+    };
+    // One image, or little to move: nothing to overlap.  A stream that is being captured keeps the plain order (the side streams
+    // would belong to the capture until it ends, and other threads may be using them).
+    if (s.N < 2 || (xb < yb ? xb : yb) < 2 * kPartBytes || d->dbg_skip >= 0) return in_order();
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        (void)cudaGetLastError();
+        return in_order();
+    }
+    if (w_packed == nullptr) return GCONV_ERR_NULL;
+    const uintptr_t bits = reinterpret_cast<uintptr_t>(x_stage) | reinterpret_cast<uintptr_t>(y_stage) | reinterpret_cast<uintptr_t>(w_packed);
+    if ((bits & 15u) != 0) return GCONV_ERR_ALIGNMENT;
+    int rc = ensure_device_state(d);
+    if (rc != GCONV_OK) return rc;
+
+    // The lock covers the whole enqueue: the part descriptors are this descriptor's.
+    std::lock_guard<std::mutex> lock(d->host_mutex);
+    if (d->host_pipe != nullptr && d->host_pipe->parts > 0 && d->host_pipe->part[0]->variant != d->variant) free_host_pipe(d);
+    if (d->host_pipe == nullptr) {
+        HostPipe* fresh = new (std::nothrow) HostPipe();
+        if (fresh == nullptr) return in_order();
+        {
+            std::lock_guard<std::mutex> lanes(g_lane_mutex);
+            ++g_lane_users;
+        }
+        d->host_pipe = fresh;
+        cut(d, fresh, xb, yb);
+    }
+    HostPipe* p = d->host_pipe;
+    if (p->parts == 0) return in_order();
+    for (int i = 0; i < 2; ++i) {
+        gconv_desc* c = p->part[i];
+        if (c == nullptr) continue;
+        c->device = d->device;
+        c->sm_count = d->sm_count;
+        c->workspace = d->workspace;               // the parts' kernels follow each other on the caller's stream
+        c->workspace_bytes = d->workspace_bytes;
+        c->wait_us = d->wait_us;
+        if (gconv_workspace_bytes(c) > c->workspace_bytes) return GCONV_ERR_WORKSPACE;
+    }
+    Lane* l = take_lane(d->device, st);
+    if (l == nullptr) return in_order();
+    cudaError_t e = cudaSuccess;
+    bool side = false;                             // the side streams hold work that uses the caller's buffers
+    auto check = [&](cudaError_t r) { if (e == cudaSuccess) e = r; return e == cudaSuccess; };
+    if (check(cudaEventRecord(l->begin, st)) && check(cudaStreamWaitEvent(l->in, l->begin, 0))) {
+        for (int i = 0; i < p->parts && e == cudaSuccess; ++i) {
+            const size_t n0 = (size_t)i * p->images, n = i + 1 < p->parts ? (size_t)p->images : (size_t)s.N - n0;
+            side = true;
+            check(cudaMemcpyAsync(reinterpret_cast<char*>(x_stage) + n0 * xi, reinterpret_cast<const char*>(x_host) + n0 * xi, n * xi,
+                                  cudaMemcpyHostToDevice, l->in));
+            check(cudaEventRecord(l->landed[i], l->in));
+        }
+        for (int i = 0; i < p->parts && e == cudaSuccess && rc == GCONV_OK; ++i) {
+            const size_t n0 = (size_t)i * p->images, n = i + 1 < p->parts ? (size_t)p->images : (size_t)s.N - n0;
+            gconv_desc* c = (i + 1 == p->parts && p->part[1] != nullptr) ? p->part[1] : p->part[0];
+            char* ys = reinterpret_cast<char*>(y_stage) + n0 * yi;
+            if (!check(cudaStreamWaitEvent(st, l->landed[i], 0))) break;
+            rc = launch_forward(c, reinterpret_cast<const float*>(reinterpret_cast<const char*>(x_stage) + n0 * xi), w_packed,
+                                reinterpret_cast<float*>(ys), d->status_dev, st, false);
+            if (rc != GCONV_OK) { d->last_cuda_error = c->last_cuda_error; break; }
+            check(cudaEventRecord(l->done[i], st));
+            check(cudaStreamWaitEvent(l->out, l->done[i], 0));
+            check(cudaMemcpyAsync(reinterpret_cast<char*>(y_host) + n0 * yi, ys, n * yi, cudaMemcpyDeviceToHost, l->out));
+        }
+    }
+    if (side) {
+        // the caller's stream takes in both side streams, after an error too
+        const bool had = e != cudaSuccess || rc != GCONV_OK;
+        if (had && cudaEventRecord(l->begin, l->in) == cudaSuccess) (void)cudaStreamWaitEvent(st, l->begin, 0);
+        cudaError_t j = cudaEventRecord(l->end, l->out);
+        if (j == cudaSuccess) j = cudaStreamWaitEvent(st, l->end, 0);
+        check(j);
+    }
+    give_back(l);
+    if (e != cudaSuccess) return fail_cuda(d, e);
+    return rc;
+}

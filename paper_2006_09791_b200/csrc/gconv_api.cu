@@ -45,6 +45,22 @@ void choose_tile(gconv_desc* d) {
         d->has_conv = conv_config(d->s, 148, d->conv);
 }
 
+inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
+IgemmLaunchOpts launch_opts(gconv_desc* d) {
+    IgemmLaunchOpts o;
+    const unsigned long long epoch = g_pack_epoch.load(std::memory_order_relaxed);
+    o.pdl = d->pack_epoch_seen == epoch;
+    d->pack_epoch_seen = epoch;
+    o.wait_us = (uint32_t)d->wait_us;
+    o.dbg_skip = d->dbg_skip;
+    return o;
+}
+
+}  // namespace
+
+namespace gconv {
+
 int fail_cuda(gconv_desc* d, cudaError_t e) {
     d->last_cuda_error = (int)e;
     (void)cudaGetLastError();  // clear the sticky-free error state
@@ -70,19 +86,33 @@ int ensure_device_state(gconv_desc* d) {
     return GCONV_OK;
 }
 
-inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
-
-IgemmLaunchOpts launch_opts(gconv_desc* d) {
-    IgemmLaunchOpts o;
-    const unsigned long long epoch = g_pack_epoch.load(std::memory_order_relaxed);
-    o.pdl = d->pack_epoch_seen == epoch;
-    d->pack_epoch_seen = epoch;
-    o.wait_us = (uint32_t)d->wait_us;
-    o.dbg_skip = d->dbg_skip;
-    return o;
+// Enqueues the kernels of the descriptor's variant.  `may_overlap`: the set-up of a tensor-core kernel may overlap the previous
+// kernel's tail (not where a copy or an event precedes it).
+int launch_forward(gconv_desc* d, const float* x, const void* packed, float* y, Status* status, cudaStream_t st, bool may_overlap) {
+    cudaError_t e = cudaSuccess;
+    switch (d->variant) {
+        case GCONV_VARIANT_DIRECT_TILED:
+            e = tiled_forward(d->s, d->conv_plan(), x, packed, y, status, d->sm_count, st);
+            break;
+        case GCONV_VARIANT_IGEMM_TF32: {
+            const IgemmPlan* plan = igemm_plan(d->plans, d->s, 0, d->device, d->sm_count, x, &e);
+            if (plan == nullptr) return fail_cuda(d, e);
+            const size_t need = igemm_plan_scratch(plan);
+            if (need > 0 && (d->workspace == nullptr || d->workspace_bytes < need)) return GCONV_ERR_WORKSPACE;
+            IgemmLaunchOpts opts = launch_opts(d);
+            opts.pdl = opts.pdl && may_overlap;
+            e = igemm_run(plan, x, packed, y, status, st, need > 0 ? d->workspace : nullptr, opts);
+            break;
+        }
+        case GCONV_VARIANT_DIRECT_GENERIC:
+        default:
+            e = generic_forward(d->s, d->conv_plan(), x, packed, y, status, d->sm_count, generic_tag(d->s), st);
+            break;
+    }
+    return e == cudaSuccess ? GCONV_OK : fail_cuda(d, e);
 }
 
-}  // namespace
+}  // namespace gconv
 
 extern "C" {
 
@@ -126,6 +156,7 @@ int gconv_desc_create_2d(gconv_desc_t* out, int N, int C_in, int H, int W, int C
     d->wait_us = 0;
     d->dbg_skip = -1;
     d->plans.store(nullptr);
+    d->host_pipe = nullptr;
     choose_tile(d);
     *out = d;
     return GCONV_OK;
@@ -139,6 +170,7 @@ int gconv_desc_create(gconv_desc_t* out, int N, int C_in, int H, int W, int C_ou
 int gconv_desc_destroy(gconv_desc_t d) {
     if (d == nullptr) return GCONV_OK;
     if (d->status_dev != nullptr) cudaFree(d->status_dev);
+    free_host_pipe(d);
     igemm_free_plans(d->plans);
     delete d;
     return GCONV_OK;
@@ -221,43 +253,7 @@ int gconv_forward(gconv_desc_t d, const float* x, const void* w_packed, float* y
     if (!aligned16(x) || !aligned16(w_packed) || !aligned16(y)) return GCONV_ERR_ALIGNMENT;
     int rc = ensure_device_state(d);
     if (rc != GCONV_OK) return rc;
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    cudaError_t e;
-    switch (d->variant) {
-        case GCONV_VARIANT_DIRECT_TILED:
-            e = tiled_forward(d->s, d->conv_plan(), x, w_packed, y, d->status_dev, d->sm_count, st);
-            break;
-        case GCONV_VARIANT_IGEMM_TF32: {
-            const IgemmPlan* plan = igemm_plan(d->plans, d->s, 0, d->device, d->sm_count, x, &e);
-            if (plan == nullptr) return fail_cuda(d, e);
-            const size_t need = igemm_plan_scratch(plan);
-            if (need > 0 && (d->workspace == nullptr || d->workspace_bytes < need)) return GCONV_ERR_WORKSPACE;
-            e = igemm_run(plan, x, w_packed, y, d->status_dev, st, need > 0 ? d->workspace : nullptr, launch_opts(d));
-            break;
-        }
-        case GCONV_VARIANT_DIRECT_GENERIC:
-        default:
-            e = generic_forward(d->s, d->conv_plan(), x, w_packed, y, d->status_dev, d->sm_count, generic_tag(d->s), st);
-            break;
-    }
-    return e == cudaSuccess ? GCONV_OK : fail_cuda(d, e);
-}
-
-int gconv_forward_host(gconv_desc_t d, const float* x_host, const void* w_packed, float* y_host, float* x_stage,
-                       float* y_stage, void* stream) {
-    if (d == nullptr || x_host == nullptr || y_host == nullptr || x_stage == nullptr || y_stage == nullptr)
-        return GCONV_ERR_NULL;
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const Shape& s = d->s;
-    const size_t xb = sizeof(float) * (size_t)s.N * s.C_in * s.H * s.W;
-    const size_t yb = sizeof(float) * (size_t)s.N * s.C_out * s.H_out * s.W_out;
-    cudaError_t e = cudaMemcpyAsync(x_stage, x_host, xb, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return fail_cuda(d, e);
-    int rc = gconv_forward(d, x_stage, w_packed, y_stage, stream);
-    if (rc != GCONV_OK) return rc;
-    e = cudaMemcpyAsync(y_host, y_stage, yb, cudaMemcpyDeviceToHost, st);
-    if (e != cudaSuccess) return fail_cuda(d, e);
-    return GCONV_OK;
+    return launch_forward(d, x, w_packed, y, d->status_dev, reinterpret_cast<cudaStream_t>(stream), true);
 }
 
 int gconv_block_supported(gconv_desc_t d, int C2) { return (d != nullptr && igemm_block_supported(d->s, C2)) ? 1 : 0; }

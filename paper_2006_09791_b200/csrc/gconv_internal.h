@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <atomic>
+#include <mutex>
 #include <stddef.h>
 #include <stdint.h>
 
@@ -10,6 +11,7 @@
 namespace gconv {
 struct Status;
 struct IgemmPlan;
+struct HostPipe;
 struct Shape {
     int N, C_in, H, W, C_out, KH, KW, stride, pad, dilation, groups;   // stride, pad, dilation: the row axis (S_h of Algorithm 1)
     int Cg, Kg, H_out, W_out;
@@ -63,6 +65,8 @@ struct gconv_desc {
     // plans of the tensor-core variant, one per (pointwise outputs of a fused block, device): immutable once published, freed
     // with the descriptor (calls of several threads may look them up and add to the list at the same time)
     std::atomic<gconv::IgemmPlan*> plans;
+    std::mutex host_mutex;       // one gconv_forward_host call of this descriptor enqueues at a time
+    gconv::HostPipe* host_pipe;  // how gconv_forward_host cuts the batch (nullptr until the first call that may)
     const gconv::ConvCfg* conv_plan() const { return has_conv ? &conv : nullptr; }
 };
 
@@ -93,6 +97,12 @@ __device__ inline void record_status(Status* st, int code, int detail) {
 }
 
 // ---- per-variant entry points (host side launchers) --------------------------------------------
+// device state and launch of a descriptor's variant (gconv_api.cu); `status` is the block the kernels record errors in
+int ensure_device_state(gconv_desc* d);
+int launch_forward(gconv_desc* d, const float* x, const void* packed, float* y, Status* status, cudaStream_t st, bool may_overlap);
+int fail_cuda(gconv_desc* d, cudaError_t e);
+void free_host_pipe(gconv_desc* d);     // forward_host.cu
+
 size_t generic_packed_bytes(const Shape& s);
 uint32_t generic_tag(const Shape& s);
 cudaError_t generic_pack(const Shape& s, const float* w, void* packed, cudaStream_t st);
@@ -202,6 +212,7 @@ struct IgemmLaunchOpts {
 bool igemm_supported(const Shape& s);
 IgemmCfg igemm_config(const Shape& s, int sm_count);
 size_t igemm_packed_bytes(const Shape& s);
+uint32_t igemm_layout_tag(const Shape& s);    // equal tags: weights packed for one shape serve the other
 cudaError_t igemm_pack(const Shape& s, const float* w, void* packed, cudaStream_t st);
 // fused block: grouped 3x3 (this shape) followed by a pointwise convolution C_out -> C2, one kernel, no intermediate in HBM
 bool igemm_block_supported(const Shape& s, int C2);

@@ -2217,6 +2217,7 @@ static uint32_t igemm_tag(const Shape& s, const IgemmCfg& c) {
     for (int i = 0; i < 10; ++i) h ^= (uint32_t)v[i] + 0x9e3779b9u + (h << 6) + (h >> 2);
     return h;
 }
+uint32_t igemm_layout_tag(const Shape& s) { return igemm_tag(s, igemm_config(s, kLayoutSMs)); }
 static uint32_t block_tag(const Shape& s, const IgemmCfg& c, int C2) { return igemm_tag(s, c) ^ (0xB10C0000u + (uint32_t)C2); }
 
 cudaError_t igemm_block_pack(const Shape& s, int C2, const float* w, const float* w2, void* packed, cudaStream_t st) {
