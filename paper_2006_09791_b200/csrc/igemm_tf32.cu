@@ -518,9 +518,9 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
     const uint32_t b_tile_bytes = (uint32_t)vt * (uint32_t)c.chunks * blk_bytes;   // weights of one (group, filter tile)
     const uint32_t bres_base = smem_base;                                // two resident weight buffers (if b_res)
     const uint32_t stage_base = smem_base + (uint32_t)c.b_res * c.bres_stride;   // b_res = number of resident weight buffers
-    const int HW = s.H * s.W;
+    const int HW = c.flat ? c.flat : s.H * s.W;
     const int rstep = s.W * s.dilation;          // flat-pixel distance between vertical taps
-    const size_t OHW = (size_t)s.H_out * s.W_out;
+    const size_t OHW = c.flat ? (size_t)c.flat : (size_t)s.H_out * s.W_out;
 
     bool run_epilogue = false;
     if (!tag_ok) {
@@ -1263,13 +1263,14 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
                     row = (int)i * c.R + (c.SR == 2 ? (wq >> 1) : wq);
                 }
                 const int col = (h ? s.W - 32 : 0) + lane;
-                valid = row < s.H && col < s.W && (c.SR == 1 || (h == 0 ? col <= 30 : col >= 31));
+                const int seam = s.W == 64 ? 32 : 31;            // (64-wide rows, pointwise only: the segments meet)
+                valid = row < s.H && col < s.W && (c.SR == 1 || (h == 0 ? col < seam : col >= seam));
                 if (c.pair) valid = valid && (int)n < s.N;   // an odd tile count leaves the last pair's second tile empty
                 f = row * s.W + (col < s.W ? col : s.W - 1);
             } else if (c.seg_mode) {
                 c.div_spi.divmod(mt * 4u + (uint32_t)wq, n, i);
                 f = (int)i * c.seg_fstep + lane;
-                valid = (int)n < s.N;
+                valid = (int)n < s.N && (!c.flat || f < c.flat);
             } else {
                 c.div_spi.divmod(mt, n, i);
                 f = (int)i * c.R * s.W + l;
@@ -1566,9 +1567,8 @@ struct IgemmGeom {
 // A pointwise convolution (1x1, pad 0) runs as the 3x3, pad 1 convolution whose only non-zero tap is the centre one
 // (same output size for either stride); the packing kernel writes the zeros.
 // With stride 1 a pointwise layer has no use for rows at all -- every output pixel reads the input pixel at the same flat
-// position -- so the plane is re-cut into rows the tilings like: 32 wide when H*W is a multiple of 128 (segment tiling,
-// every lane used, whole tiles per image); a width TMA cannot address becomes the widest multiple of 4 up to 32 that
-// divides H*W (14x14 becomes 7x28: no padded copy).
+// position -- so a plane of a multiple of 4 pixels is re-cut into rows of 32, the last one short where 32 does not divide it: the
+// segment tiling fills its lanes whatever the width (12x12 planes: 36 of 40 lanes instead of 12 of 32).
 static Shape as_3x3(const Shape& s) {
     Shape t = s;
     // One stride per axis (the paper's S_h, S_w) with a stride of 2 on one axis only: every tiling computes the stride-1 layer
@@ -1581,16 +1581,9 @@ static Shape as_3x3(const Shape& s) {
         t.dilation = 1;
         if (s.stride == 1) {
             const long long hw = (long long)s.H * s.W;
-            int w = 0;
-            if (s.W % 4 == 0) {
-                if (hw % 128 == 0) w = 32;           // whole tiles per image: one box copy per stage
-            } else {
-                for (int cand = 32; cand >= 4 && w == 0; cand -= 4)
-                    if (hw % cand == 0) w = cand;
-            }
-            if (w != 0 && hw / w < (1 << 30)) {
-                t.W = t.W_out = w;
-                t.H = t.H_out = (int)(hw / w);
+            if (hw % 4 == 0 && hw < (1ll << 30)) {
+                t.W = t.W_out = 32;              // (the last row of 32 may be short: IgemmCfg::flat)
+                t.H = t.H_out = (int)((hw + 31) / 32);
             }
         }
     }
@@ -1671,6 +1664,11 @@ bool igemm_supported(const Shape& s_any) {
         if (!((s_any.stride == 1 && s_any.stride_w == 2) || (s_any.stride == 2 && s_any.stride_w == 1))) return false;
     }
     if (s_any.KH == 1 && s_any.KW == 1 && !(s_any.pad == 0 && s_any.dilation == 1)) return false;
+    // (re-cut pointwise planes could take any size; those of fewer than 32 pixels and the wide ones that never ran here keep FP32)
+    const long long hw_any = (long long)s_any.H * s_any.W;
+    if (s_any.KH == 1 && s_any.KW == 1 && s_any.stride == 1 && hw_any % 4 == 0 &&
+        (hw_any < 32 || (s_any.W % 4 == 0 && s_any.W > 128 && hw_any % 128 != 0)))
+        return false;
     const Shape s = as_3x3(s_any);
     if (!(s.KH == 3 && s.KW == 3 && (s.stride == 1 || s.stride == 2) && s.dilation >= 1 && s.pad == s.dilation)) return false;
     if (s.dilation > 1 && (s.stride != 1 || s.dilation > 16)) return false;
@@ -1893,13 +1891,18 @@ static IgemmCfg igemm_config_c2(const Shape& s_any, int sm_count, int C2) {
     c.sub_h = s_any.stride == 2 ? 1 : 0;
     c.sub_w = s_any.stride_w == 2 ? 1 : 0;
     c.pw = (s_any.KH == 1 && s_any.KW == 1 && C2 == 0) ? 1 : 0;
+    c.flat = (s_any.KH == 1 && s_any.KW == 1 && s_any.stride == 1 && (long long)s_any.H * s_any.W % 4 == 0 && (long long)s_any.H * s_any.W < (1ll << 30)) ? s_any.H * s_any.W : 0;
+    // Pointwise with stride 2 on planes the tiled copies address: the tensor map steps two rows at a time, so the odd rows are neither
+    // fetched nor multiplied (the odd columns are: TMA cannot skip elements of the innermost dimension).
+    c.row_skip = (c.pw && c.sub_h && s_true.W % 4 == 0 && s_true.W <= 64) ? 1 : 0;
+    if (c.row_skip) c.sub_h = 0;
     const int vt = c.pw ? 1 : 3;
     const bool fuse = C2 > 0;          // fused grouped + pointwise block: heavy shape, streamed or resident grouped weights
     const IgemmGeom ge = igemm_geom(s_true);
     Shape s = s_true;          // the plane the kernel computes on
-    s.H = ge.Hp;
+    s.H = c.row_skip ? s.H_out : ge.Hp;
     s.W = ge.Wp;
-    c.Hv = s_true.H;
+    c.Hv = c.row_skip ? s.H_out : s_true.H;
     c.Wv = s_true.W;
     c.padded = ge.padded ? 1 : 0;
     c.merge = igemm_merge(s);
@@ -1908,9 +1911,13 @@ static IgemmCfg igemm_config_c2(const Shape& s_any, int sm_count, int C2) {
     c.Kg = s.Kg * c.merge;
     c.CK = (c.Cg % 32 == 0) ? 32 : (c.Cg % 16 == 0 ? 16 : 8);
     c.chunks = c.Cg / c.CK;
-    const int kt_max = c.pw ? 128 : 64;
+    // Pointwise filter tiles of up to 256 (two accumulators fill TMEM) where the input would otherwise cross into shared memory many
+    // times, or the bank has to be streamed anyway: 512 -> 512 @14x14 N = 64 28.4 -> 21.3 us, 512 -> 256 @28x28 48.7 -> 42.1,
+    // 384 -> 192 @32x32 40.6 -> 29.0, 256 -> 512 @56x56 stride 2 86.5 -> 67.0, 128 -> 512 @28x28 35.2 -> 32.0.  128 -> 256 @56x56 loses
+    // (two resident 64 KB banks, one per set of CTAs: 52.8; one of 128 KB: 57.6).
+    const int kt_max = !c.pw ? 64 : ((c.Cg >= 192 || c.Kg >= 512) ? 256 : 128);
     int kt = c.Kg <= kt_max ? c.Kg : kt_max;
-    while (c.Kg % kt != 0 || kt % 8 != 0) kt -= 8;   // largest multiple of 8 dividing Kg, at most 64 (pointwise: 128)
+    while (c.Kg % kt != 0 || kt % 8 != 0) kt -= 8;   // largest multiple of 8 dividing Kg, at most 64 (pointwise: 128 or 256)
     if (c.pw) {
         // small planes: narrower filter tiles until there is a tile per SM (each re-reads its pixels from L2)
         const long long px_tiles = ((long long)s.N * s.H * s.W + 127) / 128;
@@ -1925,7 +1932,7 @@ static IgemmCfg igemm_config_c2(const Shape& s_any, int sm_count, int C2) {
     c.div_boxpx = make_fastdiv(1);
     if (!fuse && (gather_config(c, s_true, sm_count, true) || gather_config(c, s_true, sm_count, false))) return c;
     const int HW = s.H * s.W;
-    c.seg_mode = (32 % s.W == 0) && (HW % 32 == 0);
+    c.seg_mode = !c.row_skip && (32 % s.W == 0) && (HW % 32 == 0);
     c.seg_fstep = 32;
     if (c.seg_mode) {
         c.SPI = HW / 32;
@@ -1955,7 +1962,7 @@ static IgemmCfg igemm_config_c2(const Shape& s_any, int sm_count, int C2) {
     // (no stride-2 row tiles there) is faster flat: 128 -> 256 @9x8 N = 64 g = 8 13.1 against 21.9 us.
     c.rowbox = 0;
     c.SR = 0;
-    if (!c.seg_mode && s.W <= 62 && !(s.stride == 2 && s.W <= 8)) {
+    if (!c.seg_mode && s.W <= (c.pw ? 64 : 62) && !(s.stride == 2 && s.W <= 8 && !c.row_skip)) {
         const int sr = s.W <= 32 ? 1 : 2;
         c.rowbox = 1;
         c.SR = sr;
@@ -2309,10 +2316,11 @@ static cudaError_t make_plan(IgemmPlan& p, const Shape& s_true, int sm_count, co
         p.scratch_bytes = sizeof(float) * p.pad_planes * ge.Hp * ge.Wp;
     }
     p.s = s;
+    if (c.row_skip) p.s.H = s.H_out;             // the plane of even rows
     EncodeTiledFn encode = get_encode_fn();
     if (encode == nullptr || get_replace_fn() == nullptr) return cudaErrorNotSupported;
     CUtensorMap &xmap = p.map, &xmap4 = p.map4;
-    const cuuint64_t HW = (cuuint64_t)s.H * s.W;
+    const cuuint64_t HW = c.flat ? (cuuint64_t)c.flat : (cuuint64_t)s.H * s.W;
     const cuuint64_t dims[3] = {HW, (cuuint64_t)s.C_in, (cuuint64_t)s.N};
     const cuuint64_t strides[2] = {HW * 4, HW * 4 * (cuuint64_t)s.C_in};
     const cuuint32_t box[3] = {32, (cuuint32_t)c.CK, 1};
@@ -2343,8 +2351,8 @@ static cudaError_t make_plan(IgemmPlan& p, const Shape& s_true, int sm_count, co
         }
     } else if (c.rowbox) {
         // (column, channel, row segment, row, image); the segment axis steps (W - 32) columns
-        const cuuint64_t dims5[5] = {(cuuint64_t)s.W, (cuuint64_t)s.C_in, (cuuint64_t)c.SR, (cuuint64_t)s.H, (cuuint64_t)s.N};
-        const cuuint64_t strides5[4] = {HW * 4, c.SR == 2 ? (cuuint64_t)(s.W - 32) * 4 : 128, (cuuint64_t)s.W * 4,
+        const cuuint64_t dims5[5] = {(cuuint64_t)s.W, (cuuint64_t)s.C_in, (cuuint64_t)c.SR, (cuuint64_t)p.s.H, (cuuint64_t)s.N};
+        const cuuint64_t strides5[4] = {HW * 4, c.SR == 2 ? (cuuint64_t)(s.W - 32) * 4 : 128, (cuuint64_t)s.W * 4 * (c.row_skip ? 2 : 1),
                                         HW * 4 * (cuuint64_t)s.C_in};
         const cuuint32_t box5[5] = {32, (cuuint32_t)c.CK, (cuuint32_t)(c.s2h ? 1 : c.SR), (cuuint32_t)(c.s2h ? 9 : (c.pw ? c.R : c.R + 2)), 1};
         const cuuint32_t estr5[5] = {1, 1, 1, 1, 1};
