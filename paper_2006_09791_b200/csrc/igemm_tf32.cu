@@ -1569,6 +1569,12 @@ struct IgemmGeom {
 // With stride 1 a pointwise layer has no use for rows at all -- every output pixel reads the input pixel at the same flat
 // position -- so a plane of a multiple of 4 pixels is re-cut into rows of 32, the last one short where 32 does not divide it: the
 // segment tiling fills its lanes whatever the width (12x12 planes: 36 of 40 lanes instead of 12 of 32).
+// Small planes that 28 divides and 32 does not (14x14, 7x8) and small batches of larger ones (28x28) are cut into rows of 28 instead: one
+// box a stage.  512 -> 512 @14x14 N = 64 21.3 us in rows of 28, 22.2 in segments; 512 -> 256 @28x28 N = 4 14.0 and 17.3, N = 64 42.3 and 33.2.
+static bool pw_rows_of_28(const Shape& s) {
+    const long long hw = (long long)s.H * s.W;
+    return s.KH == 1 && s.KW == 1 && s.stride == 1 && hw % 28 == 0 && hw % 32 != 0 && (hw < 400 || s.N * hw < 128ll * kLayoutSMs);
+}
 static Shape as_3x3(const Shape& s) {
     Shape t = s;
     // One stride per axis (the paper's S_h, S_w) with a stride of 2 on one axis only: every tiling computes the stride-1 layer
@@ -1581,7 +1587,10 @@ static Shape as_3x3(const Shape& s) {
         t.dilation = 1;
         if (s.stride == 1) {
             const long long hw = (long long)s.H * s.W;
-            if (hw % 4 == 0 && hw < (1ll << 30)) {
+            if (pw_rows_of_28(s)) {
+                t.W = t.W_out = 28;
+                t.H = t.H_out = (int)(hw / 28);
+            } else if (hw % 4 == 0 && hw < (1ll << 30)) {
                 t.W = t.W_out = 32;              // (the last row of 32 may be short: IgemmCfg::flat)
                 t.H = t.H_out = (int)((hw + 31) / 32);
             }
@@ -1891,7 +1900,7 @@ static IgemmCfg igemm_config_c2(const Shape& s_any, int sm_count, int C2) {
     c.sub_h = s_any.stride == 2 ? 1 : 0;
     c.sub_w = s_any.stride_w == 2 ? 1 : 0;
     c.pw = (s_any.KH == 1 && s_any.KW == 1 && C2 == 0) ? 1 : 0;
-    c.flat = (s_any.KH == 1 && s_any.KW == 1 && s_any.stride == 1 && (long long)s_any.H * s_any.W % 4 == 0 && (long long)s_any.H * s_any.W < (1ll << 30)) ? s_any.H * s_any.W : 0;
+    c.flat = (!pw_rows_of_28(s_any) && s_any.KH == 1 && s_any.KW == 1 && s_any.stride == 1 && (long long)s_any.H * s_any.W % 4 == 0 && (long long)s_any.H * s_any.W < (1ll << 30)) ? s_any.H * s_any.W : 0;
     // Pointwise with stride 2 on planes the tiled copies address: the tensor map steps two rows at a time, so the odd rows are neither
     // fetched nor multiplied (the odd columns are: TMA cannot skip elements of the innermost dimension).
     c.row_skip = (c.pw && c.sub_h && s_true.W % 4 == 0 && s_true.W <= 64) ? 1 : 0;
@@ -2375,7 +2384,7 @@ static cudaError_t make_plan(IgemmPlan& p, const Shape& s_true, int sm_count, co
             cfg.fast4 = 2;
         else
             xmap4 = xmap;
-    } else if (!c.tapb && c.seg_fstep == 32 && (!c.seg_mode || c.SPI % 4 == 0)) {
+    } else if (!c.tapb && c.seg_fstep == 32 && (!c.seg_mode || c.SPI % 4 == 0 || c.flat)) {   // (flat planes: tiles inside one image)
         const cuuint64_t dims4[4] = {HW, (cuuint64_t)s.C_in, 8, (cuuint64_t)s.N};
         const cuuint64_t strides4[3] = {HW * 4, 128, HW * 4 * (cuuint64_t)s.C_in};
         const cuuint32_t box4[4] = {32, (cuuint32_t)c.CK, (cuuint32_t)c.nseg, 1};
