@@ -56,6 +56,7 @@ __global__ void __launch_bounds__(256, TM * TN > 64 ? 1 : 2)
 direct_conv_kernel(const Shape s, const ConvCfg c, const float* __restrict__ x, const uint32_t* __restrict__ packed,
                    float* __restrict__ y, Status* status, uint32_t tag) {
     extern __shared__ __align__(16) float conv_smem[];
+    dependent_start();
     if (__ldg(packed) != tag) {                           // uniform across the grid
         if (threadIdx.x == 0) record_status(status, GCONV_ERR_PACK_MISMATCH, (int)blockIdx.x);
         return;
@@ -406,34 +407,12 @@ bool conv_config(const Shape& s, int sm_count, ConvCfg& best) {
 
 template <int TM, int TN>
 static cudaError_t launch_conv(const Shape& s, const ConvCfg& c, const float* x, const uint32_t* pk, float* y, Status* status,
-                               uint32_t tag, cudaStream_t st) {
-    auto kernel = direct_conv_kernel<TM, TN>;
-    static bool attr_set[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev >= 64 || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-        if (e != cudaSuccess) return e;
-        if (dev < 64) attr_set[dev] = true;
-    }
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(c.ctas);
-    lc.blockDim = dim3((unsigned)(32 * c.WM * c.WN));
-    lc.dynamicSmemBytes = c.smem;
-    lc.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)c.split;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    lc.attrs = attr;
-    lc.numAttrs = c.split > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&lc, kernel, s, c, x, pk, y, status, tag);
+                               uint32_t tag, const Launch& st) {
+    return launch_kernel<direct_conv_kernel<TM, TN>>(c.ctas, (unsigned)(32 * c.WM * c.WN), c.smem, st, (unsigned)c.split, s, c, x, pk, y, status, tag);
 }
 
 cudaError_t conv_forward(const Shape& s, const ConvCfg& c, const float* x, const void* packed, float* y, Status* status, uint32_t tag,
-                         cudaStream_t st) {
+                         const Launch& st) {
     const uint32_t* pk = reinterpret_cast<const uint32_t*>(packed);
 #define GCONV_CONV_CASE(M, T) \
     if (c.TM == M && c.TN == T) return launch_conv<M, T>(s, c, x, pk, y, status, tag, st);

@@ -68,6 +68,7 @@ template <int VEC, int UB>
 __global__ void __launch_bounds__(256, VEC == 0 ? 2 : (UB == 4 ? 3 : 4))
 dw_stream_s1_kernel(const Shape s, const DwCfg c, const float* __restrict__ x, const uint32_t* __restrict__ packed,
                     float* __restrict__ y, Status* status, uint32_t tag) {
+    dependent_start();
     const uint32_t tag_seen = __ldg(packed);
     const float* __restrict__ wpk = reinterpret_cast<const float*>(packed + kHeaderBytes / 4);
     const int lane = threadIdx.x & 31;
@@ -145,6 +146,7 @@ template <int VEC>
 __global__ void __launch_bounds__(256)
 dw_stream_s2_kernel(const Shape s, const DwCfg c, const float* __restrict__ x, const uint32_t* __restrict__ packed,
                     float* __restrict__ y, Status* status, uint32_t tag) {
+    dependent_start();
     const uint32_t tag_seen = __ldg(packed);
     const float* __restrict__ wpk = reinterpret_cast<const float*>(packed + kHeaderBytes / 4);
     const int lane = threadIdx.x & 31;
@@ -246,6 +248,7 @@ template <int VEC, int STRIDE>
 __global__ void __launch_bounds__(256)
 dw5_stream_kernel(const Shape s, const DwCfg c, const float* __restrict__ x, const uint32_t* __restrict__ packed,
                   float* __restrict__ y, Status* status, uint32_t tag) {
+    dependent_start();
     const uint32_t tag_seen = __ldg(packed);
     const float* __restrict__ wpk = reinterpret_cast<const float*>(packed + kHeaderBytes / 4);
     const int lane = threadIdx.x & 31;
@@ -320,6 +323,7 @@ template <int VEC>
 __global__ void __launch_bounds__(256, 2)
 dw5_stream_s1_kernel(const Shape s, const DwCfg c, const float* __restrict__ x, const uint32_t* __restrict__ packed,
                      float* __restrict__ y, Status* status, uint32_t tag) {
+    dependent_start();
     const uint32_t tag_seen = __ldg(packed);
     const float* __restrict__ wpk = reinterpret_cast<const float*>(packed + kHeaderBytes / 4);
     const int lane = threadIdx.x & 31;
@@ -437,26 +441,27 @@ DwCfg dw_config(const Shape& s, int sm_count) {
 }
 
 cudaError_t dw_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, int sm_count,
-                       cudaStream_t st) {
+                       const Launch& st) {
     // small planes go through shared memory in batches of whole planes (direct_dw_plane.cu); 3x3 stride 1 on 28x28 planes
     // measured the same on both kernels (16.5 us on 192 planes, N = 64) and stays on the stream
     if (dw_plane_supported(s) && !(s.KH == 3 && s.stride == 1 && s.W == 28)) return dw_plane_forward(s, x, packed, y, status, sm_count, st);
     const DwCfg c = dw_config(s, sm_count);
     const uint32_t tag = pack_tag(s, GCONV_VARIANT_DIRECT_TILED);
     const uint32_t* pk = reinterpret_cast<const uint32_t*>(packed);
+    cudaError_t e;
     const int vec = s.W % 4 == 0 ? 4 : (s.W % 2 == 0 ? 2 : 0);
 #define GCONV_DW_LAUNCH(KERNEL) \
     do { \
         if (vec == 4) KERNEL(4); else if (vec == 2) KERNEL(2); else KERNEL(0); \
     } while (0)
-#define GCONV_DW5_S1(V) dw5_stream_s1_kernel<V><<<c.blocks, 256, 0, st>>>(s, c, x, pk, y, status, tag)
-#define GCONV_DW5_S2(V) dw5_stream_kernel<V, 2><<<c.blocks, 256, 0, st>>>(s, c, x, pk, y, status, tag)
+#define GCONV_DW5_S1(V) e = launch_kernel<dw5_stream_s1_kernel<V>>(c.blocks, 256, 0, st, 1, s, c, x, pk, y, status, tag)
+#define GCONV_DW5_S2(V) e = launch_kernel<dw5_stream_kernel<V, 2>>(c.blocks, 256, 0, st, 1, s, c, x, pk, y, status, tag)
 #define GCONV_DW3_S1(V) \
     do { \
-        if (s.H_out >= 28) dw_stream_s1_kernel<V, 4><<<c.blocks, 256, 0, st>>>(s, c, x, pk, y, status, tag); \
-        else dw_stream_s1_kernel<V, 2><<<c.blocks, 256, 0, st>>>(s, c, x, pk, y, status, tag); \
+        if (s.H_out >= 28) e = launch_kernel<dw_stream_s1_kernel<V, 4>>(c.blocks, 256, 0, st, 1, s, c, x, pk, y, status, tag); \
+        else e = launch_kernel<dw_stream_s1_kernel<V, 2>>(c.blocks, 256, 0, st, 1, s, c, x, pk, y, status, tag); \
     } while (0)
-#define GCONV_DW3_S2(V) dw_stream_s2_kernel<V><<<c.blocks, 256, 0, st>>>(s, c, x, pk, y, status, tag)
+#define GCONV_DW3_S2(V) e = launch_kernel<dw_stream_s2_kernel<V>>(c.blocks, 256, 0, st, 1, s, c, x, pk, y, status, tag)
     if (s.KH == 5) {
         if (s.stride == 1) GCONV_DW_LAUNCH(GCONV_DW5_S1);
         else GCONV_DW_LAUNCH(GCONV_DW5_S2);
@@ -470,7 +475,7 @@ cudaError_t dw_forward(const Shape& s, const float* x, const void* packed, float
 #undef GCONV_DW5_S2
 #undef GCONV_DW3_S1
 #undef GCONV_DW3_S2
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace gconv

@@ -99,6 +99,7 @@ dw_plane_kernel(const Shape s, const DwPlaneCfg c, const float* __restrict__ x, 
     __shared__ __align__(8) unsigned long long full[2];
     __shared__ int failed;
     const int tid = threadIdx.x;
+    dependent_start();
     if (__ldg(packed) != tag) {                          // uniform across the grid
         if (tid == 0) record_status(status, GCONV_ERR_PACK_MISMATCH, (int)blockIdx.x);
         return;
@@ -256,19 +257,8 @@ dw_plane_kernel(const Shape s, const DwPlaneCfg c, const float* __restrict__ x, 
 
 template <int K, int S, int W, bool WHOLE = false>
 cudaError_t launch_plane(const Shape& s, const DwPlaneCfg& c, const float* x, const uint32_t* pk, float* y, Status* status,
-                         uint32_t tag, cudaStream_t st) {
-    auto kernel = dw_plane_kernel<K, S, W, WHOLE>;
-    static bool attr_set[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 64 && !attr_set[dev]) {
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
-        if (e != cudaSuccess) return e;
-        attr_set[dev] = true;
-    }
-    kernel<<<c.grid, c.threads, c.smem_bytes, st>>>(s, c, x, pk, y, status, tag);
-    return cudaGetLastError();
+                         uint32_t tag, const Launch& st) {
+    return launch_kernel<dw_plane_kernel<K, S, W, WHOLE>>(c.grid, c.threads, c.smem_bytes, st, 1, s, c, x, pk, y, status, tag);
 }
 
 }  // namespace
@@ -334,7 +324,7 @@ DwPlaneCfg dw_plane_config(const Shape& s, int sm_count) {
 }
 
 cudaError_t dw_plane_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, int sm_count,
-                             cudaStream_t st) {
+                             const Launch& st) {
     const DwPlaneCfg c = dw_plane_config(s, sm_count);
     const uint32_t tag = pack_tag(s, GCONV_VARIANT_DIRECT_TILED);
     const uint32_t* pk = reinterpret_cast<const uint32_t*>(packed);

@@ -21,6 +21,7 @@ uint32_t generic_tag(const Shape& s) { return pack_tag(s, GCONV_VARIANT_DIRECT_G
 __global__ void __launch_bounds__(256)
 generic_forward_kernel(Shape s, const float* __restrict__ x, const uint32_t* __restrict__ packed,
                        float* __restrict__ y, Status* status, uint32_t tag) {
+    dependent_start();
     if (packed[0] != tag) {
         if (threadIdx.x == 0) record_status(status, GCONV_ERR_PACK_MISMATCH, (int)blockIdx.x);
         return;
@@ -54,14 +55,13 @@ generic_forward_kernel(Shape s, const float* __restrict__ x, const uint32_t* __r
 }
 
 cudaError_t generic_forward(const Shape& s, const ConvCfg* conv, const float* x, const void* packed, float* y, Status* status,
-                            int sm_count, uint32_t tag, cudaStream_t st) {
+                            int sm_count, uint32_t tag, const Launch& st) {
     if (conv != nullptr) return conv_forward(s, *conv, x, packed, y, status, tag, st);
     const size_t total = (size_t)s.N * s.C_out * s.H_out * s.W_out;
     size_t want = (total + 255) / 256;
     size_t cap = (size_t)sm_count * 8 * 4;
     int blocks = (int)(want < cap ? want : cap);
-    generic_forward_kernel<<<blocks, 256, 0, st>>>(s, x, reinterpret_cast<const uint32_t*>(packed), y, status, tag);
-    return cudaGetLastError();
+    return launch_kernel<generic_forward_kernel>((unsigned)blocks, 256, 0, st, 1, s, x, reinterpret_cast<const uint32_t*>(packed), y, status, tag);
 }
 
 }  // namespace gconv

@@ -74,6 +74,7 @@ direct_rows_kernel(const Shape s, const RowsCfg c, const float* __restrict__ x, 
                    float* __restrict__ y, Status* status, uint32_t tag) {
     // The header tag is loaded now but only examined right before the stores, so the check costs no
     // memory round trip ahead of the input loads; a mismatch still leaves y untouched.
+    dependent_start();
     const uint32_t tag_seen = __ldg(packed);
     const float* __restrict__ wpk = reinterpret_cast<const float*>(packed + kHeaderBytes / 4);
     const uint32_t item = blockIdx.x * blockDim.x + threadIdx.x;
@@ -166,14 +167,12 @@ direct_rows_kernel(const Shape s, const RowsCfg c, const float* __restrict__ x, 
 
 template <int S, int KT, int PR>
 cudaError_t launch_rows(const Shape& s, const RowsCfg& c, const float* x, const void* packed, float* y, Status* status,
-                        cudaStream_t st) {
+                        const Launch& st) {
     const unsigned blocks = (c.items + 127) / 128;
     const uint32_t tag = pack_tag(s, GCONV_VARIANT_DIRECT_TILED);
-    if (c.vec)
-        direct_rows_kernel<S, KT, PR, true><<<blocks, 128, 0, st>>>(s, c, x, reinterpret_cast<const uint32_t*>(packed), y, status, tag);
-    else
-        direct_rows_kernel<S, KT, PR, false><<<blocks, 128, 0, st>>>(s, c, x, reinterpret_cast<const uint32_t*>(packed), y, status, tag);
-    return cudaGetLastError();
+    const uint32_t* pk = reinterpret_cast<const uint32_t*>(packed);
+    return c.vec ? launch_kernel<direct_rows_kernel<S, KT, PR, true>>(blocks, 128, 0, st, 1, s, c, x, pk, y, status, tag)
+                 : launch_kernel<direct_rows_kernel<S, KT, PR, false>>(blocks, 128, 0, st, 1, s, c, x, pk, y, status, tag);
 }
 
 }  // namespace
@@ -221,7 +220,7 @@ RowsCfg rows_config(const Shape& s) {
     return c;
 }
 
-cudaError_t rows_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, cudaStream_t st) {
+cudaError_t rows_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, const Launch& st) {
     const RowsCfg c = rows_config(s);
 #define GCONV_ROWS_CASE(S, K, P) \
     if (s.stride == S && s.Kg == K && c.PR == P) return launch_rows<S, K, P>(s, c, x, packed, y, status, st);

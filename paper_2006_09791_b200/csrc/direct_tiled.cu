@@ -53,7 +53,7 @@ cudaError_t tiled_pack(const Shape& s, const float* w, void* packed, cudaStream_
 }
 
 cudaError_t tiled_forward(const Shape& s, const ConvCfg* conv, const float* x, const void* packed, float* y, Status* status, int sm_count,
-                          cudaStream_t st) {
+                          const Launch& st) {
     if (dw_supported(s)) return dw_forward(s, x, packed, y, status, sm_count, st);
     if (rows_supported(s)) return rows_forward(s, x, packed, y, status, st);
     return generic_forward(s, conv, x, packed, y, status, sm_count, pack_tag(s, GCONV_VARIANT_DIRECT_TILED), st);

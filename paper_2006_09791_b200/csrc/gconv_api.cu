@@ -86,13 +86,24 @@ int ensure_device_state(gconv_desc* d) {
     return GCONV_OK;
 }
 
-// Enqueues the kernels of the descriptor's variant.  `may_overlap`: the set-up of a tensor-core kernel may overlap the previous
-// kernel's tail (not where a copy or an event precedes it).
+// FP32 kernels overlap their start-up with the previous kernel's tail while they are short.  A block that starts early finds the SM's
+// shared memory / L1 split as the previous kernel left it, and keeps it: on long kernels the smaller L1 (fewer loads in flight) or
+// the fewer resident blocks cost more than the launch gap.  Depthwise networks, all layers up to x MB of x + y overlapped: N = 2 @143
+// 95 us (none), 74 (2 MB and up); N = 35 @128 127 (none), 118 (4), 108 (24), 113 (40); N = 20 @224 252 (none), 245 (24), 236 (40);
+// N = 64 @224 438 (none), 434 (40), 500 (all).  Other filters, N = 1 @160 49 (none), 46 (2); N = 16 @224 244 (none and 2), 276 (8).
+static bool fp32_overlaps(const Shape& s) {
+    const double bytes = 4.0 * s.N * ((double)s.C_in * s.H * s.W + (double)s.C_out * s.H_out * s.W_out);
+    return bytes <= (dw_supported(s) ? 40e6 : 2e6);
+}
+
+// Enqueues the kernels of the descriptor's variant.  `may_overlap`: a kernel's start-up may overlap the previous kernel's
+// tail (not where a copy or an event precedes it).
 int launch_forward(gconv_desc* d, const float* x, const void* packed, float* y, Status* status, cudaStream_t st, bool may_overlap) {
     cudaError_t e = cudaSuccess;
+    const Launch to = {st, may_overlap && fp32_overlaps(d->s)};
     switch (d->variant) {
         case GCONV_VARIANT_DIRECT_TILED:
-            e = tiled_forward(d->s, d->conv_plan(), x, packed, y, status, d->sm_count, st);
+            e = tiled_forward(d->s, d->conv_plan(), x, packed, y, status, d->sm_count, to);
             break;
         case GCONV_VARIANT_IGEMM_TF32: {
             const IgemmPlan* plan = igemm_plan(d->plans, d->s, 0, d->device, d->sm_count, x, &e);
@@ -106,7 +117,7 @@ int launch_forward(gconv_desc* d, const float* x, const void* packed, float* y, 
         }
         case GCONV_VARIANT_DIRECT_GENERIC:
         default:
-            e = generic_forward(d->s, d->conv_plan(), x, packed, y, status, d->sm_count, generic_tag(d->s), st);
+            e = generic_forward(d->s, d->conv_plan(), x, packed, y, status, d->sm_count, generic_tag(d->s), to);
             break;
     }
     return e == cudaSuccess ? GCONV_OK : fail_cuda(d, e);

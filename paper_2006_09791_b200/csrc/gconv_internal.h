@@ -96,6 +96,46 @@ __device__ inline void record_status(Status* st, int code, int detail) {
     if (atomicCAS(&st->code, 0, code) == 0) st->detail = detail;
 }
 
+// Where and how a forward kernel is launched: `overlap` lets its start-up run beside the previous kernel's tail (programmatic
+// dependent launch; the kernel waits for that kernel to complete before it touches x, y or the packed weights).
+struct Launch {
+    cudaStream_t st;
+    bool overlap;
+};
+#ifdef __CUDACC__
+// First thing in a kernel launched this way: the next kernel may start its own set-up; wait for the previous one.
+__device__ __forceinline__ void dependent_start() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <auto Kernel, typename... A>
+inline cudaError_t launch_kernel(unsigned grid, unsigned block, size_t smem, const Launch& to, unsigned cluster, A... args) {
+    static bool attr_set[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64 || !attr_set[dev]) {
+        if (smem > 0) e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) attr_set[dev] = true;          // (a kernel either always or never takes dynamic shared memory)
+    }
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(grid);
+    lc.blockDim = dim3(block);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = to.st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = to.overlap ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    lc.attrs = attr;
+    lc.numAttrs = cluster > 1 ? 2 : (to.overlap ? 1 : 0);
+    return cudaLaunchKernelEx(&lc, Kernel, args...);
+}
+#endif
+
 // ---- per-variant entry points (host side launchers) --------------------------------------------
 // device state and launch of a descriptor's variant (gconv_api.cu); `status` is the block the kernels record errors in
 int ensure_device_state(gconv_desc* d);
@@ -107,11 +147,11 @@ size_t generic_packed_bytes(const Shape& s);
 uint32_t generic_tag(const Shape& s);
 cudaError_t generic_pack(const Shape& s, const float* w, void* packed, cudaStream_t st);
 cudaError_t generic_forward(const Shape& s, const ConvCfg* conv, const float* x, const void* packed, float* y, Status* status,
-                            int sm_count, uint32_t tag, cudaStream_t st);
+                            int sm_count, uint32_t tag, const Launch& st);
 
 bool conv_config(const Shape& s, int sm_count, ConvCfg& c);   // false: no tile fits (huge filters or dilations)
 cudaError_t conv_forward(const Shape& s, const ConvCfg& c, const float* x, const void* packed, float* y, Status* status, uint32_t tag,
-                         cudaStream_t st);
+                         const Launch& st);
 
 // DIRECT_TILED, narrow groups (Kg in {1,2,4,8}): one thread per (image, group, row strip, 4-pixel chunk).
 struct RowsCfg {
@@ -121,7 +161,7 @@ struct RowsCfg {
 };
 bool rows_supported(const Shape& s);
 RowsCfg rows_config(const Shape& s);
-cudaError_t rows_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, cudaStream_t st);
+cudaError_t rows_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, const Launch& st);
 
 // DIRECT_TILED, depthwise stream kernel: a warp holds `subs` row strips of XQ lanes each.
 struct DwCfg {
@@ -138,11 +178,11 @@ struct DwPlaneCfg {
 bool dw_plane_supported(const Shape& s);
 DwPlaneCfg dw_plane_config(const Shape& s, int sm_count);
 cudaError_t dw_plane_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, int sm_count,
-                             cudaStream_t st);
+                             const Launch& st);
 bool dw_supported(const Shape& s);
 DwCfg dw_config(const Shape& s, int sm_count);
 cudaError_t dw_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, int sm_count,
-                       cudaStream_t st);
+                       const Launch& st);
 
 // DIRECT_TILED
 bool tiled_supported(const Shape& s);
@@ -151,7 +191,7 @@ size_t tiled_packed_bytes(const Shape& s);
 cudaError_t group_pack(const Shape& s, const float* w, void* packed, uint32_t tag, cudaStream_t st);
 cudaError_t tiled_pack(const Shape& s, const float* w, void* packed, cudaStream_t st);
 cudaError_t tiled_forward(const Shape& s, const ConvCfg* conv, const float* x, const void* packed, float* y, Status* status, int sm_count,
-                          cudaStream_t st);
+                          const Launch& st);
 
 // IGEMM_TF32: tile geometry of the tcgen05 implicit-GEMM kernel.
 struct IgemmCfg {
