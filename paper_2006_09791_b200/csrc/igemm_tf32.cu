@@ -404,14 +404,13 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
     __shared__ SharedCtl ctl;
     static_assert(sizeof(SharedCtl) <= 1024, "control block must leave 226 KB of dynamic shared memory");
 
-    // Programmatic dependent launch: let the next kernel in the stream be scheduled as SMs free up, and run this
-    // kernel's own set-up (barriers, TMEM) while the previous kernel drains.  Before griddepcontrol.wait has
+    // Programmatic dependent launch: this kernel's blocks may start while the previous kernel drains, and run their
+    // own set-up (barriers, TMEM) meanwhile; they let the next kernel start once their last input copy is issued (see the producer).  Before griddepcontrol.wait has
     // returned (the previous kernel's writes complete and visible) the only global memory read is the packed weights
     // (their tag here, the first resident bank in the producer).  Only the dependency wait guarantees that an earlier
     // kernel's writes are visible, so the host launches the first forward after ANY weight packing of the process
     // without programmatic serialization (a full stream dependency); by every later launch the weights are older than
     // a completed kernel boundary.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const uint32_t tag_seen = __ldg(packed);
     const uint8_t* __restrict__ wblocks = reinterpret_cast<const uint8_t*>(packed) + kHeaderBytes;
 
@@ -788,6 +787,11 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
             run_epilogue = true;
         } else {
             for (int tile = tile_first; tile < tile_end && ok; tile = tile_next(tile)) visit(tile, false, 0u, it, stage, ph);
+            // The next kernel may start now: its set-up and L2 prefetch run beside this block's last tile.  (Released at kernel start,
+            // as it used to be, its blocks sat beside this kernel's whole work and competed with it: stack of 18 layers at N = 16 69.5
+            // against 58.0 us, ResNet-shaped g = 8 at N = 4 43.7 against 37.2, ResNeXt-shaped N = 64 225 against 222; released at the
+            // first finished accumulator 57.4, 38.8, 223; never 68.8, 44.7, 227.)
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         }
         if (producer && !ok && lane == 0) {
             // drain: wait (bounded) for the copies of every stage that may still be in flight, so that no bulk copy
