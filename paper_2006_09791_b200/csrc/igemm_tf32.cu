@@ -1614,46 +1614,59 @@ static IgemmGeom igemm_geom(const Shape& s) {
 }
 
 namespace {
-// Zero-padded copy of x for widths TMA cannot address: every plane becomes Hp x Wp (Wp a multiple of 4), one thread
-// per group of four output columns.  IDX is the index type: 32-bit whenever the padded tensor has fewer than 2^32
-// column groups (the common case: the divisions are then cheap multiply-shift ones).
-template <typename IDX>
-__global__ void igemm_pad_kernel(const float* __restrict__ x, float* __restrict__ xp, size_t planes, int H, int W, int Hp, int Wp,
-                                 FastDiv div_plane, FastDiv div_row) {
-    // the convolution kernel that follows may be scheduled now: its set-up overlaps this copy, and it reads the padded
-    // planes only after its own griddepcontrol.wait (this grid complete and visible)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+// Zero-padded copy of x for widths TMA cannot address: every plane becomes Hp x Wp (Wp a multiple of 4).  A stream: a thread moves
+// kPadItems groups of four output columns, a grid stride apart, all of their loads in flight before the first store (one group at
+// a time left the memory system idle for a latency per group): 64 -> 64 @45x45 N = 1 7.0 -> 5.9 us for the layer, 128 -> 128 @25x25 N = 64
+// g = 4 32.0 -> 30.4, 128 -> 128 @57x57 N = 64 g = 32 79.3 -> 78.0.  IDX is the index type: 32-bit whenever the padded tensor has fewer
+// than 2^31 column groups (the common case: the divisions are then cheap multiply-shift ones).
+constexpr int kPadItems = 4;
+template <typename IDX, bool EVEN>
+__global__ void __launch_bounds__(256) igemm_pad_kernel(const float* __restrict__ x, float* __restrict__ xp, size_t planes, int H, int W, int Hp, int Wp,
+                                                        FastDiv div_plane, FastDiv div_row) {
+    // (the convolution kernel that follows reads the padded planes only after its own griddepcontrol.wait: this grid complete and visible)
+    dependent_start();
     const size_t per_plane = (size_t)Hp * (Wp / 4);
-    const size_t total = planes * per_plane;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        size_t plane;
-        int h, w4;
-        if constexpr (sizeof(IDX) == 4) {
-            uint32_t pl, rem, hh, q;
-            div_plane.divmod((uint32_t)i, pl, rem);
-            div_row.divmod(rem, hh, q);
-            plane = pl;
-            h = (int)hh;
-            w4 = (int)q * 4;
-        } else {
-            plane = i / per_plane;
-            const int rem = (int)(i - plane * per_plane);
-            h = rem / (Wp / 4);
-            w4 = (rem - h * (Wp / 4)) * 4;
-        }
-        float v[4] = {0.f, 0.f, 0.f, 0.f};
-        if (h < H) {
-            const float* src = x + (plane * H + h) * (size_t)W;
-            if ((W & 1) == 0) {                    // even width: rows start on 8-byte boundaries
-                if (w4 < W) { const float2 a = __ldg(reinterpret_cast<const float2*>(src + w4)); v[0] = a.x; v[1] = a.y; }
-                if (w4 + 2 < W) { const float2 b = __ldg(reinterpret_cast<const float2*>(src + w4 + 2)); v[2] = b.x; v[3] = b.y; }
+    const size_t total = planes * per_plane, step = (size_t)gridDim.x * blockDim.x;
+    for (size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < total; i0 += kPadItems * step) {
+        float v[kPadItems][4];
+        float* dst[kPadItems];
+#pragma unroll
+        for (int k = 0; k < kPadItems; ++k) {
+            const size_t i = i0 + k * step;
+            dst[k] = nullptr;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[k][j] = 0.f;
+            if (i >= total) continue;
+            size_t plane;
+            int h, w4;
+            if constexpr (sizeof(IDX) == 4) {
+                uint32_t pl, rem, hh, q;
+                div_plane.divmod((uint32_t)i, pl, rem);
+                div_row.divmod(rem, hh, q);
+                plane = pl;
+                h = (int)hh;
+                w4 = (int)q * 4;
+            } else {
+                plane = i / per_plane;
+                const int rem = (int)(i - plane * per_plane);
+                h = rem / (Wp / 4);
+                w4 = (rem - h * (Wp / 4)) * 4;
+            }
+            dst[k] = xp + (plane * Hp + h) * (size_t)Wp + w4;
+            if (h >= H) continue;
+            const float* src = x + (plane * H + h) * (size_t)W + w4;
+            if constexpr (EVEN) {                  // rows start on 8-byte boundaries
+                if (w4 < W) { const float2 a = __ldg(reinterpret_cast<const float2*>(src)); v[k][0] = a.x; v[k][1] = a.y; }
+                if (w4 + 2 < W) { const float2 b = __ldg(reinterpret_cast<const float2*>(src + 2)); v[k][2] = b.x; v[k][3] = b.y; }
             } else {
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    if (w4 + j < W) v[j] = __ldg(src + w4 + j);
+                    if (w4 + j < W) v[k][j] = __ldg(src + j);
             }
         }
-        *reinterpret_cast<float4*>(xp + (plane * Hp + h) * (size_t)Wp + w4) = make_float4(v[0], v[1], v[2], v[3]);
+#pragma unroll
+        for (int k = 0; k < kPadItems; ++k)
+            if (dst[k] != nullptr) *reinterpret_cast<float4*>(dst[k]) = make_float4(v[k][0], v[k][1], v[k][2], v[k][3]);
     }
 }
 }  // namespace
@@ -2321,7 +2334,8 @@ static cudaError_t make_plan(IgemmPlan& p, const Shape& s_true, int sm_count, co
         p.pad_W = s.W;
         p.pad_planes = (size_t)s.N * s.C_in;
         p.pad_total = p.pad_planes * ge.Hp * (ge.Wp / 4);
-        p.pad_blocks = (int)((p.pad_total + 255) / 256 < (size_t)sm_count * 16 ? (p.pad_total + 255) / 256 : (size_t)sm_count * 16);
+        const size_t blocks = (p.pad_total + 256 * kPadItems - 1) / (256 * kPadItems), most = (size_t)sm_count * 16;
+        p.pad_blocks = (int)(blocks < most ? blocks : most);
         p.pad_div_plane = make_fastdiv((uint32_t)(ge.Hp * (ge.Wp / 4)));
         p.pad_div_row = make_fastdiv((uint32_t)(ge.Wp / 4));
         s.H = ge.Hp;
@@ -2443,6 +2457,13 @@ void igemm_free_plans(std::atomic<IgemmPlan*>& plans) {
 
 size_t igemm_plan_scratch(const IgemmPlan* p) { return p->scratch_bytes; }
 
+namespace {
+template <auto K>
+struct Kernel {
+    static constexpr auto value = K;
+};
+}  // namespace
+
 // A call takes its plan (a call used to work the configuration out twice and encode both tensor maps, 1 us of host time) and
 // puts its own input address into copies of the maps.
 cudaError_t igemm_run(const IgemmPlan* plan, const float* x, const void* packed, float* y, Status* status, cudaStream_t st, float* scratch,
@@ -2453,11 +2474,16 @@ cudaError_t igemm_run(const IgemmPlan* plan, const float* x, const void* packed,
     cfg.dbg_skip = opts.dbg_skip;
     if (p.scratch_bytes > 0) {
         if (scratch == nullptr) return cudaErrorInvalidValue;
-        if (p.pad_total < (1ull << 32))
-            igemm_pad_kernel<uint32_t><<<p.pad_blocks, 256, 0, st>>>(x, scratch, p.pad_planes, p.pad_H, p.pad_W, p.s.H, p.s.W, p.pad_div_plane, p.pad_div_row);
-        else
-            igemm_pad_kernel<uint64_t><<<p.pad_blocks, 256, 0, st>>>(x, scratch, p.pad_planes, p.pad_H, p.pad_W, p.s.H, p.s.W, p.pad_div_plane, p.pad_div_row);
-        cudaError_t e = cudaGetLastError();
+        // (the copy itself may start beside the previous kernel's tail while it is short; see the FP32 kernels)
+        const Launch to = {st, opts.pdl && p.pad_total * 16 <= 20000000};
+        const unsigned grid = (unsigned)p.pad_blocks;
+        auto copy = [&](auto kernel_tag) {
+            return launch_kernel<decltype(kernel_tag)::value>(grid, 256, 0, to, 1, x, scratch, p.pad_planes, p.pad_H, p.pad_W, p.s.H, p.s.W,
+                                                              p.pad_div_plane, p.pad_div_row);
+        };
+        const bool small = p.pad_total < (1ull << 31), even = (p.pad_W & 1) == 0;
+        const cudaError_t e = small ? (even ? copy(Kernel<igemm_pad_kernel<uint32_t, true>>()) : copy(Kernel<igemm_pad_kernel<uint32_t, false>>()))
+                                    : (even ? copy(Kernel<igemm_pad_kernel<uint64_t, true>>()) : copy(Kernel<igemm_pad_kernel<uint64_t, false>>()));
         if (e != cudaSuccess) return e;
         x = scratch;
     }
