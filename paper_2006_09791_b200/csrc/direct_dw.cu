@@ -14,8 +14,6 @@ namespace gconv {
 
 namespace {
 
-constexpr int U = 4;   // output rows per pipeline block (strip lengths are multiples of it)
-
 // Four consecutive pixels of row h starting at column col (zero outside the image).  VEC = 4: W % 4 == 0, so the
 // address is 16-byte aligned and the four pixels are in range; VEC = 2: W is even, two 8-byte loads (the second pair
 // may be past the row); VEC = 0: four bounds-checked scalar loads.
@@ -415,22 +413,34 @@ DwCfg dw_config(const Shape& s, int sm_count) {
     DwCfg c;
     c.XQ = s.stride == 1 ? (s.W + 3) / 4 : (s.W + 7) / 8;
     c.subs = 32 / c.XQ;
-    // rows per thread: long strips amortise the two halo rows, short ones give more parallelism; aim for
-    // at least ~6 waves of 1024 threads per SM.  5x5: four halo rows per strip and 25 FMAs per output make the strip
-    // length matter more than the thread count (measured): split only below ~0.4 waves.
+    // Output rows per thread.  A strip pays for its first rows (`start`, in rows: the halo rows and the first loads' latency),
+    // and blocks that start together end together, so what counts is how many strips follow one another on an SM: waves x
+    // (rows + start), where a last, partly filled wave costs half of one plus its share.  Strips end at whole pipeline blocks
+    // (`unit` rows).  On 159 drawn layers (N 1 ... 128, planes of 4 ... 128 rows, both filters, strides and every alignment),
+    // each timed at up to 14 strip lengths, the choice is 1 % slower than the best on average (19 % at most); the earlier rule
+    // (28 rows, or halved until a wave or six were filled) was 15 and 37 % (3x3 stride 1, tall and short planes), 67 % (3x3
+    // stride 2), 21 and 77 % (5x5) slower than the best.  64 x 96 planes of 56x56, 5x5 stride 2: 33.7 us at 28 rows, 25.4 us at 10.
+    const bool tall = s.KH == 3 && s.stride == 1 && s.H_out >= 28;
+    const int vec = s.W % 4 == 0 ? 4 : (s.W % 2 == 0 ? 2 : 0);
+    const int unit = s.stride == 2 ? 1 : (s.KH == 5 ? U5 : (tall ? 4 : 2));
+    const double start = s.stride == 1 && (s.KH == 5 || tall) ? 3.0 : 0.5;
+    const int per_sm = s.KH == 5 ? 2 : (tall ? (vec ? 3 : 2) : (vec ? 4 : 3));   // blocks an SM holds (registers)
+    const double slots = (double)sm_count * per_sm;
     const long long planes = (long long)s.N * s.C_in;
-    const long long want = s.KH == 5 ? 410LL * sm_count : 6LL * 1024 * sm_count;
-    int rh = s.H_out;
-    if (s.KH == 3 && s.stride == 1 && s.H_out >= 28) {
-        // 3x3 stride 1 on planes of 28 rows and more: strips of 28 rows measured best at 28x28, 56x56 and 112x112
-        // (7 % halo rows, long enough to amortise the set-up) as long as about half a wave of lanes remains
-        rh = 28;
-        while (rh > 8 && planes * ((s.H_out + rh - 1) / rh) * c.XQ < 512LL * sm_count) rh = (rh + 1) / 2;
-    } else {
-        while (rh > 8 && planes * ((s.H_out + rh - 1) / rh) * c.XQ < want) rh = (rh + 1) / 2;
-        if (s.KH == 3 && s.stride == 1 && s.H_out <= 8 && planes * c.XQ * 2 >= 512LL * sm_count) rh = 4;   // 7x7, 8x8: two short strips
+    int rh = 0;
+    double best = 0.0;
+    for (int r = (s.H_out + unit - 1) / unit * unit;;) {
+        const int chunks = (s.H_out + r - 1) / r;
+        const double blocks = ceil(ceil((double)planes * chunks / c.subs) / 8.0), waves = blocks / slots, whole = floor(waves);
+        const double cost = (waves <= 1.0 ? 1.0 : whole + (waves > whole ? 0.5 + 0.5 * (waves - whole) : 0.0)) * (r + start);
+        if (rh == 0 || cost < best) {
+            best = cost;
+            rh = r;
+        }
+        if (r == unit) break;
+        const int more = (s.H_out + r - unit - 1) / (r - unit);               // the next count of strips that shortens them
+        r = ((s.H_out + more - 1) / more + unit - 1) / unit * unit;
     }
-    rh = ((rh + U - 1) / U) * U;
     c.RH = rh;
     c.chunks = (s.H_out + rh - 1) / rh;
     c.div_chunks = make_fastdiv((uint32_t)c.chunks);
@@ -440,12 +450,20 @@ DwCfg dw_config(const Shape& s, int sm_count) {
     return c;
 }
 
-cudaError_t dw_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, int sm_count,
-                       const Launch& st) {
+DwPlan dw_plan(const Shape& s, int sm_count) {
+    DwPlan p = {};
     // small planes go through shared memory in batches of whole planes (direct_dw_plane.cu); 3x3 stride 1 on 28x28 planes
     // measured the same on both kernels (16.5 us on 192 planes, N = 64) and stays on the stream
-    if (dw_plane_supported(s) && !(s.KH == 3 && s.stride == 1 && s.W == 28)) return dw_plane_forward(s, x, packed, y, status, sm_count, st);
-    const DwCfg c = dw_config(s, sm_count);
+    p.planes = dw_plane_supported(s) && !(s.KH == 3 && s.stride == 1 && s.W == 28);
+    if (p.planes) p.batches = dw_plane_config(s, sm_count);
+    else p.strips = dw_config(s, sm_count);
+    return p;
+}
+
+cudaError_t dw_forward(const Shape& s, const DwPlan& plan, const float* x, const void* packed, float* y, Status* status,
+                       const Launch& st) {
+    if (plan.planes) return dw_plane_forward(s, plan.batches, x, packed, y, status, st);
+    const DwCfg& c = plan.strips;
     const uint32_t tag = pack_tag(s, GCONV_VARIANT_DIRECT_TILED);
     const uint32_t* pk = reinterpret_cast<const uint32_t*>(packed);
     cudaError_t e;

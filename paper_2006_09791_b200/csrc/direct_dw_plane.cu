@@ -323,9 +323,8 @@ DwPlaneCfg dw_plane_config(const Shape& s, int sm_count) {
     return c;
 }
 
-cudaError_t dw_plane_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, int sm_count,
+cudaError_t dw_plane_forward(const Shape& s, const DwPlaneCfg& c, const float* x, const void* packed, float* y, Status* status,
                              const Launch& st) {
-    const DwPlaneCfg c = dw_plane_config(s, sm_count);
     const uint32_t tag = pack_tag(s, GCONV_VARIANT_DIRECT_TILED);
     const uint32_t* pk = reinterpret_cast<const uint32_t*>(packed);
 #define GCONV_PLANE_W(K, S) \

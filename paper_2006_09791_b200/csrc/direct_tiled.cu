@@ -52,9 +52,9 @@ cudaError_t tiled_pack(const Shape& s, const float* w, void* packed, cudaStream_
     return group_pack(s, w, packed, pack_tag(s, GCONV_VARIANT_DIRECT_TILED), st);
 }
 
-cudaError_t tiled_forward(const Shape& s, const ConvCfg* conv, const float* x, const void* packed, float* y, Status* status, int sm_count,
-                          const Launch& st) {
-    if (dw_supported(s)) return dw_forward(s, x, packed, y, status, sm_count, st);
+cudaError_t tiled_forward(const Shape& s, const ConvCfg* conv, const DwPlan& dw, const float* x, const void* packed, float* y, Status* status,
+                          int sm_count, const Launch& st) {
+    if (dw_supported(s)) return dw_forward(s, dw, x, packed, y, status, st);
     if (rows_supported(s)) return rows_forward(s, x, packed, y, status, st);
     return generic_forward(s, conv, x, packed, y, status, sm_count, pack_tag(s, GCONV_VARIANT_DIRECT_TILED), st);
 }

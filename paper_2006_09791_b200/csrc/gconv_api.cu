@@ -38,11 +38,13 @@ int select_variant(const Shape& s) {
     return GCONV_VARIANT_DIRECT_GENERIC;
 }
 
-// What the descriptor's variant keeps from call to call: the staged FP32 kernel's tile (a search over a few hundred choices).
+// What the descriptor's variant keeps from call to call: the staged FP32 kernel's tile (a search over a few hundred choices), the
+// depthwise kernels' strips and batches.
 void choose_tile(gconv_desc* d) {
     d->has_conv = false;
     if (d->variant == GCONV_VARIANT_DIRECT_GENERIC || (d->variant == GCONV_VARIANT_DIRECT_TILED && tiled_takes_conv(d->s)))
         d->has_conv = conv_config(d->s, 148, d->conv);
+    if (d->variant == GCONV_VARIANT_DIRECT_TILED && dw_supported(d->s)) d->dw = dw_plan(d->s, 148);
 }
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -103,7 +105,7 @@ int launch_forward(gconv_desc* d, const float* x, const void* packed, float* y, 
     const Launch to = {st, may_overlap && fp32_overlaps(d->s)};
     switch (d->variant) {
         case GCONV_VARIANT_DIRECT_TILED:
-            e = tiled_forward(d->s, d->conv_plan(), x, packed, y, status, d->sm_count, to);
+            e = tiled_forward(d->s, d->conv_plan(), d->dw, x, packed, y, status, d->sm_count, to);
             break;
         case GCONV_VARIANT_IGEMM_TF32: {
             const IgemmPlan* plan = igemm_plan(d->plans, d->s, 0, d->device, d->sm_count, x, &e);

@@ -43,6 +43,23 @@ struct ConvCfg {
     size_t smem;
     FastDiv div_ph, div_cc, div_sw, div_bm, div_tile, div_tw;
 };
+// DIRECT_TILED, depthwise stream kernel: a warp holds `subs` row strips of XQ lanes each.
+struct DwCfg {
+    int XQ, subs, RH, chunks;   // lanes per row, rows' strips per warp, output rows per thread, row chunks per plane
+    FastDiv div_chunks;
+    uint32_t items, blocks;
+};
+// depthwise on small planes (direct_dw_plane.cu): batches of whole planes through shared memory
+struct DwPlaneCfg {
+    int PB, upp;                 // planes per batch, units (one strip of one or two output rows) per plane
+    uint32_t planes, batches, grid, threads, smem_bytes;
+    FastDiv div_upp, div_c;
+};
+struct DwPlan {
+    bool planes;                 // which of the two kernels runs
+    DwCfg strips;
+    DwPlaneCfg batches;
+};
 }  // namespace gconv
 
 // The descriptor behind gconv_desc_t.
@@ -62,6 +79,7 @@ struct gconv_desc {
     int dbg_skip;                // failure-path test hook: stage fill that CTA 0's producer leaves out (-1 = none)
     gconv::ConvCfg conv;         // tile and launch geometry of the staged FP32 kernel, where the variant runs it (chosen once)
     bool has_conv;
+    gconv::DwPlan dw;            // depthwise shapes of the tiled variant: strip or batch geometry (chosen once)
     // plans of the tensor-core variant, one per (pointwise outputs of a fused block, device): immutable once published, freed
     // with the descriptor (calls of several threads may look them up and add to the list at the same time)
     std::atomic<gconv::IgemmPlan*> plans;
@@ -163,25 +181,13 @@ bool rows_supported(const Shape& s);
 RowsCfg rows_config(const Shape& s);
 cudaError_t rows_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, const Launch& st);
 
-// DIRECT_TILED, depthwise stream kernel: a warp holds `subs` row strips of XQ lanes each.
-struct DwCfg {
-    int XQ, subs, RH, chunks;   // lanes per row, rows' strips per warp, output rows per thread, row chunks per plane
-    FastDiv div_chunks;
-    uint32_t items, blocks;
-};
-// depthwise on small planes (direct_dw_plane.cu): batches of whole planes through shared memory
-struct DwPlaneCfg {
-    int PB, upp;                 // planes per batch, units (one strip of one or two output rows) per plane
-    uint32_t planes, batches, grid, threads, smem_bytes;
-    FastDiv div_upp, div_c;
-};
 bool dw_plane_supported(const Shape& s);
 DwPlaneCfg dw_plane_config(const Shape& s, int sm_count);
-cudaError_t dw_plane_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, int sm_count,
+cudaError_t dw_plane_forward(const Shape& s, const DwPlaneCfg& c, const float* x, const void* packed, float* y, Status* status,
                              const Launch& st);
 bool dw_supported(const Shape& s);
-DwCfg dw_config(const Shape& s, int sm_count);
-cudaError_t dw_forward(const Shape& s, const float* x, const void* packed, float* y, Status* status, int sm_count,
+DwPlan dw_plan(const Shape& s, int sm_count);
+cudaError_t dw_forward(const Shape& s, const DwPlan& plan, const float* x, const void* packed, float* y, Status* status,
                        const Launch& st);
 
 // DIRECT_TILED
@@ -190,8 +196,8 @@ bool tiled_takes_conv(const Shape& s);   // neither depthwise nor narrow groups:
 size_t tiled_packed_bytes(const Shape& s);
 cudaError_t group_pack(const Shape& s, const float* w, void* packed, uint32_t tag, cudaStream_t st);
 cudaError_t tiled_pack(const Shape& s, const float* w, void* packed, cudaStream_t st);
-cudaError_t tiled_forward(const Shape& s, const ConvCfg* conv, const float* x, const void* packed, float* y, Status* status, int sm_count,
-                          const Launch& st);
+cudaError_t tiled_forward(const Shape& s, const ConvCfg* conv, const DwPlan& dw, const float* x, const void* packed, float* y, Status* status,
+                          int sm_count, const Launch& st);
 
 // IGEMM_TF32: tile geometry of the tcgen05 implicit-GEMM kernel.
 struct IgemmCfg {
