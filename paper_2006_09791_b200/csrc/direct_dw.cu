@@ -452,9 +452,16 @@ DwCfg dw_config(const Shape& s, int sm_count) {
 
 DwPlan dw_plan(const Shape& s, int sm_count) {
     DwPlan p = {};
-    // small planes go through shared memory in batches of whole planes (direct_dw_plane.cu); 3x3 stride 1 on 28x28 planes
-    // measured the same on both kernels (16.5 us on 192 planes, N = 64) and stays on the stream
-    p.planes = dw_plane_supported(s) && !(s.KH == 3 && s.stride == 1 && s.W == 28);
+    // Small planes go through shared memory in batches of whole planes (direct_dw_plane.cu) once there are enough of them: a
+    // batch passes through two bulk copies and two barriers one after the other, and a few batches do not hide that.  Planes
+    // below which the strips were faster (us on batches / on strips): 28x28, 5x5 stride 1, 3000 planes 10.2 / 8.2, 10000 21.4 /
+    // 24.6; 28x28 stride 2, 5x5, 10000 14.8 / 13.9, 20000 22.1 / 25.3; 14x14, 3x3, 9000 4.8 / 4.4, 30000 12.5 / 15.1;
+    // 14x14, 5x5, 3000 5.1 / 4.1, 7000 5.6 / 6.3; 7x7, 500 2.4 / 2.1, 20000 3.7 / 4.6; 7x7, 3x3 stride 2, 20000 3.4 / 2.9, 50000
+    // 4.1 / 5.1.  3x3 stride 1 on 28x28 planes measured the same on both and stays on the strips.
+    const int fewest = s.W == 28 ? (s.stride == 2 ? 16384 : 4096)
+                                 : s.W == 14 ? (s.KH == 3 ? 12288 : 6144) : (s.KH == 3 && s.stride == 2 ? 24576 : 2048);
+    p.planes = dw_plane_supported(s) && !(s.KH == 3 && s.stride == 1 && s.W == 28) &&
+               (double)s.N * s.C_in * s.H > (double)fewest * s.W;
     if (p.planes) p.batches = dw_plane_config(s, sm_count);
     else p.strips = dw_config(s, sm_count);
     return p;

@@ -118,13 +118,14 @@ dw_plane_kernel(const Shape s, const DwPlaneCfg c, const float* __restrict__ x, 
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncthreads();
-    // a whole batch goes through the bulk copies (sizes and addresses are multiples of 16 bytes: PB is a multiple of 4);
-    // the last batch of the tensor may be short and is moved with plain loads and stores
+    // Bulk copies start and end on multiples of 16 bytes.  PB is a multiple of 4, so every batch starts on one; the last
+    // batch of the tensor may be short, and its last one to three floats go through plain loads and stores (moving all of a
+    // short batch that way took 5 ... 8 us, longer than the rest of the kernel).
+    auto planes_of = [&](uint32_t b) { return min((uint32_t)c.PB, c.planes - b * (uint32_t)c.PB); };
     auto issue = [&](uint32_t b, uint32_t buf) {
-        if ((uint64_t)(b + 1) * (uint64_t)c.PB > (uint64_t)c.planes) return;
-        const uint32_t bar = smem_addr(&full[buf]);
-        bar_expect_tx(bar, in_elems * 4u);
-        bulk_load(smem_addr(in_buf + buf * in_elems), x + (size_t)b * in_elems, in_elems * 4u, bar);
+        const uint32_t bar = smem_addr(&full[buf]), bytes = (planes_of(b) * (uint32_t)HW & ~3u) * 4u;
+        bar_expect_tx(bar, bytes);
+        bulk_load(smem_addr(in_buf + buf * in_elems), x + (size_t)b * in_elems, bytes, bar);
     };
     uint32_t b = blockIdx.x, it = 0;
     if (tid == 0 && b < c.batches) issue(b, 0);
@@ -135,21 +136,16 @@ dw_plane_kernel(const Shape s, const DwPlaneCfg c, const float* __restrict__ x, 
         __syncthreads();                                 // ... and every thread is done with the previous batch's input
         if (tid == 0 && nb < c.batches) issue(nb, buf ^ 1u);
         const uint32_t plane0 = b * (uint32_t)c.PB;
-        const int np = (int)min((uint32_t)c.PB, c.planes - plane0);
-        const bool whole = np == c.PB;
+        const int np = (int)planes_of(b);
         float* const in = in_buf + buf * in_elems;
         float* const out = out_buf + buf * out_elems;
-        if (whole) {
-            // one thread polls; the others sleep in the barrier below instead of spending issue slots on the poll loop
-            if (tid == 0 && !bar_wait(smem_addr(&full[buf]), (it >> 1) & 1u)) failed = 1;
-            if (__syncthreads_or(failed)) {
-                if (tid == 0) record_status(status, GCONV_ERR_TIMEOUT, 50 + (int)buf);
-                break;
-            }
-        } else {
-            const float* src = x + (size_t)plane0 * HW;
-            for (int i = tid; i < np * HW; i += (int)blockDim.x) in[i] = __ldg(src + i);
-            __syncthreads();
+        const int in_tail = np * HW & 3, out_tail = np * OHW & 3;
+        if (tid < in_tail) in[np * HW - in_tail + tid] = __ldg(x + (size_t)plane0 * HW + np * HW - in_tail + tid);
+        // one thread polls; the others sleep in the barrier below instead of spending issue slots on the poll loop
+        if (tid == 0 && !bar_wait(smem_addr(&full[buf]), (it >> 1) & 1u)) failed = 1;
+        if (__syncthreads_or(failed)) {
+            if (tid == 0) record_status(status, GCONV_ERR_TIMEOUT, 50 + (int)buf);
+            break;
         }
         if constexpr (WHOLE) {
             for (int pl = tid; pl < np; pl += (int)blockDim.x) {
@@ -233,15 +229,10 @@ dw_plane_kernel(const Shape s, const DwPlaneCfg c, const float* __restrict__ x, 
                 }
             }
         }
-        if (whole) {
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the bulk store reads shared memory through the async proxy
-            __syncthreads();
-            if (tid == 0) bulk_store(y + (size_t)plane0 * OHW, smem_addr(out), out_elems * 4u);
-        } else {
-            __syncthreads();
-            float* dst = y + (size_t)plane0 * OHW;
-            for (int i = tid; i < np * OHW; i += (int)blockDim.x) dst[i] = out[i];
-        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the bulk store reads shared memory through the async proxy
+        __syncthreads();
+        if (tid == 0) bulk_store(y + (size_t)plane0 * OHW, smem_addr(out), (uint32_t)(np * OHW & ~3) * 4u);
+        if (tid < out_tail) y[(size_t)plane0 * OHW + np * OHW - out_tail + tid] = out[np * OHW - out_tail + tid];
     }
     if (tid == 0) {
         asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // every bulk store of this CTA has completed (shared memory must

@@ -31,3 +31,16 @@ def test_depthwise_strips(cfg):
     N, C, H, W, k, stride = cfg
     err, used = check_layer(Layer("dw", N, C, H, W, C, k, k, stride, k // 2, 1, C), seed=47)
     assert used == gconv.GCONV_VARIANT_DIRECT_TILED and err <= 2e-6      # sums of at most 25 products: 2^-24 x 25 is 1.5e-6
+
+
+BATCHES = [  # N, C, H, W, filter, stride: enough small planes for batches in shared memory; N * C and H * W leave a short last batch
+    # whose floats end 1, 2 or 3 past a multiple of four, one plane in the last batch, whole batches only
+    (1, 2049, 7, 7, 3, 1), (1, 2051, 7, 7, 5, 1), (3, 1367, 5, 7, 3, 1), (64, 64, 7, 7, 5, 1), (11, 2235, 7, 7, 3, 2), (2, 1087, 7, 7, 5, 2),
+    (9, 1367, 14, 14, 3, 1), (7, 1888, 13, 14, 3, 2), (1, 6151, 14, 14, 5, 1), (5, 1231, 14, 14, 5, 2), (1, 4251, 27, 28, 5, 1),
+    (2, 8197, 28, 28, 5, 2), (3, 5667, 27, 28, 3, 2),
+]
+
+
+@pytest.mark.parametrize("cfg", BATCHES)
+def test_depthwise_batches_of_planes(cfg):
+    test_depthwise_strips(cfg)
