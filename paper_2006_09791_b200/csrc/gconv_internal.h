@@ -223,6 +223,7 @@ struct IgemmCfg {
     int soft;                     // gather producer: raw input rows land in a ring by bulk copy, copy warps build the operand stages from
                                   // them (1: stride 1, three vertical-tap blocks; 2: stride 2, even/odd column blocks per tap)
     int flat;                     // pointwise, stride 1: pixels of a plane cut into segments of 32, the last one short (0: rows as they are)
+    int flat_in;                  // ... and of a plane of the input it reads (a multiple of 4: the padded copy on odd planes)
     int row_skip;                 // pointwise, stride 2: the tensor map holds the even rows only
     int sub_h, sub_w;             // 1: a stride of 2 on that axis, taken as the even rows (columns) of the stride-1 result when it is stored
     int rps, IPT;                 // gather tilings: output rows per 32-lane segment; whole images per tile (1: a tile is part of one image)

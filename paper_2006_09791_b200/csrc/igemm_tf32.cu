@@ -358,9 +358,9 @@ __host__ __device__ constexpr Family family(int f) {
          : f == 14 ? Family{1,  0,  3,  0,   2,  2,  0,  1,  1, 32,  1, 32,  96,  1,  2,  2, -1,  0, -1,  -1, -1,  1,  0,  1, -1,  0,  0}     // fused block, row boxes, two resident banks
          : f == 15 ? Family{0,  0,  3,  0,   1,  1,  0,  1,  1, 16, -1, -1,  -1, -1,  2,  2,  0,  0,  4,  12,  0, -1,  0,  0,  0,  1,  0}     // gather producer, stride 1 (14x14, 7x7, ... planes), narrow groups, 16-channel stages
          : f == 16 ? Family{0,  0,  3,  0,   1,  1,  0,  1,  2, 16, -1, -1,  -1, -1,  2,  2,  0,  0,  8,  24,  0, -1,  0,  0,  0,  2,  0}     // gather producer, stride 2 (even/odd column blocks), narrow groups, 16-channel stages
-         : f == 17 ? Family{0, 1, 1, 0, 1, 1, 0, 1, -1, 32, -1, -1, -1, -1, 2, 2, 0, 0, 0, 4, 0, -1, 0, 0, 0, 0, 1}     // pointwise, segment tilings, two CTAs per SM
+         : f == 17 ? Family{0, 1, 1, 0, 1, 1, 0, 1, -1, 32, -1, -1, -1, -1, 2, 2, -1, 0, 0, 4, 0, -1, 0, 0, 0, 0, 1}     // pointwise, segment tilings, two CTAs per SM
          : f == 18 ? Family{1, 0, 1, 0, -1, -1, 0, 1, -1, 32, -1, -1, -1, -1, -1, -1, 0, -1, 0, 4, -1, 1, 0, 0, 0, 0, 1}     // pointwise, row boxes
-         : f == 19 ? Family{0, 1, 1, 0, -1, -1, 0, 1, -1, 32, -1, -1, -1, -1, -1, -1, 0, -1, 0, 4, 0, -1, 0, 0, 0, 0, 1}     // pointwise, segment tilings, one CTA per SM
+         : f == 19 ? Family{0, 1, 1, 0, -1, -1, 0, 1, -1, 32, -1, -1, -1, -1, -1, -1, -1, -1, 0, 4, 0, -1, 0, 0, 0, 0, 1}     // pointwise, segment tilings, one CTA per SM
          : f == 20 ? Family{1,   0,  3,  0,   1,  1,  1,  2,  2, 16,  1, 32,  96,  1,  2,  2, -1,  0,  1,   9, -1,  1,  0,  0,  0,  0,  0}     // stride-2 row tiles, 16-channel merged groups (channel-doubling transitions)
          : f == 21 ? Family{1,   0,  3,  0,   0,  2,  0,  1,  1, 16, -1, 64, 192, -1,  1,  1, -1, -1, -1,  -1, -1,  1,  0,  0,  0,  0,  0,  1}     // row boxes, 64-filter tiles, streamed weights shared by a pair of pixel tiles
          : f == 22 ? Family{1,   0,  3,  0,   1,  2,  1,  2,  2, 32, -1, 64, 192, -1,  2,  2, -1,  0,  1,   9, -1,  1,  0,  0,  0,  0,  0,  0}     // stride-2 row tiles, 64-filter tiles, one resident bank
@@ -517,7 +517,7 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
     const uint32_t b_tile_bytes = (uint32_t)vt * (uint32_t)c.chunks * blk_bytes;   // weights of one (group, filter tile)
     const uint32_t bres_base = smem_base;                                // two resident weight buffers (if b_res)
     const uint32_t stage_base = smem_base + (uint32_t)c.b_res * c.bres_stride;   // b_res = number of resident weight buffers
-    const int HW = c.flat ? c.flat : s.H * s.W;
+    const int HW = c.flat ? c.flat_in : s.H * s.W;
     const int rstep = s.W * s.dilation;          // flat-pixel distance between vertical taps
     const size_t OHW = c.flat ? (size_t)c.flat : (size_t)s.H_out * s.W_out;
 
@@ -1565,7 +1565,8 @@ EncodeTiledFn get_encode_fn() {
 // the row count padded until the plane is a whole number of 32-pixel segments).  The zero columns and rows are
 // exactly the convolution's right and bottom padding; outputs that fall in them are never stored.
 struct IgemmGeom {
-    int Hp, Wp;
+    int Hp, Wp;                  // the plane the kernel computes on
+    int copy_H, copy_W;          // rows and columns of a plane of the padded copy (a re-cut pointwise plane is one row)
     bool padded;
 };
 // A pointwise convolution (1x1, pad 0) runs as the 3x3, pad 1 convolution whose only non-zero tap is the centre one
@@ -1579,6 +1580,34 @@ static bool pw_rows_of_28(const Shape& s) {
     const long long hw = (long long)s.H * s.W;
     return s.KH == 1 && s.KW == 1 && s.stride == 1 && hw % 28 == 0 && hw % 32 != 0 && (hw < 400 || s.N * hw < 128ll * kLayoutSMs);
 }
+static int igemm_merge(const Shape& s) {
+    int m = 1;
+    // Stride 2: stop at 32 filters per merged group, so that channel-doubling transition layers (Kg = 2 Cg) keep one
+    // resident 32-filter bank and the two-CTA launch shape instead of streaming 64-filter banks (measured: 64 -> 128
+    // channels at 56x56, 32 groups, 35.5 -> 17.0 us).
+    const int kcap = s.stride == 2 ? 32 : 64;
+    while (m * 2 <= s.groups && s.groups % (m * 2) == 0 && s.Cg * m * 2 <= 32 && s.Kg * m * 2 <= kcap) m *= 2;
+    return m;
+}
+
+// Wide pointwise layers on planes the tiled copies cannot address (a width, or with stride 1 a pixel count, that is not a multiple of 4) read
+// a copy of x whose planes are one row each: with stride 1 the pixels as they are, with stride 2 only those the layer reads.  The planes
+// start on 16 bytes and take the same segments of 32 pixels.  (As rows of the padded width, 7x7 planes crossed in boxes of 32-byte rows and
+// in the generic instantiation, and stride 2 computed and dropped three of four pixels.)  Copy and layer, rows -> one row: 512 -> 512 @7x7
+// N = 64 34.1 -> 15.4 us, 256 -> 512 @13x13 N = 64 40.1 -> 19.9, 192 -> 384 @29x29 N = 41 55.6 -> 31.4, 256 -> 128 @25x25 N = 13 25.8 -> 11.1.
+// The planes are those that had a padded copy before; groups that merge to 32 channels at most, up to 32 wide, are gathered without one.
+static bool pw_one_row(const Shape& s) {
+    if (!(s.KH == 1 && s.KW == 1 && s.stride == s.stride_w && (s.stride == 1 || s.stride == 2)) || s.W > 128) return false;
+    const int Wp = (s.W + 3) & ~3;
+    const long long hw = (long long)s.H * s.W;
+    if (hw >= (1ll << 30) || !(32 % Wp == 0 || (long long)s.H * Wp >= 32)) return false;
+    return s.stride == 1 ? hw % 4 != 0 && (s.W > 32 || s.Cg * igemm_merge(s) > 32) : s.W % 4 != 0 && s.Cg > 32;
+}
+// Stride-1 planes cut into segments of 32 pixels whatever their rows.
+static bool pw_recut(const Shape& s) {
+    const long long hw = (long long)s.H * s.W;
+    return pw_one_row(s) || (s.KH == 1 && s.KW == 1 && s.stride == 1 && hw % 4 == 0 && hw < (1ll << 30));
+}
 static Shape as_3x3(const Shape& s) {
     Shape t = s;
     // One stride per axis (the paper's S_h, S_w) with a stride of 2 on one axis only: every tiling computes the stride-1 layer
@@ -1589,27 +1618,33 @@ static Shape as_3x3(const Shape& s) {
         t.KW = 3;
         t.pad = 1;
         t.dilation = 1;
-        if (s.stride == 1) {
-            const long long hw = (long long)s.H * s.W;
-            if (pw_rows_of_28(s)) {
-                t.W = t.W_out = 28;
-                t.H = t.H_out = (int)(hw / 28);
-            } else if (hw % 4 == 0 && hw < (1ll << 30)) {
-                t.W = t.W_out = 32;              // (the last row of 32 may be short: IgemmCfg::flat)
-                t.H = t.H_out = (int)((hw + 31) / 32);
-            }
+        if (pw_rows_of_28(s)) {
+            t.W = t.W_out = 28;
+            t.H = t.H_out = s.H * s.W / 28;
+        } else if (pw_recut(s)) {
+            t.stride = t.stride_w = 1;
+            t.W = t.W_out = 32;                  // (the last row of 32 may be short: IgemmCfg::flat)
+            t.H = t.H_out = (s.H_out * s.W_out + 31) / 32;
         }
     }
     return t;
 }
 
-static IgemmGeom igemm_geom(const Shape& s) {
+static IgemmGeom igemm_geom(const Shape& s_any) {
+    const Shape s = as_3x3(s_any);
     IgemmGeom g;
     g.Wp = (s.W + 3) & ~3;
     g.Hp = s.H;
     g.padded = g.Wp != s.W;
     if (g.padded && 32 % g.Wp == 0)
         while ((g.Hp * g.Wp) % 32 != 0) ++g.Hp;
+    g.copy_H = g.Hp;
+    g.copy_W = g.Wp;
+    if (pw_one_row(s_any)) {
+        g.padded = true;
+        g.copy_H = 1;
+        g.copy_W = (s_any.H_out * s_any.W_out + 3) & ~3;
+    }
     return g;
 }
 
@@ -1669,17 +1704,53 @@ __global__ void __launch_bounds__(256) igemm_pad_kernel(const float* __restrict_
             if (dst[k] != nullptr) *reinterpret_cast<float4*>(dst[k]) = make_float4(v[k][0], v[k][1], v[k][2], v[k][3]);
     }
 }
-}  // namespace
 
-static int igemm_merge(const Shape& s) {
-    int m = 1;
-    // Stride 2: stop at 32 filters per merged group, so that channel-doubling transition layers (Kg = 2 Cg) keep one
-    // resident 32-filter bank and the two-CTA launch shape instead of streaming 64-filter banks (measured: 64 -> 128
-    // channels at 56x56, 32 groups, 35.5 -> 17.0 us).
-    const int kcap = s.stride == 2 ? 32 : 64;
-    while (m * 2 <= s.groups && s.groups % (m * 2) == 0 && s.Cg * m * 2 <= 32 && s.Kg * m * 2 <= kcap) m *= 2;
-    return m;
+// The pixels a stride-2 pointwise layer reads, every plane one row of `pitch` floats.  As above; a thread's four pixels are 32 bytes apart at
+// most, so a warp's loads touch whole runs of the rows it reads.
+template <typename IDX>
+__global__ void __launch_bounds__(256) igemm_take_kernel(const float* __restrict__ x, float* __restrict__ xp, size_t planes, int H, int W, int W_out,
+                                                         int pixels, int pitch, FastDiv div_plane, FastDiv div_row) {
+    dependent_start();
+    const size_t per_plane = (size_t)(pitch / 4), total = planes * per_plane, step = (size_t)gridDim.x * blockDim.x;
+    for (size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < total; i0 += kPadItems * step) {
+        float v[kPadItems][4];
+#pragma unroll
+        for (int k = 0; k < kPadItems; ++k) {
+            const size_t i = i0 + k * step;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[k][j] = 0.f;
+            if (i >= total) continue;
+            size_t plane;
+            uint32_t f;
+            if constexpr (sizeof(IDX) == 4) {
+                uint32_t pl;
+                div_plane.divmod((uint32_t)i, pl, f);
+                plane = pl;
+            } else {
+                plane = i / per_plane;
+                f = (uint32_t)(i - plane * per_plane);
+            }
+            f *= 4;
+            uint32_t h, w;
+            div_row.divmod(f, h, w);
+            const float* src = x + (plane * H + 2 * h) * (size_t)W;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if ((int)f + j < pixels) v[k][j] = __ldg(src + 2 * w);
+                if ((int)++w == W_out) {
+                    w = 0;
+                    src += 2 * (size_t)W;
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kPadItems; ++k) {
+            const size_t i = i0 + k * step;
+            if (i < total) *reinterpret_cast<float4*>(xp + 4 * i) = make_float4(v[k][0], v[k][1], v[k][2], v[k][3]);
+        }
+    }
 }
+}  // namespace
 
 bool igemm_supported(const Shape& s_any) {
     if (!s_any.square()) {
@@ -1700,7 +1771,7 @@ bool igemm_supported(const Shape& s_any) {
     if (s.dilation > 1 && (s.stride != 1 || s.dilation > 16)) return false;
     const int m = igemm_merge(s);
     if ((s.Cg * m) % 8 != 0 || (s.Kg * m) % 8 != 0) return false;
-    const IgemmGeom ge = igemm_geom(s);
+    const IgemmGeom ge = igemm_geom(s_any);
     if (ge.Wp > 128) return false;
     if ((long long)ge.Hp * ge.Wp < 32) return false;
     if (s.C_in > 65535 * 8) return false;
@@ -1712,10 +1783,9 @@ bool igemm_supported(const Shape& s_any) {
 }
 
 size_t igemm_scratch_bytes(const Shape& s_any) {
-    const Shape s = as_3x3(s_any);
-    const IgemmGeom ge = igemm_geom(s);
+    const IgemmGeom ge = igemm_geom(s_any);
     if (!ge.padded || igemm_config(s_any, kLayoutSMs).soft) return 0;   // the gather producer reads the real rows: no padded copy
-    return sizeof(float) * (size_t)s.N * s.C_in * ge.Hp * ge.Wp;
+    return sizeof(float) * (size_t)s_any.N * s_any.C_in * ge.copy_H * ge.copy_W;
 }
 
 
@@ -1914,17 +1984,19 @@ static IgemmCfg igemm_config_c2(const Shape& s_any, int sm_count, int C2) {
     // Pointwise: one vertical tap (a third of the stages and MMAs), one accumulator per filter (N = Kt), filter tiles of
     // up to 128.  Stride 2 computes every pixel and stores the even ones (no stride-2 row tiles: those are built around
     // nine staged rows).
-    c.sub_h = s_any.stride == 2 ? 1 : 0;
-    c.sub_w = s_any.stride_w == 2 ? 1 : 0;
+    const bool one_row = pw_one_row(s_any);              // (with stride 2 only the pixels the layer reads are there)
+    c.sub_h = s_any.stride == 2 && !one_row ? 1 : 0;
+    c.sub_w = s_any.stride_w == 2 && !one_row ? 1 : 0;
     c.pw = (s_any.KH == 1 && s_any.KW == 1 && C2 == 0) ? 1 : 0;
-    c.flat = (!pw_rows_of_28(s_any) && s_any.KH == 1 && s_any.KW == 1 && s_any.stride == 1 && (long long)s_any.H * s_any.W % 4 == 0 && (long long)s_any.H * s_any.W < (1ll << 30)) ? s_any.H * s_any.W : 0;
+    c.flat = !pw_rows_of_28(s_any) && pw_recut(s_any) ? s_any.H_out * s_any.W_out : 0;
+    c.flat_in = (c.flat + 3) & ~3;
     // Pointwise with stride 2 on planes the tiled copies address: the tensor map steps two rows at a time, so the odd rows are neither
     // fetched nor multiplied (the odd columns are: TMA cannot skip elements of the innermost dimension).
     c.row_skip = (c.pw && c.sub_h && s_true.W % 4 == 0 && s_true.W <= 64) ? 1 : 0;
     if (c.row_skip) c.sub_h = 0;
     const int vt = c.pw ? 1 : 3;
     const bool fuse = C2 > 0;          // fused grouped + pointwise block: heavy shape, streamed or resident grouped weights
-    const IgemmGeom ge = igemm_geom(s_true);
+    const IgemmGeom ge = igemm_geom(s_any);
     Shape s = s_true;          // the plane the kernel computes on
     s.H = c.row_skip ? s.H_out : ge.Hp;
     s.W = ge.Wp;
@@ -1945,9 +2017,16 @@ static IgemmCfg igemm_config_c2(const Shape& s_any, int sm_count, int C2) {
     int kt = c.Kg <= kt_max ? c.Kg : kt_max;
     while (c.Kg % kt != 0 || kt % 8 != 0) kt -= 8;   // largest multiple of 8 dividing Kg, at most 64 (pointwise: 128 or 256)
     if (c.pw) {
-        // small planes: narrower filter tiles until there is a tile per SM (each re-reads its pixels from L2)
+        // small planes: narrower filter tiles where they fill more SMs.  A tile's time goes with what it copies, 128 pixels and kt
+        // filters of every channel: the least waves x (128 + kt).  (512 -> 512 @7x7 N = 64: 128 tiles of 128 filters.)
         const long long px_tiles = ((long long)s.N * s.H * s.W + 127) / 128;
-        while (kt >= 64 && kt % 16 == 0 && (long long)c.groups * (c.Kg / kt) * px_tiles < (long long)kLayoutSMs) kt /= 2;
+        auto cost = [&](int k) { return ((long long)c.groups * (c.Kg / k) * px_tiles + kLayoutSMs - 1) / kLayoutSMs * (128 + k); };
+        int best = kt;
+        while (kt >= 64 && kt % 16 == 0) {
+            kt /= 2;
+            if (cost(kt) < cost(best)) best = kt;
+        }
+        kt = best;
     }
     c.Kt = kt;
     c.NT = c.Kg / kt;
@@ -2317,7 +2396,8 @@ struct IgemmPlan {
     CUtensorMap map, map4;
     // zero-padded copy of x (widths no tiling addresses): the true plane and the launch that fills the copy
     size_t scratch_bytes, pad_total, pad_planes;
-    int pad_blocks, pad_H, pad_W;
+    int pad_blocks, pad_H, pad_W, pad_Hp, pad_Wp, take_W;
+    bool take;                   // ... with the pixels a stride-2 pointwise layer reads
     FastDiv pad_div_plane, pad_div_row;
     IgemmPlan* next;
 };
@@ -2329,25 +2409,29 @@ static cudaError_t make_plan(IgemmPlan& p, const Shape& s_true, int sm_count, co
     Shape s = as_3x3(s_true);
     p.scratch_bytes = 0;
     if (c.padded) {
-        const IgemmGeom ge = igemm_geom(s);
-        p.pad_H = s.H;
-        p.pad_W = s.W;
+        const IgemmGeom ge = igemm_geom(s_true);
+        p.take = c.flat > 0 && s_true.stride == 2;
+        p.pad_H = p.take ? s_true.H : (c.flat ? 1 : s.H);
+        p.pad_W = p.take ? s_true.W : (c.flat ? c.flat : s.W);
+        p.pad_Hp = ge.copy_H;
+        p.pad_Wp = ge.copy_W;
         p.pad_planes = (size_t)s.N * s.C_in;
-        p.pad_total = p.pad_planes * ge.Hp * (ge.Wp / 4);
+        p.pad_total = p.pad_planes * ge.copy_H * (ge.copy_W / 4);
         const size_t blocks = (p.pad_total + 256 * kPadItems - 1) / (256 * kPadItems), most = (size_t)sm_count * 16;
         p.pad_blocks = (int)(blocks < most ? blocks : most);
-        p.pad_div_plane = make_fastdiv((uint32_t)(ge.Hp * (ge.Wp / 4)));
-        p.pad_div_row = make_fastdiv((uint32_t)(ge.Wp / 4));
+        p.pad_div_plane = make_fastdiv((uint32_t)(ge.copy_H * (ge.copy_W / 4)));
+        p.pad_div_row = make_fastdiv(p.take ? (uint32_t)s_true.W_out : (uint32_t)(ge.copy_W / 4));
+        p.take_W = s_true.W_out;
         s.H = ge.Hp;
         s.W = ge.Wp;
-        p.scratch_bytes = sizeof(float) * p.pad_planes * ge.Hp * ge.Wp;
+        p.scratch_bytes = sizeof(float) * p.pad_planes * ge.copy_H * ge.copy_W;
     }
     p.s = s;
     if (c.row_skip) p.s.H = s.H_out;             // the plane of even rows
     EncodeTiledFn encode = get_encode_fn();
     if (encode == nullptr || get_replace_fn() == nullptr) return cudaErrorNotSupported;
     CUtensorMap &xmap = p.map, &xmap4 = p.map4;
-    const cuuint64_t HW = c.flat ? (cuuint64_t)c.flat : (cuuint64_t)s.H * s.W;
+    const cuuint64_t HW = c.flat ? (cuuint64_t)c.flat_in : (cuuint64_t)s.H * s.W;
     const cuuint64_t dims[3] = {HW, (cuuint64_t)s.C_in, (cuuint64_t)s.N};
     const cuuint64_t strides[2] = {HW * 4, HW * 4 * (cuuint64_t)s.C_in};
     const cuuint32_t box[3] = {32, (cuuint32_t)c.CK, 1};
@@ -2478,11 +2562,16 @@ cudaError_t igemm_run(const IgemmPlan* plan, const float* x, const void* packed,
         const Launch to = {st, opts.pdl && p.pad_total * 16 <= 20000000};
         const unsigned grid = (unsigned)p.pad_blocks;
         auto copy = [&](auto kernel_tag) {
-            return launch_kernel<decltype(kernel_tag)::value>(grid, 256, 0, to, 1, x, scratch, p.pad_planes, p.pad_H, p.pad_W, p.s.H, p.s.W,
+            return launch_kernel<decltype(kernel_tag)::value>(grid, 256, 0, to, 1, x, scratch, p.pad_planes, p.pad_H, p.pad_W, p.pad_Hp, p.pad_Wp,
                                                               p.pad_div_plane, p.pad_div_row);
         };
         const bool small = p.pad_total < (1ull << 31), even = (p.pad_W & 1) == 0;
-        const cudaError_t e = small ? (even ? copy(Kernel<igemm_pad_kernel<uint32_t, true>>()) : copy(Kernel<igemm_pad_kernel<uint32_t, false>>()))
+        auto take = [&](auto kernel_tag) {
+            return launch_kernel<decltype(kernel_tag)::value>(grid, 256, 0, to, 1, x, scratch, p.pad_planes, p.pad_H, p.pad_W, p.take_W, p.cfg.flat,
+                                                              p.pad_Wp, p.pad_div_plane, p.pad_div_row);
+        };
+        const cudaError_t e = p.take ? (small ? take(Kernel<igemm_take_kernel<uint32_t>>()) : take(Kernel<igemm_take_kernel<uint64_t>>()))
+                            : small ? (even ? copy(Kernel<igemm_pad_kernel<uint32_t, true>>()) : copy(Kernel<igemm_pad_kernel<uint32_t, false>>()))
                                     : (even ? copy(Kernel<igemm_pad_kernel<uint64_t, true>>()) : copy(Kernel<igemm_pad_kernel<uint64_t, false>>()));
         if (e != cudaSuccess) return e;
         x = scratch;

@@ -37,3 +37,17 @@ def test_planes_that_stay_on_the_fp32_variants(cfg):
     N, C, H, W, K = cfg
     err, used = check_layer(Layer("pw32", N, C, H, W, K, 1, 1, 1, 0, 1, 1), seed=19)
     assert used != gconv.GCONV_VARIANT_IGEMM_TF32
+
+
+ONE_ROW = [  # N, C_in, H, W, C_out, stride, groups: planes copied to one row each (1, 2 or 3 floats of padding, one segment or many, images
+    # that share a tile); stride 2 on odd, even and single-row planes, a last odd row or column; groups; every filter tile width
+    (5, 64, 7, 7, 64, 1, 1), (3, 96, 5, 5, 160, 1, 1), (2, 64, 9, 9, 72, 1, 1), (1, 128, 13, 13, 512, 1, 2), (2, 48, 25, 30, 64, 1, 1), (1, 40, 57, 57, 48, 1, 1),
+    (1, 64, 1, 127, 64, 1, 1), (4, 256, 3, 3, 256, 1, 1), (130, 512, 7, 7, 512, 1, 1), (2, 320, 5, 7, 320, 1, 1), (3, 32, 3, 33, 32, 1, 1),
+    (5, 64, 7, 7, 128, 2, 1), (3, 96, 15, 15, 96, 2, 1), (2, 256, 29, 29, 512, 2, 1), (1, 64, 50, 50, 128, 2, 1), (2, 128, 13, 26, 64, 2, 2), (1, 64, 1, 90, 64, 2, 1),
+    (2, 72, 58, 57, 200, 2, 1), (4, 512, 5, 5, 512, 2, 1), (1, 48, 33, 35, 48, 2, 1), (2, 64, 127, 127, 64, 2, 1),
+]
+
+
+@pytest.mark.parametrize("cfg", ONE_ROW)
+def test_pointwise_planes_of_one_row(cfg):
+    test_pointwise_tiles(cfg)
