@@ -454,12 +454,14 @@ DwPlan dw_plan(const Shape& s, int sm_count) {
     DwPlan p = {};
     // Small planes go through shared memory in batches of whole planes (direct_dw_plane.cu) once there are enough of them: a
     // batch passes through two bulk copies and two barriers one after the other, and a few batches do not hide that.  Planes
-    // below which the strips were faster (us on batches / on strips): 28x28, 5x5 stride 1, 3000 planes 10.2 / 8.2, 10000 21.4 /
-    // 24.6; 28x28 stride 2, 5x5, 10000 14.8 / 13.9, 20000 22.1 / 25.3; 14x14, 3x3, 9000 4.8 / 4.4, 30000 12.5 / 15.1;
-    // 14x14, 5x5, 3000 5.1 / 4.1, 7000 5.6 / 6.3; 7x7, 500 2.4 / 2.1, 20000 3.7 / 4.6; 7x7, 3x3 stride 2, 20000 3.4 / 2.9, 50000
-    // 4.1 / 5.1.  3x3 stride 1 on 28x28 planes measured the same on both and stays on the strips.
-    const int fewest = s.W == 28 ? (s.stride == 2 ? 16384 : 4096)
-                                 : s.W == 14 ? (s.KH == 3 ? 12288 : 6144) : (s.KH == 3 && s.stride == 2 ? 24576 : 2048);
+    // below which the strips were faster (us on batches / on strips): 28x28, 5x5 stride 1, 3000 planes 9.0 / 8.2, 5000 11.5 /
+    // 14.4; 28x28, 3x3 stride 2, 9000 9.2 / 8.4, 16384 13.1 / 13.8; 28x28, 5x5 stride 2, 6000 8.2 / 8.0, 10000 10.6 / 13.9; 14x14, 3x3, 12000 6.5 /
+    // 6.1, 16000 7.2 / 8.6; 14x14, 5x5, 1500 3.7 / 3.3, 3000 3.7 / 4.1, stride 2 5000 4.1 / 3.2, 9000 4.3 / 4.8; 7x7, 3x3, 2000 2.6 / 2.3, 6000 equal,
+    // 20000 3.9 / 4.7; 7x7, 5x5, 6000 4.4 / 3.5, 20000 5.5 / 7.8; 7x7 stride 2, 3x3, 20000 3.4 / 2.9, 50000 4.3 / 5.1, 5x5, 10000 3.9 / 3.4, 20000 4.2 / 4.6.
+    // 3x3 stride 1 on 28x28 planes measured the same on both and stays on the strips.
+    const bool k3 = s.KH == 3, s2 = s.stride == 2;
+    const int fewest = s.W == 28 ? (k3 ? 12288 : (s2 ? 6144 : 4096))
+                                 : s.W == 14 ? (k3 ? 12288 : (s2 ? 6144 : 2048)) : (s2 ? (k3 ? 24576 : 12288) : (k3 ? 2048 : 6144));
     p.planes = dw_plane_supported(s) && !(s.KH == 3 && s.stride == 1 && s.W == 28) &&
                (double)s.N * s.C_in * s.H > (double)fewest * s.W;
     if (p.planes) p.batches = dw_plane_config(s, sm_count);

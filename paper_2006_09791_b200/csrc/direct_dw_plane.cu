@@ -5,10 +5,8 @@
 // kernel of direct_dw.cu is bound by instruction issue: with rows of 7 or 14 pixels its 16-byte loads degrade to scalar
 // loads with a bounds check each.  Here the planes of NCHW are taken for what they are in memory, one contiguous run of
 // floats: a CTA brings a batch of PB whole planes into shared memory with ONE bulk copy (no per-element address
-// arithmetic, no bounds check, the next batch's copy in flight during this batch's math), every thread computes units
-// of two output rows by up to seven adjacent columns from shared memory (an input row's window is read once for both
-// output rows and all filter columns; the columns that fall into the padding are known at compile time and simply not
-// read), the results go to a second
+// arithmetic, no bounds check, the next batch's copy in flight during this batch's math), every thread computes whole
+// output rows from shared memory (the columns that fall into the padding are known at compile time), the results go to a second
 // shared-memory buffer and leave as ONE bulk store of the batch's output planes, which are contiguous as well.  This
 // plays the role of Algorithm 1's input and output reshaping without a pass over HBM: x is read once, y written once.
 // Sum order per output: (r, s) as in the convolution stage of Algorithm 1.
@@ -71,20 +69,19 @@ __device__ __forceinline__ void bulk_store_wait_read() {
     asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
 }
 
+// A unit is RPU whole output rows of a plane: an input row is 14 8-byte (28-wide planes: 7 16-byte) shared loads, no column of it outside the
+// image, and rows of 14 and 28 floats start an odd number of vectors apart, in different banks.  One row a unit: more units keep more
+// warps in flight, which is worth more than the rows that neighbouring units read again (N = 64, us with 1, 2 and 3 rows: 672 planes
+// of 14x14, 5x5 17.7, 18.8, 20.0; 384 of 28x28, 5x5 stride 2 19.9, 25.9, 24.4).  Two where a row is a handful of outputs (960 of 7x7, 5x5
+// stride 2 7.7, 6.2, 7.0; 672 of 14x14, 5x5 stride 2 12.5, 12.0, 12.8).
+constexpr int rows_per_unit(int K, int S, int W) { return W == 7 || (W == 14 && S == 2 && K == 5) ? 2 : 1; }
 template <int K, int S, int W>
 struct PlaneGeom {
     static constexpr int PAD = K / 2;
     static constexpr int W_OUT = (W - 1) / S + 1;
-    static constexpr int SW = W_OUT <= 8 ? W_OUT : 7;     // outputs per strip
-    static constexpr int NS = W_OUT / SW;                 // strips per output row: 1, 2 or 4
-    static constexpr int WN = (SW - 1) * S + K;           // input columns a strip reads
-    static constexpr int RLIM = W + PAD - (NS - 1) * SW * S;   // window columns from here on are right of the image in a row's last strip
-    // output rows per unit: two where an input row then serves both (stride 1), or where the planes are so small that
-    // fewer, longer units win anyway (14x14 and 7x7 with stride 2: measured 13.5 against 17.2 us on 672 planes of 14x14, 5x5);
-    // 28x28 planes with stride 2 need the threads more (17.6 against 27.3 us on 240 planes, 5x5)
-    static constexpr int RPU = (S == 1 || W <= 14) ? 2 : 1;
+    static constexpr int VEC = W % 4 == 0 ? 4 : (W % 2 == 0 ? 2 : 1);   // floats per shared load and, where W_OUT allows, store
+    static constexpr int RPU = rows_per_unit(K, S, W);
     static constexpr int NR = K + (RPU - 1) * S;          // input rows a unit reads
-    static_assert(W_OUT % SW == 0 && (NS & (NS - 1)) == 0, "rows are cut into equal strips");
 };
 
 // WHOLE (7x7 planes, stride 1): a thread computes a whole plane -- 49 inputs, the filter and 49 accumulators in
@@ -110,6 +107,8 @@ dw_plane_kernel(const Shape s, const DwPlaneCfg c, const float* __restrict__ x, 
     const uint32_t in_elems = (uint32_t)c.PB * (uint32_t)HW, out_elems = (uint32_t)c.PB * (uint32_t)OHW;
     float* const in_buf = plane_smem;                    // [2][PB * HW]
     float* const out_buf = plane_smem + 2 * in_elems;    // [2][PB * OHW]
+    const uint32_t w_elems = (uint32_t)c.PB * (K * K);
+    float* const w_buf = out_buf + 2 * out_elems;        // [2][PB * K * K]
     if (tid == 0) {
         bar_init(smem_addr(&full[0]), 1);
         bar_init(smem_addr(&full[1]), 1);
@@ -127,18 +126,40 @@ dw_plane_kernel(const Shape s, const DwPlaneCfg c, const float* __restrict__ x, 
         bar_expect_tx(bar, bytes);
         bulk_load(smem_addr(in_buf + buf * in_elems), x + (size_t)b * in_elems, bytes, bar);
     };
+    // The filters of a batch's planes: one run of the packed weights that starts over at channel 0 (16-byte copies where a multiple
+    // of four channels keeps it on 16 bytes).  Read from global memory by each unit, a warp's planes were as many lines per weight:
+    // 960 planes of 7x7 (N = 64) 10.3 -> 8.3 us with 5x5 filters, 7.8 -> 6.6 with 3x3.
+    auto stage_weights = [&](uint32_t b, uint32_t buf) {
+        if (b < c.batches) {
+            const uint32_t row = (uint32_t)s.C_in * (K * K), total = planes_of(b) * (K * K), step = (s.C_in & 3) == 0 ? 4 : 1;
+            uint32_t pq, ch;
+            c.div_c.divmod(b * (uint32_t)c.PB, pq, ch);
+            const uint32_t dst = smem_addr(w_buf + buf * w_elems);
+            for (uint32_t i = (uint32_t)tid * step; i < total; i += blockDim.x * step) {
+                uint32_t e = ch * (K * K) + i;
+                while (e >= row) e -= row;
+                if (step == 4) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 4u * i), "l"(wpk + e) : "memory");
+                else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4u * i), "l"(wpk + e) : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
     uint32_t b = blockIdx.x, it = 0;
     if (tid == 0 && b < c.batches) issue(b, 0);
+    stage_weights(b, 0);
     for (; b < c.batches; b += gridDim.x, ++it) {
         const uint32_t buf = it & 1u;
         const uint32_t nb = b + gridDim.x;
         if (tid == 0) bulk_store_wait_read<1>();         // the store that read out_buf[buf] two batches ago is done with it
         __syncthreads();                                 // ... and every thread is done with the previous batch's input
         if (tid == 0 && nb < c.batches) issue(nb, buf ^ 1u);
+        stage_weights(nb, buf ^ 1u);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");   // (this batch's weights are there; the barrier below shows them to everyone)
         const uint32_t plane0 = b * (uint32_t)c.PB;
         const int np = (int)planes_of(b);
         float* const in = in_buf + buf * in_elems;
         float* const out = out_buf + buf * out_elems;
+        const float* const w_smem = w_buf + buf * w_elems;
         const int in_tail = np * HW & 3, out_tail = np * OHW & 3;
         if (tid < in_tail) in[np * HW - in_tail + tid] = __ldg(x + (size_t)plane0 * HW + np * HW - in_tail + tid);
         // one thread polls; the others sleep in the barrier below instead of spending issue slots on the poll loop
@@ -149,15 +170,13 @@ dw_plane_kernel(const Shape s, const DwPlaneCfg c, const float* __restrict__ x, 
         }
         if constexpr (WHOLE) {
             for (int pl = tid; pl < np; pl += (int)blockDim.x) {
-                uint32_t pq, ch;
-                c.div_c.divmod(plane0 + (uint32_t)pl, pq, ch);
-                const float* __restrict__ wk = wpk + (size_t)ch * (K * K);
+                const float* __restrict__ wk = w_smem + pl * (K * K);
                 const float* __restrict__ ip = in + pl * (W * W);
                 float xin[W * W], wr[K * K], acc[W * W];
 #pragma unroll
                 for (int i = 0; i < W * W; ++i) xin[i] = ip[i];
 #pragma unroll
-                for (int i = 0; i < K * K; ++i) wr[i] = __ldg(wk + i);
+                for (int i = 0; i < K * K; ++i) wr[i] = wk[i];
 #pragma unroll
                 for (int p = 0; p < W; ++p)
 #pragma unroll
@@ -181,41 +200,47 @@ dw_plane_kernel(const Shape s, const DwPlaneCfg c, const float* __restrict__ x, 
         for (int u = tid; u < units; u += (int)blockDim.x) {
             uint32_t pl, rem;
             c.div_upp.divmod((uint32_t)u, pl, rem);
-            const int orow = (int)(rem / (uint32_t)G::NS) * G::RPU, st = (int)(rem % (uint32_t)G::NS);
-            uint32_t pq, ch;
-            c.div_c.divmod(plane0 + pl, pq, ch);
-            const float* __restrict__ wk = wpk + (size_t)ch * (K * K);
-            const float* __restrict__ ip = in + pl * (uint32_t)HW + (st * G::SW * S - G::PAD);
-            const bool first = st == 0, last = st == G::NS - 1;
+            const int orow = (int)rem * G::RPU;
+            const float* __restrict__ wk = w_smem + pl * (K * K);
+            const float* __restrict__ ip = in + pl * (uint32_t)HW;
             float wr[K][K];
 #pragma unroll
-            for (int i = 0; i < K * K; ++i) wr[i / K][i % K] = __ldg(wk + i);
-            float acc[G::RPU][G::SW];
+            for (int i = 0; i < K * K; ++i) wr[i / K][i % K] = wk[i];
+            float acc[G::RPU][G::W_OUT];
 #pragma unroll
             for (int i = 0; i < G::RPU; ++i)
 #pragma unroll
-                for (int q = 0; q < G::SW; ++q) acc[i][q] = 0.f;
+                for (int q = 0; q < G::W_OUT; ++q) acc[i][q] = 0.f;
             // input row rr of the unit is filter row rr - i*S of the unit's output row i
 #pragma unroll
             for (int rr = 0; rr < G::NR; ++rr) {
                 const int h = orow * S - G::PAD + rr;
                 if (h >= 0 && h < H) {
                     const float* __restrict__ row = ip + h * W;
-                    float win[G::WN];
+                    float v[W];
 #pragma unroll
-                    for (int j = 0; j < G::WN; ++j) {
-                        // columns left of the image exist only in a row's first strip, columns right of it only in its last
-                        const bool in_image = (j >= G::PAD || !first) && (j < G::RLIM || !last);
-                        win[j] = in_image ? row[j] : 0.f;
+                    for (int j = 0; j < W; j += G::VEC) {
+                        if constexpr (G::VEC == 4) {
+                            const float4 t = *reinterpret_cast<const float4*>(row + j);
+                            v[j] = t.x; v[j + 1] = t.y; v[j + 2] = t.z; v[j + 3] = t.w;
+                        } else if constexpr (G::VEC == 2) {
+                            const float2 t = *reinterpret_cast<const float2*>(row + j);
+                            v[j] = t.x; v[j + 1] = t.y;
+                        } else {
+                            v[j] = row[j];
+                        }
                     }
 #pragma unroll
                     for (int i = 0; i < G::RPU; ++i) {
                         const int r = rr - i * S;
                         if (r >= 0 && r < K) {
 #pragma unroll
-                            for (int q = 0; q < G::SW; ++q)
+                            for (int q = 0; q < G::W_OUT; ++q)
 #pragma unroll
-                                for (int t = 0; t < K; ++t) acc[i][q] = fmaf(win[q * S + t], wr[r][t], acc[i][q]);
+                                for (int t = 0; t < K; ++t) {
+                                    const int col = q * S + t - G::PAD;
+                                    if (col >= 0 && col < W) acc[i][q] = fmaf(v[col], wr[r][t], acc[i][q]);
+                                }
                         }
                     }
                 }
@@ -223,9 +248,17 @@ dw_plane_kernel(const Shape s, const DwPlaneCfg c, const float* __restrict__ x, 
 #pragma unroll
             for (int i = 0; i < G::RPU; ++i) {
                 if (orow + i < H_out) {
-                    float* __restrict__ op = out + pl * (uint32_t)OHW + (orow + i) * G::W_OUT + st * G::SW;
+                    float* __restrict__ op = out + pl * (uint32_t)OHW + (orow + i) * G::W_OUT;
+                    if constexpr (G::W_OUT % 4 == 0) {
 #pragma unroll
-                    for (int q = 0; q < G::SW; ++q) op[q] = acc[i][q];
+                        for (int q = 0; q < G::W_OUT; q += 4) *reinterpret_cast<float4*>(op + q) = make_float4(acc[i][q], acc[i][q + 1], acc[i][q + 2], acc[i][q + 3]);
+                    } else if constexpr (G::W_OUT % 2 == 0) {
+#pragma unroll
+                        for (int q = 0; q < G::W_OUT; q += 2) *reinterpret_cast<float2*>(op + q) = make_float2(acc[i][q], acc[i][q + 1]);
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < G::W_OUT; ++q) op[q] = acc[i][q];
+                    }
                 }
             }
         }
@@ -269,12 +302,11 @@ bool dw_plane_supported(const Shape& s) {
 DwPlaneCfg dw_plane_config(const Shape& s, int sm_count) {
     DwPlaneCfg c;
     const long long planes = (long long)s.N * s.C_in;
-    const int per_plane = s.H * s.W + s.H_out * s.W_out;
-    const int sw = s.W_out <= 8 ? s.W_out : 7;
-    const int rpu = (s.stride == 1 || s.W <= 14) ? 2 : 1;
+    const int per_plane = s.H * s.W + s.H_out * s.W_out + s.KH * s.KW;      // floats in shared memory, per buffer
+    const int rpu = rows_per_unit(s.KH, s.stride, s.W);
     const bool whole = s.W == 7 && s.H == 7 && s.stride == 1;     // a thread per plane
-    c.upp = whole ? 1 : ((s.H_out + rpu - 1) / rpu) * (s.W_out / sw);   // a unit is one strip of one (stride 1: two) output rows, or a plane
-    int pb_max = (50 * 1024) / (per_plane * 8);
+    c.upp = whole ? 1 : (s.H_out + rpu - 1) / rpu;
+    int pb_max = (54 * 1024) / (per_plane * 8);
     pb_max &= ~3;
     if (pb_max > 64) pb_max = 64;
     int best = 4;
@@ -326,7 +358,7 @@ cudaError_t dw_plane_forward(const Shape& s, const DwPlaneCfg& c, const float* x
         return launch_plane<K, S, 28>(s, c, x, pk, y, status, tag, st); \
     } while (0)
     if (s.KH == 3) {
-        if (s.stride == 1) GCONV_PLANE_W(3, 1);
+        if (s.stride == 1) GCONV_PLANE_W(3, 1);   // (28 wide: on the strips, see dw_plan)
         else GCONV_PLANE_W(3, 2);
     } else {
         if (s.stride == 1) GCONV_PLANE_W(5, 1);

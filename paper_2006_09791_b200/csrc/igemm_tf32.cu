@@ -1592,8 +1592,8 @@ static int igemm_merge(const Shape& s) {
 
 // Wide pointwise layers on planes the tiled copies cannot address (a width, or with stride 1 a pixel count, that is not a multiple of 4) read
 // a copy of x whose planes are one row each: with stride 1 the pixels as they are, with stride 2 only those the layer reads.  The planes
-// start on 16 bytes and take the same segments of 32 pixels.  (As rows of the padded width, 7x7 planes crossed in boxes of 32-byte rows and
-// in the generic instantiation, and stride 2 computed and dropped three of four pixels.)  Copy and layer, rows -> one row: 512 -> 512 @7x7
+// start on 16 bytes and take the same segments of 32 pixels.  (As rows of the padded width they all ran the generic
+// instantiation, and stride 2 computed and dropped three of four pixels.)  Copy and layer, rows -> one row: 512 -> 512 @7x7
 // N = 64 34.1 -> 15.4 us, 256 -> 512 @13x13 N = 64 40.1 -> 19.9, 192 -> 384 @29x29 N = 41 55.6 -> 31.4, 256 -> 128 @25x25 N = 13 25.8 -> 11.1.
 // The planes are those that had a padded copy before; groups that merge to 32 channels at most, up to 32 wide, are gathered without one.
 static bool pw_one_row(const Shape& s) {

@@ -35,9 +35,10 @@ def test_depthwise_strips(cfg):
 
 BATCHES = [  # N, C, H, W, filter, stride: enough small planes for batches in shared memory; N * C and H * W leave a short last batch
     # whose floats end 1, 2 or 3 past a multiple of four, one plane in the last batch, whole batches only
-    (1, 2049, 7, 7, 3, 1), (1, 2051, 7, 7, 5, 1), (3, 1367, 5, 7, 3, 1), (64, 64, 7, 7, 5, 1), (11, 2235, 7, 7, 3, 2), (2, 1087, 7, 7, 5, 2),
-    (9, 1367, 14, 14, 3, 1), (7, 1888, 13, 14, 3, 2), (1, 6151, 14, 14, 5, 1), (5, 1231, 14, 14, 5, 2), (1, 4251, 27, 28, 5, 1),
-    (2, 8197, 28, 28, 5, 2), (3, 5667, 27, 28, 3, 2),
+    # (filters copied one by one), one plane in the last batch, whole batches only, fewer channels than a batch has planes
+    (1, 2049, 7, 7, 3, 1), (1, 6151, 7, 7, 5, 1), (3, 1367, 5, 7, 3, 1), (97, 64, 7, 7, 5, 1), (11, 2235, 7, 7, 3, 2), (3, 4099, 7, 7, 5, 2),
+    (9, 1367, 14, 14, 3, 1), (7, 1999, 13, 14, 3, 2), (1, 6151, 14, 14, 5, 1), (5, 1231, 14, 14, 5, 2), (1, 4251, 27, 28, 5, 1),
+    (1, 6149, 28, 28, 5, 2), (3, 5667, 27, 28, 3, 2), (2100, 3, 7, 7, 5, 1), (1600, 4, 7, 7, 3, 1), (2500, 1, 14, 14, 5, 1),
 ]
 
 
