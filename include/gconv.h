@@ -58,9 +58,9 @@ enum gconv_status {
  * max|y - y_ref| / max|y_ref| <= 1e-5 for the FP32 variants, <= 5e-3 for the TF32 variant. */
 enum gconv_variant_id {
     GCONV_VARIANT_AUTO = 0,           /* let the selector choose (default) */
-    GCONV_VARIANT_DIRECT_GENERIC = 1, /* FP32 FFMA, one thread per output, any shape */
-    GCONV_VARIANT_DIRECT_TILED = 2,   /* FP32 FFMA, shared-memory halo + register tiles; 3x3, dilation 1, narrow groups;
-                                         depthwise 3x3 (pad 1) and 5x5 (pad 2) on a software-pipelined stream kernel */
+    GCONV_VARIANT_DIRECT_GENERIC = 1, /* FP32 FFMA, any shape: staged register tiles */
+    GCONV_VARIANT_DIRECT_TILED = 2,   /* FP32 FFMA, 3x3, dilation 1: register tiles; depthwise 3x3 (pad 1) and 5x5
+                                         (pad 2) on streams of row strips or batches of small planes */
     GCONV_VARIANT_IGEMM_TF32 = 3      /* TF32 tcgen05 implicit GEMM per (merged) group; 3x3 with pad = dilation or 1x1 with pad 0,
                                          stride 1 or 2 (per axis: gconv_desc_create_2d), W <= 128; dilation > 1 only with
                                          stride 1 on planes whose (padded) rows divide 32 pixels */
