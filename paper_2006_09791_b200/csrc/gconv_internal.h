@@ -260,6 +260,7 @@ struct IgemmLaunchOpts {
 };
 bool igemm_supported(const Shape& s);
 IgemmCfg igemm_config(const Shape& s, int sm_count);
+bool igemm_runnable(const Shape& s, int C2, int sm_count);   // an instantiation takes the configuration (holds for every supported shape; tests)
 size_t igemm_packed_bytes(const Shape& s);
 uint32_t igemm_layout_tag(const Shape& s);    // equal tags: weights packed for one shape serve the other
 cudaError_t igemm_pack(const Shape& s, const float* w, void* packed, cudaStream_t st);

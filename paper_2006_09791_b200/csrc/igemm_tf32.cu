@@ -395,6 +395,13 @@ static bool family_matches(int f, const Shape& s, const IgemmCfg& c) {
     if (fam.stride >= 0 && s.stride != fam.stride) return false;
     return s.dilation == 1;          // every family fixes dilation 1; dilated layers run the generic instantiation
 }
+// The instantiation that runs a configuration, or -1: the generic one (0) has no code for pair tiles, split channels or the 29 warps
+// of the gather producer's one-CTA shape.  (`fast4` has to be what the launch uses; the gather families leave it open.)
+static int instantiation(const Shape& s, const IgemmCfg& c) {
+    for (int f = 1; f < kFamilies; ++f)
+        if (family_matches(f, s, c)) return f;
+    return c.spl || c.pair || (c.soft && c.egroups == 2) ? -1 : 0;
+}
 
 __device__ __forceinline__ void
 igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& s, const IgemmCfg& c,
@@ -1948,7 +1955,7 @@ static bool gather_config(IgemmCfg& out, const Shape& st, int sm_count, bool sin
         break;
     }
     if (heavy && !c.b_res) split_channels(c);
-    if (heavy && (c.stages < 2 || (mode == 2 && !c.pair && !c.spl))) return false;
+    if (heavy && c.stages < 2) return false;
     c.raw_off = bank + (uint32_t)c.stages * c.stage_bytes;
     c.xchg_off = c.raw_off + (uint32_t)c.raw_stages * c.raw_bytes;
     c.smem_bytes = (size_t)c.xchg_off + 1024;
@@ -1969,6 +1976,8 @@ static bool gather_config(IgemmCfg& out, const Shape& st, int sm_count, bool sin
         if (c.cps > c.MT) c.cps = c.MT;
         c.grid = c.cps * c.n_gn;
     }
+    // (wide stride-2 groups with one pixel tile each have 8-channel stages and no pair: nothing runs those, split or not)
+    if (instantiation(st, c) < 0) return false;
     out = c;
     return true;
 }
@@ -2402,6 +2411,34 @@ struct IgemmPlan {
     IgemmPlan* next;
 };
 
+// Which second tensor map a configuration copies whole tiles with (IgemmCfg::fast4 once it is encoded): 0 none, 1 raw parts of the gather
+// producer, row boxes or runs of pixels, 2 segments of the plane.
+static int whole_tile_map(const Shape& s, const IgemmCfg& c) {
+    if (c.soft) return c.raw_bulk ? 0 : 1;
+    if (c.rowbox) return 1;
+    if (c.nr == 3 && !c.tapb && (c.flat ? c.flat_in : s.H * s.W) % 32 == 0) return 2;
+    return !c.tapb && c.seg_fstep == 32 && (!c.seg_mode || c.SPI % 4 == 0 || c.flat) ? 1 : 0;   // (flat planes: tiles inside one image)
+}
+
+// The problem as the kernel sees it: the padded plane, the re-cut pointwise plane, the even rows of a stride-2 pointwise layer.
+static Shape kernel_shape(const Shape& s_true, const IgemmCfg& c) {
+    Shape s = as_3x3(s_true);
+    if (c.padded) {
+        const IgemmGeom ge = igemm_geom(s_true);
+        s.H = ge.Hp;
+        s.W = ge.Wp;
+    }
+    if (c.row_skip) s.H = s.H_out;
+    return s;
+}
+
+bool igemm_runnable(const Shape& s, int C2, int sm_count) {
+    IgemmCfg c = igemm_config_c2(s, sm_count, C2);
+    const Shape ks = kernel_shape(s, c);
+    c.fast4 = whole_tile_map(ks, c);
+    return instantiation(ks, c) >= 0 && c.smem_bytes <= (size_t)kMaxDynSmem && c.grid >= 1 && c.stages >= 1;
+}
+
 static cudaError_t make_plan(IgemmPlan& p, const Shape& s_true, int sm_count, const float* x) {
     p.cfg = igemm_config_c2(s_true, sm_count, p.C2);
     const IgemmCfg c = p.cfg;
@@ -2472,7 +2509,7 @@ static cudaError_t make_plan(IgemmPlan& p, const Shape& s_true, int sm_count, co
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
         cfg.fast4 = 1;   // the second map is in use (prefetch it)
-    } else if (c.nr == 3 && !c.tapb && HW % 32 == 0) {
+    } else if (whole_tile_map(p.s, c) == 2) {
         // Halo stages of segment or flat-row tiles: (pixel in segment, channel, segment of the plane, image).  The box
         // starts wseg segments before the tile; segments before or after the plane are out of range and read as zeros,
         // so the first and last tiles of a plane are whole boxes too.
@@ -2486,7 +2523,7 @@ static cudaError_t make_plan(IgemmPlan& p, const Shape& s_true, int sm_count, co
             cfg.fast4 = 2;
         else
             xmap4 = xmap;
-    } else if (!c.tapb && c.seg_fstep == 32 && (!c.seg_mode || c.SPI % 4 == 0 || c.flat)) {   // (flat planes: tiles inside one image)
+    } else if (whole_tile_map(p.s, c) == 1) {
         const cuuint64_t dims4[4] = {HW, (cuuint64_t)s.C_in, 8, (cuuint64_t)s.N};
         const cuuint64_t strides4[3] = {HW * 4, 128, HW * 4 * (cuuint64_t)s.C_in};
         const cuuint32_t box4[4] = {32, (cuuint32_t)c.CK, (cuuint32_t)c.nseg, 1};
@@ -2499,12 +2536,8 @@ static cudaError_t make_plan(IgemmPlan& p, const Shape& s_true, int sm_count, co
             xmap4 = xmap;
     }
     p.use_map4 = cfg.fast4 != 0;
-    int fam = 0;
-    for (int f = 1; f < kFamilies && fam == 0; ++f)
-        if (family_matches(f, s, cfg)) fam = f;
-    if (cfg.spl && family(fam).spl != 1) return cudaErrorInvalidValue;     // nor split-channel code
-    if (cfg.pair && family(fam).pair != 1) return cudaErrorInvalidValue;   // the generic instantiation has no pair-tile code
-    if (cfg.soft && cfg.egroups == 2 && family(fam).soft != cfg.soft) return cudaErrorInvalidValue;   // 29 warps: only the wide-group gather instantiations take them
+    const int fam = instantiation(s, cfg);
+    if (fam < 0) return cudaErrorInvalidValue;
     p.kernel = kernels[fam];
     return cudaFuncSetAttribute(p.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
 }

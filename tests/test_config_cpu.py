@@ -1,0 +1,61 @@
+"""The host side's choices, without a GPU: every shape the tensor-core variant takes has a kernel that runs its configuration."""
+import math
+import os
+import random
+import subprocess
+
+import pytest
+
+from paper_2006_09791_b200 import build as gbuild
+from paper_2006_09791_b200 import gconv
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def probe(tmp_path_factory):
+    lib = gbuild.build()
+    exe = str(tmp_path_factory.mktemp("probe") / "config_probe")
+    subprocess.check_call([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-o", exe, os.path.join(HERE, "config_probe.cu"), lib,
+                           "-Xlinker", "-rpath=" + os.path.dirname(lib)])
+
+    def run(shapes):
+        out = subprocess.run([exe], input="\n".join(" ".join(str(v) for v in s) for s in shapes), capture_output=True, text=True, check=True)
+        rows = [tuple(int(v) for v in line.split()) if line != "refused" else None for line in out.stdout.splitlines()]
+        assert len(rows) == len(shapes)
+        return rows
+
+    return run
+
+
+def _square(N, Ci, H, W, Co, k, stride, g, pad=None):
+    p = k // 2 if pad is None else pad
+    return (N, Ci, H, W, Co, k, k, stride, stride, p, p, 1, 1, g)
+
+
+def _drawn(count, seed=11):
+    """Shapes around the tensor-core variant's range: pointwise and 3x3, both strides, all alignments, few tiles and many."""
+    rng = random.Random(seed)
+
+    def log_int(lo, hi):
+        return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
+
+    for _ in range(count):
+        H = log_int(4, 130)
+        W = H if rng.random() < 0.4 else log_int(4, 128)
+        cg = rng.choice([2, 4, 8, 12, 16, 24, 32, 40, 48, 64, 72, 96, 128, 192, 256, 320, 512])
+        kg = rng.choice([cg, cg, 2 * cg, 4 * cg, 8, 16, 32, 64, 128, 256, 512])
+        g = rng.choice([1, 1, 2, 3, 4, 6, 8, 16, 32])
+        yield _square(log_int(1, 256), g * cg, H, W, g * kg, rng.choice([3, 3, 1]), rng.choice([1, 1, 2]), g)
+
+
+# stride 2 on odd planes, wide groups, one pixel tile each and more (group, filter tile) pairs than count as few
+ONE_TILE = [(2, 64, 7, 7, 256, 4), (1, 64, 9, 9, 256, 4), (2, 32, 9, 9, 256, 2), (1, 128, 7, 7, 512, 8), (2, 256, 10, 10, 1024, 8)]
+
+
+def test_every_supported_shape_has_a_kernel(probe):
+    shapes = [_square(N, Ci, H, W, Co, 3, 2, g) for N, Ci, H, W, Co, g in ONE_TILE] + list(_drawn(60000))
+    rows = probe(shapes)
+    assert sum(r is not None and r[0] == gconv.GCONV_VARIANT_IGEMM_TF32 for r in rows) > 20000
+    bad = [s for s, r in zip(shapes, rows) if r is not None and r[1] != 1]
+    assert not bad, (len(bad), bad[:5])

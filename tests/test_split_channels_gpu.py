@@ -40,6 +40,14 @@ def test_split_channels(cfg):
     assert used == gconv.GCONV_VARIANT_IGEMM_TF32
 
 
+# stride 2 on odd planes, wide groups, one pixel tile each, more than fifteen (group, filter tile) pairs: the padded copy's row tiles
+@pytest.mark.parametrize("cfg", [(2, 64, 7, 7, 256, 4), (1, 64, 9, 9, 256, 4), (2, 32, 9, 9, 256, 2), (1, 128, 7, 7, 512, 8), (2, 256, 10, 10, 1024, 8)])
+def test_one_tile_wide_groups_stride_2(cfg):
+    N, Ci, H, W, Co, g = cfg
+    err, used = check_layer(Layer("one_tile", N, Ci, H, W, Co, stride=2, groups=g), seed=78)
+    assert used == gconv.GCONV_VARIANT_IGEMM_TF32
+
+
 def test_split_channels_back_to_back():
     """Dependent launches: the next kernel's clusters start while this one's still exchange partial sums."""
     L = Layer("chain", 2, 256, 13, 13, 256)
