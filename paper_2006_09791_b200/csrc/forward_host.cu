@@ -35,6 +35,7 @@ static int g_lane_users = 0;         // descriptors with a HostPipe
 // What a descriptor keeps: how its batch is cut.
 struct HostPipe {
     int parts, images;               // parts the batch is cut into (0: not cut), images of each but the last
+    size_t workspace;                // bytes the whole batch needs; a part needs no more
     gconv_desc* part[2];             // descriptors of `images` images and of the last, shorter part
 };
 
@@ -121,7 +122,8 @@ void free_host_pipe(gconv_desc* d) {
     }
 }
 
-// A descriptor of the same layer with n images that runs on weights packed for `d`, or nullptr.
+// A descriptor of the same layer with n images that runs on weights packed for `d` and in the workspace the caller attaches for `d`
+// (the tiling follows the batch: a shorter one may need the padded copy where the whole one does not), or nullptr.
 static gconv_desc* part_of(gconv_desc* d, int n) {
     const Shape& s = d->s;
     gconv_desc* c = nullptr;
@@ -129,16 +131,18 @@ static gconv_desc* part_of(gconv_desc* d, int n) {
                              s.groups) != GCONV_OK)
         return nullptr;
     if (gconv_desc_set_variant(c, d->variant) != GCONV_OK ||
-        (d->variant == GCONV_VARIANT_IGEMM_TF32 && igemm_layout_tag(c->s) != igemm_layout_tag(s))) {
+        (d->variant == GCONV_VARIANT_IGEMM_TF32 && igemm_layout_tag(c->s) != igemm_layout_tag(s)) ||
+        gconv_workspace_bytes(c) > gconv_workspace_bytes(d)) {
         gconv_desc_destroy(c);
         return nullptr;
     }
     return c;
 }
 
-// Cuts the batch: as many parts as the size allows, fewer where the packed layout of a shorter batch differs.
+// Cuts the batch: as many parts as the size allows, fewer where the packed layout or the workspace of a shorter batch differs.
 static void cut(gconv_desc* d, HostPipe* p, size_t xb, size_t yb) {
     const Shape& s = d->s;
+    p->workspace = gconv_workspace_bytes(d);
     const size_t most = (xb < yb ? xb : yb) / kPartBytes;
     // parts start on 16-byte boundaries of x and y
     const bool odd = ((size_t)s.C_in * s.H * s.W) % 4 != 0 || ((size_t)s.C_out * s.H_out * s.W_out) % 4 != 0;
@@ -207,7 +211,7 @@ extern "C" int gconv_forward_host(gconv_desc_t d, const float* x_host, const voi
         cut(d, fresh, xb, yb);
     }
     HostPipe* p = d->host_pipe;
-    if (p->parts == 0) return in_order();
+    if (p->parts == 0 || d->workspace_bytes < p->workspace) return in_order();   // (gconv_forward reports a missing workspace)
     for (int i = 0; i < 2; ++i) {
         gconv_desc* c = p->part[i];
         if (c == nullptr) continue;
@@ -216,7 +220,6 @@ extern "C" int gconv_forward_host(gconv_desc_t d, const float* x_host, const voi
         c->workspace = d->workspace;               // the parts' kernels follow each other on the caller's stream
         c->workspace_bytes = d->workspace_bytes;
         c->wait_us = d->wait_us;
-        if (gconv_workspace_bytes(c) > c->workspace_bytes) return GCONV_ERR_WORKSPACE;
     }
     Lane* l = take_lane(d->device, st);
     if (l == nullptr) return in_order();

@@ -53,7 +53,9 @@ class _Host:
 
 @pytest.mark.parametrize("cfg", [(64, 64, 28, 28, 64, 3, 1, 8), (37, 64, 32, 32, 64, 3, 1, 2), (61, 60, 15, 15, 60, 3, 1, 60), (50, 64, 13, 13, 64, 3, 2, 1),
                                  (33, 128, 10, 54, 128, 3, 1, 4), (40, 16, 30, 31, 16, 5, 1, 2), (2, 64, 112, 112, 64, 3, 1, 4),
-                                 (1, 64, 112, 112, 64, 3, 1, 4), (128, 32, 8, 8, 32, 3, 1, 4), (64, 128, 56, 56, 32, 1, 1, 1)])
+                                 (1, 64, 112, 112, 64, 3, 1, 4), (128, 32, 8, 8, 32, 3, 1, 4), (64, 128, 56, 56, 32, 1, 1, 1),
+                                 # no workspace for the whole batch, one for a shorter part
+                                 (103, 64, 19, 19, 256, 3, 1, 8), (88, 192, 19, 19, 512, 3, 1, 4)])
 def test_host_parts(cfg):
     L = _Host(*cfg)
     try:
