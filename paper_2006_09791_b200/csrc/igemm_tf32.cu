@@ -2022,7 +2022,9 @@ static IgemmCfg igemm_config_c2(const Shape& s_any, int sm_count, int C2) {
     // times, or the bank has to be streamed anyway: 512 -> 512 @14x14 N = 64 28.4 -> 21.3 us, 512 -> 256 @28x28 48.7 -> 42.1,
     // 384 -> 192 @32x32 40.6 -> 29.0, 256 -> 512 @56x56 stride 2 86.5 -> 67.0, 128 -> 512 @28x28 35.2 -> 32.0.  128 -> 256 @56x56 loses
     // (two resident 64 KB banks, one per set of CTAs: 52.8; one of 128 KB: 57.6).
-    const int kt_max = !c.pw ? 64 : ((c.Cg >= 192 || c.Kg >= 512) ? 256 : 128);
+    // (128 at most where the gather producer takes the layer: two accumulators in 256 columns, and no workspace)
+    const bool gathered = c.Cg <= 32 && s_true.W % 4 != 0 && s_true.W_out <= 32;
+    const int kt_max = !c.pw ? 64 : (!gathered && (c.Cg >= 192 || c.Kg >= 512) ? 256 : 128);
     int kt = c.Kg <= kt_max ? c.Kg : kt_max;
     while (c.Kg % kt != 0 || kt % 8 != 0) kt -= 8;   // largest multiple of 8 dividing Kg, at most 64 (pointwise: 128 or 256)
     if (c.pw) {

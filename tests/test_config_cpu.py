@@ -59,3 +59,10 @@ def test_every_supported_shape_has_a_kernel(probe):
     assert sum(r is not None and r[0] == gconv.GCONV_VARIANT_IGEMM_TF32 for r in rows) > 20000
     bad = [s for s, r in zip(shapes, rows) if r is not None and r[1] != 1]
     assert not bad, (len(bad), bad[:5])
+
+
+def test_gathered_pointwise_layers_need_no_workspace(probe):
+    """Narrow groups with many filters on planes the tiled copies cannot address: the gather producer, whatever the filter tile."""
+    shapes = [_square(31, 128, 7, 7, 2048, 1, 1, 4), _square(14, 512, 7, 3, 8192, 1, 1, 16), _square(23, 48, 117, 7, 1024, 1, 2, 2),
+              _square(19, 72, 195, 2, 1536, 1, 1, 3), _square(64, 32, 14, 14, 512, 1, 2, 1)]
+    assert [(r[0], r[2]) for r in probe(shapes)] == [(gconv.GCONV_VARIANT_IGEMM_TF32, 0)] * len(shapes)

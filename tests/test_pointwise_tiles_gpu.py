@@ -51,3 +51,13 @@ ONE_ROW = [  # N, C_in, H, W, C_out, stride, groups: planes copied to one row ea
 @pytest.mark.parametrize("cfg", ONE_ROW)
 def test_pointwise_planes_of_one_row(cfg):
     test_pointwise_tiles(cfg)
+
+
+# narrow groups with 512 filters and more on such planes: the gather producer's tiles of at most 128 filters, no workspace
+@pytest.mark.parametrize("cfg", [(5, 128, 7, 7, 2048, 1, 4), (3, 64, 7, 3, 1024, 1, 2), (2, 48, 17, 7, 1024, 2, 2), (4, 32, 14, 14, 512, 2, 1)])
+def test_gathered_pointwise_planes(cfg):
+    N, C, H, W, K, stride, g = cfg
+    d = gconv.gconv_desc_create(N, C, H, W, K, 1, 1, stride, 0, 1, g)
+    assert gconv.gconv_workspace_bytes(d) == 0
+    gconv.gconv_desc_destroy(d)
+    test_pointwise_tiles(cfg)
