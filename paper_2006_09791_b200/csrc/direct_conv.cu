@@ -276,8 +276,11 @@ bool conv_geometry(const Shape& s, ConvCfg& c, int TW) {
     c.PH = (int)ph;
     c.PW = (int)pw;
     c.vec = (s.stride_w == 1 && s.W % 4 == 0) ? 1 : 0;
-    c.phase = c.vec ? ((c.PW + 3 + 3) & ~3) : (c.PW + s.stride_w - 1) / s.stride_w;
-    c.pitch = c.phase * s.stride_w;
+    // (a row is whole column phases: with a stride beyond the patch's width it is far longer than the patch)
+    const long long phase = c.vec ? ((pw + 3 + 3) & ~3) : (pw + s.stride_w - 1) / s.stride_w, pitch = phase * s.stride_w;
+    if (pitch > kSmemMax / 4 || c.NI * ph * pitch > kSmemMax / 4) return false;
+    c.phase = (int)phase;
+    c.pitch = (int)pitch;
     c.plane = c.PH * c.pitch;
     c.wvec = (s.Kg % 4 == 0 && BM % 4 == 0) ? 1 : 0;
     const long long per_channel = 4LL * ((long long)c.NI * c.plane + (long long)taps * BM);
@@ -368,7 +371,7 @@ bool conv_config(const Shape& s, int sm_count, ConvCfg& best) {
                 for (int wn = 1; wn * wm <= 8; wn *= 2) {
                     if (wm * wn < 2) continue;
                     const int BN = 32 * tn * wn;
-                    if (wn > 1 && BN / 2 >= s.N * s.H_out * s.W_out) break;      // half of the tile would already hold everything
+                    if (wn > 1 && BN / 2 >= (long long)s.N * s.H_out * s.W_out) break;      // half of the tile would already hold everything
                     ConvCfg c;
                     c.TM = tm; c.TN = tn; c.WM = wm; c.WN = wn;
                     int last_tw = 0;

@@ -1,4 +1,5 @@
-"""The host side's choices, without a GPU: every shape the tensor-core variant takes has a kernel that runs its configuration."""
+"""The host side's choices, without a GPU: every shape the tensor-core variant takes has a kernel that runs its configuration, and the
+staged FP32 kernel's buffers hold what it puts there."""
 import math
 import os
 import random
@@ -66,3 +67,25 @@ def test_gathered_pointwise_layers_need_no_workspace(probe):
     shapes = [_square(31, 128, 7, 7, 2048, 1, 1, 4), _square(14, 512, 7, 3, 8192, 1, 1, 16), _square(23, 48, 117, 7, 1024, 1, 2, 2),
               _square(19, 72, 195, 2, 1536, 1, 1, 3), _square(64, 32, 14, 14, 512, 1, 2, 1)]
     assert [(r[0], r[2]) for r in probe(shapes)] == [(gconv.GCONV_VARIANT_IGEMM_TF32, 0)] * len(shapes)
+
+
+def test_staged_fp32_buffers_in_64_bits(probe):
+    """Column strides up to 2^31 - 1: a staged row is whole column phases, however few columns of it the patch has."""
+    huge = [(1, 1, 5000, 1, 1, 3, 1, 1, 3000000, 0, 0, 1, 1, 1), (1, 1, 8, 1, 1, 4, 1, 1, 1 << 30, 0, 0, 1, 1, 1), (2, 8, 30, 5, 8, 3, 3, 1, 2147483647, 1, 1, 1, 1, 1),
+            (1, 4, 40, 3, 4, 3, 3, 2, 2147483646, 0, 0, 1, 1, 2), (1, 2, 9, 200000, 2, 3, 3, 1, 70000, 1, 1, 1, 1, 1), (3, 4, 64, 7, 4, 5, 7, 1, 65536, 2, 0, 1, 1, 4)]
+    rng = random.Random(3)
+    drawn = []
+    while len(drawn) < 1500:
+        sw = int(math.exp(rng.uniform(0, math.log(2.0 ** 31 - 1))))
+        kh, kw, W = rng.randint(1, 9), rng.randint(1, 9), rng.choice([1, 3, 4, 7, 12, 28, 33, 224, 3000])
+        pw = rng.randint(0, 4)
+        if W + 2 * pw >= kw:
+            g = rng.choice([1, 2, 4])
+            drawn.append((rng.randint(1, 40), g * rng.randint(1, 9), rng.choice([9, 16, 33, 500]), W, g * rng.randint(1, 20), kh, kw, rng.choice([1, 1, 2, 3]),
+                          sw if rng.random() < 0.7 else rng.randint(1, 4), rng.randint(0, 4), pw, 1, 1, g))
+    rows = probe(huge + drawn)
+    bad = [s for s, r in zip(huge + drawn, rows) if r is None or r[3] == 0]
+    assert not bad, (len(bad), bad[:5])
+    assert sum(r[3] == 1 for r in rows) > 700, sum(r[3] == 1 for r in rows)
+    # more output pixels than 31 bits count: still staged
+    assert probe([(70000, 1, 180, 180, 1, 7, 7, 1, 1, 3, 3, 1, 1, 1)])[0][3] == 1

@@ -34,6 +34,9 @@ CASES = [  # N, C_in, H, W, C_out, (filter), (stride), (pad), (dilation), groups
     (2, 48, 28, 28, 48, (7, 1), (2, 1), (3, 0), (1, 1), 3),
     # no tile holds a patch of this dilation: the one-thread-per-output kernel
     (1, 2, 560, 560, 3, (3, 3), (1, 1), (0, 0), (270, 270), 1), (1, 2, 40, 40, 2, (35, 35), (1, 1), (17, 17), (1, 1), 2),
+    # column strides far beyond the width: whole column phases of a staged row would be millions of columns
+    (1, 1, 5000, 1, 1, (3, 1), (1, 3000000), (0, 0), (1, 1), 1), (2, 8, 30, 5, 8, (3, 3), (1, 2147483647), (1, 1), (1, 1), 1),
+    (2, 6, 9, 40, 4, (3, 3), (2, 50), (1, 1), (1, 1), 2),
 ]
 
 
