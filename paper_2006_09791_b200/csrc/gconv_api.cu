@@ -289,8 +289,8 @@ int gconv_block_pack_weights(gconv_desc_t d, int C2, const float* w_ochw, const 
 int gconv_block_forward(gconv_desc_t d, int C2, const float* x, const void* w_packed, float* y2, void* stream) {
     if (d == nullptr || x == nullptr || w_packed == nullptr || y2 == nullptr) return GCONV_ERR_NULL;
     if (!aligned16(x) || !aligned16(w_packed) || !aligned16(y2)) return GCONV_ERR_ALIGNMENT;
-    // (a plan exists for supported pairs only)
-    if (!igemm_has_plan(d->plans, C2) && !igemm_block_supported(d->s, C2)) return GCONV_ERR_UNSUPPORTED;
+    // (a plan exists for supported pairs only; under 0 stands the plain convolution's)
+    if (C2 < 1 || (!igemm_has_plan(d->plans, C2) && !igemm_block_supported(d->s, C2))) return GCONV_ERR_UNSUPPORTED;
     int rc = ensure_device_state(d);
     if (rc != GCONV_OK) return rc;
     cudaError_t e = cudaSuccess;

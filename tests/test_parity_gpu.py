@@ -624,6 +624,28 @@ def test_fused_block_rejects_what_it_cannot_run():
             gconv.gconv_desc_destroy(d)
 
 
+def test_fused_block_without_pointwise_outputs_is_refused():
+    """C2 = 0 (and below) is refused, also once the descriptor has run the plain convolution: y2 stays untouched."""
+    L = Layer("block0", 2, 32, 16, 16, 32, groups=4)
+    dev = torch.device("cuda:0")
+    x, w = synth.make_layer_tensors(L.N, L.C_in, L.H, L.W, L.C_out, 3, 3, L.groups, 6)
+    d = gconv.gconv_desc_create(*L.desc_args())
+    try:
+        wp = torch.empty(gconv.gconv_packed_bytes(d) // 4, dtype=torch.float32, device=dev)
+        xd, y = torch.from_numpy(x).to(dev), torch.empty(L.y_elems, dtype=torch.float32, device=dev)
+        y2 = torch.full((L.y_elems,), 7.0, dtype=torch.float32, device=dev)
+        gconv.gconv_pack_weights(d, torch.from_numpy(w).to(dev), wp)
+        for _ in range(2):
+            for C2 in (0, -1, -16):
+                with pytest.raises(gconv.GconvError) as e:
+                    gconv.gconv_block_forward(d, C2, xd, wp, y2)
+                assert e.value.status == gconv.GCONV_ERR_UNSUPPORTED
+            gconv.gconv_forward(d, xd, wp, y)
+        assert gconv.gconv_last_status(d) == gconv.GCONV_OK and bool((y2 == 7.0).all())
+    finally:
+        gconv.gconv_desc_destroy(d)
+
+
 def test_pack_mismatch_is_reported_not_fatal():
     (L,) = config0()
     x, w = synth.make_layer_tensors(L.N, L.C_in, L.H, L.W, L.C_out, 3, 3, L.groups, 5)
