@@ -183,9 +183,11 @@ extern "C" int gconv_forward_host(gconv_desc_t d, const float* x_host, const voi
         e = cudaMemcpyAsync(y_host, y_stage, yb, cudaMemcpyDeviceToHost, st);
         return e == cudaSuccess ? GCONV_OK : fail_cuda(d, e);
     };
-    // One image, or little to move: nothing to overlap.  A stream that is being captured keeps the plain order (the side streams
+    // One image, or little to move: nothing to overlap.  Host buffers that share memory (y in the place of x): a part's copy out would
+    // reach the next parts' input before it has been read.  A stream that is being captured keeps the plain order (the side streams
     // would belong to the capture until it ends, and other threads may be using them).
-    if (s.N < 2 || (xb < yb ? xb : yb) < 2 * kPartBytes || d->dbg_skip >= 0) return in_order();
+    const uintptr_t xh = reinterpret_cast<uintptr_t>(x_host), yh = reinterpret_cast<uintptr_t>(y_host);
+    if (s.N < 2 || (xb < yb ? xb : yb) < 2 * kPartBytes || (xh < yh + yb && yh < xh + xb) || d->dbg_skip >= 0) return in_order();
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
         (void)cudaGetLastError();

@@ -69,6 +69,25 @@ def test_host_parts(cfg):
         L.close()
 
 
+@pytest.mark.parametrize("cfg,shift", [((64, 32, 56, 56, 128, 3, 1, 4), 0), ((64, 64, 56, 56, 64, 3, 1, 4), -1000), ((64, 64, 56, 56, 64, 3, 1, 4), 1 << 20)])
+def test_host_buffers_that_share_memory(cfg, shift):
+    """y in the place of x, before it and behind it: the whole input is read before any output is written."""
+    L = _Host(*cfg)
+    try:
+        s = torch.cuda.Stream()
+        at_x, at_y = max(0, -shift), max(0, shift)
+        both = torch.empty(max(at_x + L.xh.numel(), at_y + L.want.size)).pin_memory()
+        x, y = both[at_x:at_x + L.xh.numel()], both[at_y:at_y + L.want.size]
+        torch.cuda.synchronize()
+        for _ in range(3):
+            x.copy_(L.xh.view(-1))
+            gconv.gconv_forward_host(L.d, x, L.wp, y, L.xs, L.ys, s)
+            assert gconv.gconv_last_status(L.d, s) == gconv.GCONV_OK
+            L.check(y.view(L.want.shape))
+    finally:
+        L.close()
+
+
 def test_host_parts_from_several_threads_and_in_a_graph():
     L = _Host(48, 64, 32, 32, 64, 3, 1, 4)
     other = [(torch.empty_like(L.xs), torch.empty_like(L.ys)) for _ in range(2)]
