@@ -130,7 +130,8 @@ int gconv_desc_set_variant(gconv_desc_t desc, int variant);
  *   w_ochw    device, fp32 [C_out, Cg, KH, KW], read only.
  *   w_packed  device, gconv_packed_bytes(desc) bytes, written.  The blob is position independent
  *             and may be copied, saved and reloaded.
- * One kernel launch on `stream`.  Errors: GCONV_ERR_NULL, GCONV_ERR_ALIGNMENT, GCONV_ERR_CUDA.
+ * One kernel launch on `stream` (FP32 variants: the header is cleared before it).  Errors: GCONV_ERR_NULL, GCONV_ERR_ALIGNMENT,
+ * GCONV_ERR_CUDA.
  */
 int gconv_pack_weights(gconv_desc_t desc, const float *w_ochw, void *w_packed, void *stream);
 

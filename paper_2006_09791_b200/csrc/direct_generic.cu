@@ -12,7 +12,7 @@ size_t generic_packed_bytes(const Shape& s) {
 }
 
 cudaError_t generic_pack(const Shape& s, const float* w, void* packed, cudaStream_t st) {
-    return group_pack(s, w, packed, generic_tag(s), st);
+    return group_pack(s, w, packed, generic_tag(s), true, st);
 }
 
 // The tag names the layout as well as the shape (a blob packed as a plain OIHW copy by an earlier build is refused).
@@ -22,7 +22,7 @@ __global__ void __launch_bounds__(256)
 generic_forward_kernel(Shape s, const float* __restrict__ x, const uint32_t* __restrict__ packed,
                        float* __restrict__ y, Status* status, uint32_t tag) {
     dependent_start();
-    if (packed[0] != tag) {
+    if (packed[0] != tag && packed[0] != (tag ^ kNonFiniteMark)) {
         if (threadIdx.x == 0) record_status(status, GCONV_ERR_PACK_MISMATCH, (int)blockIdx.x);
         return;
     }

@@ -7,14 +7,11 @@ namespace gconv {
 
 namespace {
 
-__global__ void group_pack_kernel(Shape s, const float* __restrict__ w, uint32_t* __restrict__ packed, uint32_t tag) {
+__global__ void group_pack_kernel(Shape s, const float* __restrict__ w, uint32_t* __restrict__ packed, uint32_t tag, bool mark) {
     const int taps = s.KH * s.KW;
     const size_t n = (size_t)s.C_out * s.Cg * taps;
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) {
-        packed[0] = tag;
-        for (int j = 1; j < kHeaderBytes / 4; ++j) packed[j] = 0;
-    }
+    if (i == 0) atomicXor(packed, tag);                     // (the header is zeros; any block may add the mark)
     float* dst = reinterpret_cast<float*>(packed + kHeaderBytes / 4);
     for (; i < n; i += (size_t)gridDim.x * blockDim.x) {
         // destination index i = (((g*Cg + c)*taps + rs)*Kg + k)
@@ -24,17 +21,22 @@ __global__ void group_pack_kernel(Shape s, const float* __restrict__ w, uint32_t
         t /= taps;
         const int c = (int)(t % s.Cg);
         const int g = (int)(t / s.Cg);
-        dst[i] = w[(((size_t)g * s.Kg + k) * s.Cg + c) * taps + rs];
+        const float v = w[(((size_t)g * s.Kg + k) * s.Cg + c) * taps + rs];
+        dst[i] = v;
+        if (mark && !isfinite(v) && atomicExch(packed + 1, 1u) == 0u) atomicXor(packed, kNonFiniteMark);
     }
 }
 
 }  // namespace
 
-// Weights as [g][c][r][s][Kg] behind the header (the filters of one tap are one vector load).
-cudaError_t group_pack(const Shape& s, const float* w, void* packed, uint32_t tag, cudaStream_t st) {
+// Weights as [g][c][r][s][Kg] behind the header (the filters of one tap are one vector load).  `mark`: weights that are infinite or not a
+// number are marked in the tag (the staged kernel leaves its main path for them; the depthwise and row kernels take them as they are).
+cudaError_t group_pack(const Shape& s, const float* w, void* packed, uint32_t tag, bool mark, cudaStream_t st) {
     const size_t n = (size_t)s.C_out * s.Cg * s.KH * s.KW;
     const int blocks = (int)((n + 255) / 256 < 1184 ? (n + 255) / 256 : 1184);
-    group_pack_kernel<<<blocks, 256, 0, st>>>(s, w, reinterpret_cast<uint32_t*>(packed), tag);
+    const cudaError_t e = cudaMemsetAsync(packed, 0, kHeaderBytes, st);
+    if (e != cudaSuccess) return e;
+    group_pack_kernel<<<blocks, 256, 0, st>>>(s, w, reinterpret_cast<uint32_t*>(packed), tag, mark);
     return cudaGetLastError();
 }
 
@@ -49,7 +51,7 @@ bool tiled_takes_conv(const Shape& s) { return !dw_supported(s) && !rows_support
 size_t tiled_packed_bytes(const Shape& s) { return kHeaderBytes + sizeof(float) * (size_t)s.C_out * s.Cg * s.KH * s.KW; }
 
 cudaError_t tiled_pack(const Shape& s, const float* w, void* packed, cudaStream_t st) {
-    return group_pack(s, w, packed, pack_tag(s, GCONV_VARIANT_DIRECT_TILED), st);
+    return group_pack(s, w, packed, pack_tag(s, GCONV_VARIANT_DIRECT_TILED), tiled_takes_conv(s), st);
 }
 
 cudaError_t tiled_forward(const Shape& s, const ConvCfg* conv, const DwPlan& dw, const float* x, const void* packed, float* y, Status* status,

@@ -91,6 +91,7 @@ struct gconv_desc {
 namespace gconv {
 
 constexpr int kHeaderBytes = 64;  // packed-weight blob header; keeps the payload 16-byte aligned
+constexpr uint32_t kNonFiniteMark = 0x80000000u;  // in the tag of a blob for the staged FP32 kernel: some weight is infinite or not a number
 constexpr uint32_t kMagic = 0x47434e56u;  // "GCNV"
 
 // Device status block: word 0 = first error recorded by a kernel (0 = none), word 1 = detail.
@@ -194,7 +195,7 @@ cudaError_t dw_forward(const Shape& s, const DwPlan& plan, const float* x, const
 bool tiled_supported(const Shape& s);
 bool tiled_takes_conv(const Shape& s);   // neither depthwise nor narrow groups: the staged kernel
 size_t tiled_packed_bytes(const Shape& s);
-cudaError_t group_pack(const Shape& s, const float* w, void* packed, uint32_t tag, cudaStream_t st);
+cudaError_t group_pack(const Shape& s, const float* w, void* packed, uint32_t tag, bool mark, cudaStream_t st);
 cudaError_t tiled_pack(const Shape& s, const float* w, void* packed, cudaStream_t st);
 cudaError_t tiled_forward(const Shape& s, const ConvCfg* conv, const DwPlan& dw, const float* x, const void* packed, float* y, Status* status,
                           int sm_count, const Launch& st);

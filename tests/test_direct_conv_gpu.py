@@ -62,3 +62,31 @@ def test_staged_fp32_kernel(cfg):
         assert rel_err(got, ref) <= 1e-5          # FP32 sums of at most 4608 products: 2^-24 x sqrt(4608) is 4e-6
     finally:
         gconv.gconv_desc_destroy(d)
+
+
+@pytest.mark.parametrize("cfg", [(2, 3, 29, 37, 20, (7, 7), (2, 2), (3, 3), (1, 1), 1), (3, 250, 2, 2, 96, (3, 3), (1, 1), (1, 1), (1, 1), 1),
+                                 (2, 8, 20, 28, 17, (3, 5), (1, 1), (2, 4), (2, 2), 1), (9, 72, 3, 5, 40, (5, 5), (1, 1), (2, 2), (1, 1), 2)])
+def test_weights_that_are_not_finite(cfg):
+    """Taps outside the image are left out, whatever their weight; packing finite weights into the same buffer afterwards is as ever."""
+    N, C_in, H, W, C_out, k, st, pd, dl, g = cfg
+    dev = torch.device("cuda:0")
+    x, w = synth.make_layer_tensors(N, C_in, H, W, C_out, k[0], k[1], g, 17)
+    x[x == 0] = 0.5
+    bad = w.copy()
+    bad[0, 0, 0, 0], bad[1, -1, -1, -1], bad[C_out - 1, 0, 0, -1] = np.inf, -np.inf, np.nan
+    d = gconv.gconv_desc_create_2d(N, C_in, H, W, C_out, k[0], k[1], st[0], st[1], pd[0], pd[1], dl[0], dl[1], g)
+    try:
+        gconv.gconv_desc_set_variant(d, gconv.GCONV_VARIANT_DIRECT_GENERIC)
+        Ho, Wo = gconv.gconv_out_shape(d)
+        wp = torch.empty(gconv.gconv_packed_bytes(d) // 4, dtype=torch.float32, device=dev)
+        for weights in (bad, w):
+            y = torch.empty(N, C_out, Ho, Wo, device=dev)
+            gconv.gconv_pack_weights(d, torch.from_numpy(weights).to(dev), wp)
+            gconv.gconv_forward(d, torch.from_numpy(x).to(dev), wp, y)
+            assert gconv.gconv_last_status(d) == gconv.GCONV_OK
+            ref, got = oracle.gconv_ref(x, weights, st, pd, dl, g, threads=oracle.max_threads()), y.cpu().numpy().astype(np.float64)
+            fin = np.isfinite(ref)
+            assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(got[np.isinf(ref)], ref[np.isinf(ref)])
+            assert 0 < fin.sum() and rel_err(got[fin], ref[fin]) <= 1e-5
+    finally:
+        gconv.gconv_desc_destroy(d)
