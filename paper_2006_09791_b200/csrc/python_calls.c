@@ -2,9 +2,11 @@
  *
  * A forward of a small layer takes the GPU 2 to 3 us, and marshalling its five arguments through ctypes took the host
  * 1.8 us of every call (0.2 us per tensor for data_ptr() and the conversion, the argument array, the foreign call).  The
- * functions here do the same -- an argument is None, an integer, or an object with data_ptr() (stream: cuda_stream) -- and
- * call the library through the addresses that gconv.py hands over when it loads libgconv.so.  A status other than GCONV_OK
- * goes to gconv.py's `_check`, which raises.  The interpreter lock is released during the call, as ctypes does.
+ * functions here do the same for the usual arguments -- a descriptor and a C2 that are integers, tensors and a stream that are
+ * None, an integer, or an object with data_ptr() (stream: cuda_stream) -- and call the library through the addresses that
+ * gconv.py hands over when it loads libgconv.so.  Everything else, wrong arguments included, goes to gconv.py's own function
+ * of the same name, so both accept and refuse the same.  A status other than GCONV_OK goes to gconv.py's `_check`, which
+ * raises.  The interpreter lock is released during the call, as ctypes does.
  */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
@@ -17,8 +19,9 @@ typedef int (*host_fn)(void *, const void *, const void *, void *, void *, void 
 static forward_fn f_forward;
 static block_fn f_block;
 static host_fn f_host;
-static PyObject *s_data_ptr, *s_cuda_stream, *o_load, *o_check;
+static PyObject *s_data_ptr, *s_cuda_stream, *o_load, *o_check, *o_own[3];   /* o_own: gconv.py's functions, in the order of bind() */
 
+/* None, an integer, or -- `attr` given -- what an object's method (`call`) or attribute of that name gives; 0: none of these */
 static int to_pointer(PyObject *o, PyObject *attr, int call, void **out) {
     if (o == Py_None) {
         *out = NULL;
@@ -26,49 +29,39 @@ static int to_pointer(PyObject *o, PyObject *attr, int call, void **out) {
     }
     PyObject *v = NULL;
     if (!PyLong_Check(o)) {
+        if (attr == NULL) return 0;
         v = call ? PyObject_CallMethodNoArgs(o, attr) : PyObject_GetAttr(o, attr);
-        if (v == NULL) return 0;
+        if (v == NULL || !PyLong_Check(v)) {
+            Py_XDECREF(v);
+            PyErr_Clear();                   /* (gconv.py's function raises it again) */
+            return 0;
+        }
         o = v;
     }
-    const unsigned long long a = PyLong_AsUnsignedLongLongMask(o);
+    *out = (void *)(uintptr_t)PyLong_AsUnsignedLongLongMask(o);
     Py_XDECREF(v);
-    if (a == (unsigned long long)-1 && PyErr_Occurred()) return 0;
-    *out = (void *)(uintptr_t)a;
     return 1;
 }
 
-/* positional and keyword arguments into out[0 .. count), borrowed; the last one defaults to None */
-static int take(const char *name, const char *const *names, int count, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames, PyObject **out) {
-    if (nargs == count && kwnames == NULL) {
-        for (int i = 0; i < count; ++i) out[i] = args[i];
-        return 1;
-    }
-    if (nargs > count) {
-        PyErr_Format(PyExc_TypeError, "%s() takes %d arguments but %zd were given", name, count, nargs);
-        return 0;
-    }
+/* positional and keyword arguments into out[0 .. count), borrowed; the last one defaults to None; 0: they do not fit */
+static int take(const char *const *names, int count, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames, PyObject **out) {
+    if (nargs > count) return 0;
     for (int i = 0; i < count; ++i) out[i] = i < nargs ? args[i] : NULL;
     const Py_ssize_t nkw = kwnames ? PyTuple_GET_SIZE(kwnames) : 0;
     for (Py_ssize_t k = 0; k < nkw; ++k) {
         PyObject *kw = PyTuple_GET_ITEM(kwnames, k);
         int i = 0;
         while (i < count && PyUnicode_CompareWithASCIIString(kw, names[i]) != 0) ++i;
-        if (i == count || out[i] != NULL) {
-            PyErr_Format(PyExc_TypeError, "%s() got %s argument '%U'", name, i == count ? "an unexpected keyword" : "multiple values for", kw);
-            return 0;
-        }
+        if (i == count || out[i] != NULL) return 0;
         out[i] = args[nargs + k];
     }
-    for (int i = 0; i < count; ++i) {
-        if (out[i] != NULL) continue;
-        if (i != count - 1) {
-            PyErr_Format(PyExc_TypeError, "%s() missing required argument: '%s'", name, names[i]);
-            return 0;
-        }
-        out[i] = Py_None;
-    }
+    for (int i = 0; i < count - 1; ++i)
+        if (out[i] == NULL) return 0;
+    if (out[count - 1] == NULL) out[count - 1] = Py_None;
     return 1;
 }
+
+static PyObject *own(int which, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames) { return PyObject_Vectorcall(o_own[which], args, nargs, kwnames); }
 
 static int loaded(void) {
     if (f_forward != NULL) return 1;
@@ -87,11 +80,10 @@ static PyObject *py_forward(PyObject *self, PyObject *const *args, Py_ssize_t na
     static const char *const names[] = {"desc", "x_nchw", "w_packed", "y_nchw", "stream"};
     PyObject *a[5];
     void *p[5];
-    int rc;
-    if (!take("gconv_forward", names, 5, args, nargs, kwnames, a) || !loaded()) return NULL;
-    for (int i = 0; i < 4; ++i)
-        if (!to_pointer(a[i], s_data_ptr, 1, &p[i])) return NULL;
-    if (!to_pointer(a[4], s_cuda_stream, 0, &p[4])) return NULL;
+    int rc, ok = take(names, 5, args, nargs, kwnames, a);
+    for (int i = 0; ok && i < 4; ++i) ok = to_pointer(a[i], i > 0 ? s_data_ptr : NULL, 1, &p[i]);
+    if (!ok || !to_pointer(a[4], s_cuda_stream, 0, &p[4])) return own(0, args, nargs, kwnames);
+    if (!loaded()) return NULL;
     Py_BEGIN_ALLOW_THREADS
     rc = f_forward(p[0], p[1], p[2], p[3], p[4]);
     Py_END_ALLOW_THREADS
@@ -102,16 +94,13 @@ static PyObject *py_block(PyObject *self, PyObject *const *args, Py_ssize_t narg
     static const char *const names[] = {"desc", "C2", "x_nchw", "w_packed", "y2_nchw", "stream"};
     PyObject *a[6];
     void *p[6];
-    int rc;
-    if (!take("gconv_block_forward", names, 6, args, nargs, kwnames, a) || !loaded()) return NULL;
-    if (!to_pointer(a[0], s_data_ptr, 1, &p[0])) return NULL;
-    const long c2 = PyLong_AsLong(a[1]);
-    if (c2 == -1 && PyErr_Occurred()) return NULL;
-    for (int i = 2; i < 5; ++i)
-        if (!to_pointer(a[i], s_data_ptr, 1, &p[i])) return NULL;
-    if (!to_pointer(a[5], s_cuda_stream, 0, &p[5])) return NULL;
+    int rc, ok = take(names, 6, args, nargs, kwnames, a) && PyLong_Check(a[1]) && to_pointer(a[0], NULL, 0, &p[0]);
+    for (int i = 2; ok && i < 5; ++i) ok = to_pointer(a[i], s_data_ptr, 1, &p[i]);
+    if (!ok || !to_pointer(a[5], s_cuda_stream, 0, &p[5])) return own(1, args, nargs, kwnames);
+    const int c2 = (int)PyLong_AsUnsignedLongLongMask(a[1]);
+    if (!loaded()) return NULL;
     Py_BEGIN_ALLOW_THREADS
-    rc = f_block(p[0], (int)c2, p[2], p[3], p[4], p[5]);
+    rc = f_block(p[0], c2, p[2], p[3], p[4], p[5]);
     Py_END_ALLOW_THREADS
     return finish(rc, "gconv_block_forward");
 }
@@ -120,25 +109,24 @@ static PyObject *py_host(PyObject *self, PyObject *const *args, Py_ssize_t nargs
     static const char *const names[] = {"desc", "x_host", "w_packed", "y_host", "x_stage", "y_stage", "stream"};
     PyObject *a[7];
     void *p[7];
-    int rc;
-    if (!take("gconv_forward_host", names, 7, args, nargs, kwnames, a) || !loaded()) return NULL;
-    for (int i = 0; i < 6; ++i)
-        if (!to_pointer(a[i], s_data_ptr, 1, &p[i])) return NULL;
-    if (!to_pointer(a[6], s_cuda_stream, 0, &p[6])) return NULL;
+    int rc, ok = take(names, 7, args, nargs, kwnames, a);
+    for (int i = 0; ok && i < 6; ++i) ok = to_pointer(a[i], i > 0 ? s_data_ptr : NULL, 1, &p[i]);
+    if (!ok || !to_pointer(a[6], s_cuda_stream, 0, &p[6])) return own(2, args, nargs, kwnames);
+    if (!loaded()) return NULL;
     Py_BEGIN_ALLOW_THREADS
     rc = f_host(p[0], p[1], p[2], p[3], p[4], p[5], p[6]);
     Py_END_ALLOW_THREADS
     return finish(rc, "gconv_forward_host");
 }
 
-/* setup(load, check): the functions that open the library and turn a status into an exception */
+/* setup(load, check, forward, block_forward, forward_host): the functions that open the library and turn a status into an
+ * exception, and gconv.py's own functions */
 static PyObject *py_setup(PyObject *self, PyObject *args) {
-    PyObject *load, *check;
-    if (!PyArg_ParseTuple(args, "OO", &load, &check)) return NULL;
-    Py_INCREF(load);
-    Py_INCREF(check);
-    Py_XSETREF(o_load, load);
-    Py_XSETREF(o_check, check);
+    PyObject *load, *check, *o[3];
+    if (!PyArg_ParseTuple(args, "OOOOO", &load, &check, &o[0], &o[1], &o[2])) return NULL;
+    Py_XSETREF(o_load, Py_NewRef(load));
+    Py_XSETREF(o_check, Py_NewRef(check));
+    for (int i = 0; i < 3; ++i) Py_XSETREF(o_own[i], Py_NewRef(o[i]));
     Py_RETURN_NONE;
 }
 

@@ -246,8 +246,9 @@ def gconv_last_status_detail(desc) -> int:
     return int(load().gconv_last_status_detail(desc))
 
 
+_BY_CTYPES = (gconv_forward, gconv_block_forward, gconv_forward_host)
 if _calls is not None:       # same names, arguments and results
-    _calls.setup(load, _check)
+    _calls.setup(load, _check, *_BY_CTYPES)
     gconv_forward = _calls.gconv_forward
     gconv_block_forward = _calls.gconv_block_forward
     gconv_forward_host = _calls.gconv_forward_host

@@ -1,5 +1,6 @@
 """Host-side checks of the C ABI that need no GPU: the library loads, exports every symbol the
 header declares, validates descriptors and reports shapes/MACs."""
+import ctypes
 import os
 import re
 
@@ -152,3 +153,72 @@ def test_workspace_is_caller_owned_and_rarely_needed():
     assert lib.gconv_desc_set_workspace(None, 0, 0) == gconv.GCONV_ERR_NULL
     assert lib.gconv_desc_set_debug(None, 0, -1) == gconv.GCONV_ERR_NULL
     assert "workspace" in gconv.status_string(gconv.GCONV_ERR_WORKSPACE)
+
+
+class _At:
+    def __init__(self, p):
+        self.p = p
+
+    def data_ptr(self):
+        return self.p
+
+    @property
+    def cuda_stream(self):
+        return self.p
+
+
+class _Broken:
+    def data_ptr(self):
+        raise ValueError("no pointer")
+
+
+def test_native_calls_take_and_refuse_what_ctypes_does():
+    """Every form of argument, right and wrong, has the same outcome through the C call module as through ctypes (no call gets past the
+    library's argument checks: a pointer is always missing or misaligned)."""
+    assert gconv._calls is not None and gconv.gconv_forward is not gconv._BY_CTYPES[0]
+    d = gconv.gconv_desc_create(1, 32, 8, 8, 32, 3, 3, 1, 1, 1, 4)
+
+    def outcome(fn, args, kw):
+        try:
+            fn(*args, **kw)
+            return "returned"
+        except gconv.GconvError as e:
+            return ("status", e.status)
+        except Exception as e:      # noqa: BLE001
+            return type(e).__name__
+
+    handles = [d, ctypes.c_void_p(d), None, _At(16), _Broken(), "16", 1.0, [d], d + (1 << 64)]
+    pointers = [None, 4, _At(4), _At(16), _At(4.0), _At("4"), _At(None), _Broken(), "4", 4.0, ctypes.c_void_p(4), -4, 4 + (1 << 70), True]
+    c2s = [32, 32.0, "32", None, _At(32), 32 + (1 << 64), -32, 1 << 40]
+    try:
+        seen = set()
+
+        def same(k, args, kw):
+            a, b = outcome(gconv._BY_CTYPES[k], args, kw), outcome((gconv.gconv_forward, gconv.gconv_block_forward, gconv.gconv_forward_host)[k], args, kw)
+            assert a == b and a != "returned", (k, args, kw, a, b)
+            seen.add(a)
+
+        for h in handles:
+            same(0, (h, None, 16, 16), {})
+            same(1, (h, 32, None, 16, 16), {})
+            same(2, (h, None, 16, 16, 16, 16), {})
+            same(0, (), {"desc": h, "x_nchw": None, "w_packed": 16, "y_nchw": 16})
+        for p in pointers:
+            for i in range(3):
+                args = [16, 16, 4]
+                args[i] = p
+                same(0, (d, *args), {})
+                same(1, (d, 32, *args), {})
+            for i in range(4):
+                args = [16, 16, 16, 16, None]           # (no y_stage)
+                args[i] = p
+                same(2, (d, *args), {})
+            same(0, (d, 16, 16, 4, p), {})
+            same(0, (d, 16, 16), {"y_nchw": 4, "stream": p})
+        for c in c2s:
+            same(1, (d, c, 16, 16, 4), {})
+        for args, kw in (((), {}), ((d,), {}), ((d, 16, 16, 4, None, None), {}), ((d, 16, 16, 4), {"desc": d}), ((d, 16, 16, 4), {"strm": None}), ((d, 16), {"y_nchw": 4})):
+            same(0, args, kw)
+        assert {"ArgumentError", "TypeError", "AttributeError", "ValueError"} <= seen, seen
+    finally:
+        gconv.gconv_desc_destroy(d)
