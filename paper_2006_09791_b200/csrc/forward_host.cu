@@ -34,6 +34,7 @@ static int g_lane_users = 0;         // descriptors with a HostPipe
 
 // What a descriptor keeps: how its batch is cut.
 struct HostPipe {
+    int variant;                     // the descriptor's when it was cut
     int parts, images;               // parts the batch is cut into (0: not cut), images of each but the last
     size_t workspace;                // bytes the whole batch needs; a part needs no more
     gconv_desc* part[2];             // descriptors of `images` images and of the last, shorter part
@@ -142,6 +143,7 @@ static gconv_desc* part_of(gconv_desc* d, int n) {
 // Cuts the batch: as many parts as the size allows, fewer where the packed layout or the workspace of a shorter batch differs.
 static void cut(gconv_desc* d, HostPipe* p, size_t xb, size_t yb) {
     const Shape& s = d->s;
+    p->variant = d->variant;
     p->workspace = gconv_workspace_bytes(d);
     const size_t most = (xb < yb ? xb : yb) / kPartBytes;
     // parts start on 16-byte boundaries of x and y
@@ -164,6 +166,23 @@ static void cut(gconv_desc* d, HostPipe* p, size_t xb, size_t yb) {
         p->part[1] = b;
         return;
     }
+}
+
+// Parts the batch of `d` is cut into, 0 if it is not cut; decided once for a variant (another one's layout may allow other parts).
+int host_parts(gconv_desc* d) {
+    if (d->host_pipe != nullptr && d->host_pipe->variant != d->variant) free_host_pipe(d);
+    if (d->host_pipe == nullptr) {
+        HostPipe* fresh = new (std::nothrow) HostPipe();
+        if (fresh == nullptr) return 0;
+        {
+            std::lock_guard<std::mutex> lanes(g_lane_mutex);
+            ++g_lane_users;
+        }
+        d->host_pipe = fresh;
+        const Shape& s = d->s;
+        cut(d, fresh, sizeof(float) * (size_t)s.N * s.C_in * s.H * s.W, sizeof(float) * (size_t)s.N * s.C_out * s.H_out * s.W_out);
+    }
+    return d->host_pipe->parts;
 }
 
 }  // namespace gconv
@@ -201,19 +220,8 @@ extern "C" int gconv_forward_host(gconv_desc_t d, const float* x_host, const voi
 
     // The lock covers the whole enqueue: the part descriptors are this descriptor's.
     std::lock_guard<std::mutex> lock(d->host_mutex);
-    if (d->host_pipe != nullptr && d->host_pipe->parts > 0 && d->host_pipe->part[0]->variant != d->variant) free_host_pipe(d);
-    if (d->host_pipe == nullptr) {
-        HostPipe* fresh = new (std::nothrow) HostPipe();
-        if (fresh == nullptr) return in_order();
-        {
-            std::lock_guard<std::mutex> lanes(g_lane_mutex);
-            ++g_lane_users;
-        }
-        d->host_pipe = fresh;
-        cut(d, fresh, xb, yb);
-    }
+    if (host_parts(d) == 0 || d->workspace_bytes < d->host_pipe->workspace) return in_order();   // (gconv_forward reports a missing workspace)
     HostPipe* p = d->host_pipe;
-    if (p->parts == 0 || d->workspace_bytes < p->workspace) return in_order();   // (gconv_forward reports a missing workspace)
     for (int i = 0; i < 2; ++i) {
         gconv_desc* c = p->part[i];
         if (c == nullptr) continue;

@@ -160,7 +160,8 @@ inline cudaError_t launch_kernel(unsigned grid, unsigned block, size_t smem, con
 int ensure_device_state(gconv_desc* d);
 int launch_forward(gconv_desc* d, const float* x, const void* packed, float* y, Status* status, cudaStream_t st, bool may_overlap);
 int fail_cuda(gconv_desc* d, cudaError_t e);
-void free_host_pipe(gconv_desc* d);     // forward_host.cu
+int host_parts(gconv_desc* d);          // forward_host.cu
+void free_host_pipe(gconv_desc* d);
 
 size_t generic_packed_bytes(const Shape& s);
 uint32_t generic_tag(const Shape& s);

@@ -1,6 +1,7 @@
 // Reads descriptors (one per line: N C_in H W C_out KH KW stride_h stride_w pad_h pad_w dilation_h dilation_w groups) and prints what the
 // library's host code makes of each: the variant, whether an instantiation runs its configuration, the workspace, and for the staged FP32
-// kernel whether its shared memory holds what the kernel puts there (-1: the one-thread-per-output kernel runs).  Host code only.
+// kernel whether its shared memory holds what the kernel puts there (-1: the one-thread-per-output kernel runs), the parts a batch of host
+// buffers is cut into, and those after the descriptor has been set to the generic variant.  Host code only.
 #include <stdio.h>
 
 #include "../paper_2006_09791_b200/csrc/gconv_internal.h"
@@ -30,7 +31,10 @@ int main() {
         const bool tc = gconv::igemm_supported(d->s);
         gconv::ConvCfg c;
         const int staged = gconv::conv_config(d->s, 148, c) ? staging_fits(d->s, c) : -1;
-        printf("%d %d %zu %d\n", d->variant, !tc || gconv::igemm_runnable(d->s, 0, 148) ? 1 : 0, tc ? gconv::igemm_scratch_bytes(d->s) : (size_t)0, staged);
+        const int variant = d->variant, parts = gconv::host_parts(d);
+        gconv_desc_set_variant(d, GCONV_VARIANT_DIRECT_GENERIC);
+        printf("%d %d %zu %d %d %d\n", variant, !tc || gconv::igemm_runnable(d->s, 0, 148) ? 1 : 0, tc ? gconv::igemm_scratch_bytes(d->s) : (size_t)0, staged, parts,
+               gconv::host_parts(d));
         gconv_desc_destroy(d);
     }
 }

@@ -89,3 +89,9 @@ def test_staged_fp32_buffers_in_64_bits(probe):
     assert sum(r[3] == 1 for r in rows) > 700, sum(r[3] == 1 for r in rows)
     # more output pixels than 31 bits count: still staged
     assert probe([(70000, 1, 180, 180, 1, 7, 7, 1, 1, 3, 3, 1, 1, 1)])[0][3] == 1
+
+
+def test_host_batches_are_cut_for_the_variant_that_runs(probe):
+    """A batch whose tensor-core layout allows no parts is cut once the descriptor runs the generic variant."""
+    rows = probe([_square(8, 576, 16, 16, 2304, 1, 1, 3), _square(92, 6144, 20, 20, 512, 3, 1, 32), _square(27, 384, 42, 42, 32, 3, 1, 2)])
+    assert [r[4] for r in rows] == [0, 0, 0] and [r[5] for r in rows] == [4, 5, 5]
