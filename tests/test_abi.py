@@ -3,6 +3,7 @@ header declares, validates descriptors and reports shapes/MACs."""
 import ctypes
 import os
 import re
+import sysconfig
 
 import pytest
 
@@ -153,6 +154,18 @@ def test_workspace_is_caller_owned_and_rarely_needed():
     assert lib.gconv_desc_set_workspace(None, 0, 0) == gconv.GCONV_ERR_NULL
     assert lib.gconv_desc_set_debug(None, 0, -1) == gconv.GCONV_ERR_NULL
     assert "workspace" in gconv.status_string(gconv.GCONV_ERR_WORKSPACE)
+
+
+def test_library_builds_without_the_call_module(monkeypatch, tmp_path, capsys):
+    """A machine without a C compiler gets libgconv.so and a message (calls then go through ctypes); the module's name carries the
+    Python it was built for."""
+    suffix = sysconfig.get_config_var("EXT_SUFFIX")
+    assert os.path.basename(gbuild.CALLS) == "_calls" + suffix and os.path.exists(gbuild.CALLS)
+    monkeypatch.setattr(gbuild, "CALLS", str(tmp_path / ("_calls" + suffix)))
+    for cc in ("/nonexistent/cc", "/bin/false"):
+        monkeypatch.setenv("CC", cc)
+        assert gbuild.build() == gbuild.LIB and os.path.exists(gbuild.LIB)
+        assert "not built" in capsys.readouterr().err and not os.listdir(tmp_path)
 
 
 class _At:
