@@ -10,13 +10,10 @@ device memory and streams; this module accepts raw integer pointers or anything 
 from __future__ import annotations
 
 import ctypes
+import importlib
 import os
 
-try:
-    from . import _calls
-except ImportError:          # not built yet (a fresh checkout): the ctypes functions below are used as they are
-    _calls = None
-
+_calls = None                # the C call module, once it is in use
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libgconv.so")
 _lib = None
 
@@ -97,6 +94,8 @@ def load() -> ctypes.CDLL:
             fn = getattr(lib, name)
             fn.restype = res
             fn.argtypes = args
+        if _calls is None:
+            _use_native_calls()
         if _calls is not None:
             _calls.bind(*(ctypes.cast(getattr(lib, name), _vp).value for name in _NATIVE_CALLS))
         _lib = lib
@@ -247,8 +246,20 @@ def gconv_last_status_detail(desc) -> int:
 
 
 _BY_CTYPES = (gconv_forward, gconv_block_forward, gconv_forward_host)
-if _calls is not None:       # same names, arguments and results
-    _calls.setup(load, _check, *_BY_CTYPES)
-    gconv_forward = _calls.gconv_forward
-    gconv_block_forward = _calls.gconv_block_forward
-    gconv_forward_host = _calls.gconv_forward_host
+
+
+def _use_native_calls() -> None:
+    """The hot calls through the C module: same names, arguments and results.  Not built (a fresh checkout; tried again when the library is
+    loaded) or built from other sources than these: the ctypes functions above stay."""
+    global _calls, gconv_forward, gconv_block_forward, gconv_forward_host
+    importlib.invalidate_caches()
+    try:
+        from . import _calls as module
+        module.setup(load, _check, *_BY_CTYPES)
+    except (ImportError, TypeError):
+        return
+    _calls = module
+    gconv_forward, gconv_block_forward, gconv_forward_host = module.gconv_forward, module.gconv_block_forward, module.gconv_forward_host
+
+
+_use_native_calls()

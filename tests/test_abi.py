@@ -3,6 +3,9 @@ header declares, validates descriptors and reports shapes/MACs."""
 import ctypes
 import os
 import re
+import shutil
+import subprocess
+import sys
 import sysconfig
 
 import pytest
@@ -166,6 +169,22 @@ def test_library_builds_without_the_call_module(monkeypatch, tmp_path, capsys):
         monkeypatch.setenv("CC", cc)
         assert gbuild.build() == gbuild.LIB and os.path.exists(gbuild.LIB)
         assert "not built" in capsys.readouterr().err and not os.listdir(tmp_path)
+
+
+def test_call_module_of_other_sources_or_built_later(tmp_path):
+    """A call module whose interface is another one is left alone; one that appears after the import is in use once the library is."""
+    pkg = tmp_path / "paper_2006_09791_b200"
+    pkg.mkdir()
+    for name in ("__init__.py", "gconv.py"):
+        shutil.copy(os.path.join(gbuild.PKG, name), pkg / name)
+    os.symlink(gbuild.LIB, pkg / "libgconv.so")
+    (pkg / "_calls.py").write_text("def setup(load, check):\n    pass\n")
+    check = "from paper_2006_09791_b200 import gconv; assert gconv._calls is None; gconv.load(); assert gconv.gconv_forward is gconv._BY_CTYPES[0]"
+    subprocess.run([sys.executable, "-c", check], cwd=tmp_path, check=True)
+    os.remove(pkg / "_calls.py")
+    check = ("import shutil; from paper_2006_09791_b200 import gconv; assert gconv._calls is None; shutil.copy(%r, %r); gconv.load(); "
+             "assert gconv._calls is not None and gconv.gconv_forward is gconv._calls.gconv_forward" % (gbuild.CALLS, str(pkg)))
+    subprocess.run([sys.executable, "-c", check], cwd=tmp_path, check=True)
 
 
 class _At:
