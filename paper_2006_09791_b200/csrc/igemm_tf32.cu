@@ -1428,10 +1428,10 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&ctl.tmem_empty[buf]));
             if (c.fuse) {
-                if (lane == 0) mbar_arrive(smem_u32(&ctl.a2_full[egroup]));
+                const bool last_gn = (int)gn + 1 == c.n_gn;   // the pixel tile's pointwise result is complete once the MMAs requested here are done
+                if (lane == 0 && (c.d2_bufs == 2 || !last_gn)) mbar_arrive(smem_u32(&ctl.a2_full[egroup]));   // (else below, after the wait)
                 ++a2_uses;
                 float* y2_tile = y + ((size_t)n * c.C2 + (size_t)c2beg) * OHW + fo;
-                const bool last_gn = (int)gn + 1 == c.n_gn;   // the pixel tile's pointwise result is complete once the MMAs just requested are done
                 if (c.d2_bufs == 2) {
                     // each accumulator's phases are seen in order by one group: group p % 2 when n_gn is odd, else the second
                     if (pend) {
@@ -1446,12 +1446,16 @@ igemm_tf32_body(const CUtensorMap& xmap, const CUtensorMap& xmap4, const Shape& 
                         ++ptiles;
                     }
                 } else if (last_gn) {
-                    // one accumulator, both groups wait on the same barrier: a parity wait is only meaningful one phase at
-                    // a time, so first observe, in order, the phases of the pixel tiles the other group finished
+                    // One accumulator, both groups wait on the same barrier: a parity wait is only meaningful one phase at a time, so
+                    // observe, in order, the phases of the pixel tiles the other group finished -- and only then hand over this tile's
+                    // A2: its own phase cannot complete before.  (Handed over first, short pointwise MMAs (8 channels) completed that phase
+                    // before a warp held up in between looked for the earlier one, and its wait ran out.)
                     bool ok2 = true;
                     for (; d2_seen < ptiles && ok2; ++d2_seen)
                         ok2 = mbar_wait_warp(smem_u32(&ctl.d2_full[0]), d2_seen & 1u, abort_flag, status, 941);
-                    if (!ok2 || !epilogue2(0u, d2_seen & 1u, y2_tile, valid)) break;
+                    if (!ok2) break;
+                    if (lane == 0) mbar_arrive(smem_u32(&ctl.a2_full[egroup]));
+                    if (!epilogue2(0u, d2_seen & 1u, y2_tile, valid)) break;
                     ++d2_seen;
                     ++ptiles;
                 }

@@ -612,6 +612,37 @@ def test_fused_grouped_pointwise_block(cfg):
         gconv.gconv_desc_destroy(d)
 
 
+@pytest.mark.parametrize("cfg", [(138, 24, 57, 28, 3, 256), (64, 24, 32, 32, 3, 256), (40, 8, 56, 56, 1, 256), (33, 40, 20, 24, 5, 240), (50, 72, 16, 16, 9, 256)])
+def test_fused_block_with_one_pointwise_accumulator(cfg):
+    """So many pointwise outputs that one accumulator fills TMEM, an odd number of groups (the two epilogue groups take turns at finishing a
+    pixel tile) and groups so narrow that its MMAs take less than a warp's delay: many tiles a CTA, many launches."""
+    N, C, H, W, groups, C2 = cfg
+    L = Layer("block1", N, C, H, W, C, groups=groups)
+    dev = torch.device("cuda:0")
+    x, w = synth.make_layer_tensors(N, C, H, W, C, 3, 3, groups, synth.layer_seed(43, N, C, groups))
+    _, w2 = synth.make_layer_tensors(1, C, 1, 1, C2, 1, 1, 1, synth.layer_seed(44, C, C2))
+    d = gconv.gconv_desc_create(*L.desc_args())
+    try:
+        assert gconv.gconv_block_supported(d, C2)
+        wp = torch.empty(gconv.gconv_block_packed_bytes(d, C2) // 4, dtype=torch.float32, device=dev)
+        gconv.gconv_block_pack_weights(d, C2, torch.from_numpy(w).to(dev), torch.from_numpy(w2.reshape(C2, C)).to(dev), wp)
+        xd = torch.from_numpy(x).to(dev)
+        first = None
+        for _ in range(20):
+            y2 = torch.full((N, C2, H, W), float("nan"), dtype=torch.float32, device=dev)
+            gconv.gconv_block_forward(d, C2, xd, wp, y2)
+            assert gconv.gconv_last_status(d) == gconv.GCONV_OK
+            assert first is None or torch.equal(y2, first)
+            first = y2
+        n = min(N, 2)                                          # (whole images; the last one too)
+        for part in (slice(0, n), slice(N - 1, N)):
+            y1 = oracle.gconv_ref(x[part], w, 1, 1, 1, groups, threads=oracle.max_threads())
+            ref = oracle.gconv_ref(y1.astype(np.float32), w2, 1, 0, 1, 1, threads=oracle.max_threads())
+            assert rel_err(first[part].cpu().numpy(), ref) <= 5e-3
+    finally:
+        gconv.gconv_desc_destroy(d)
+
+
 def test_fused_block_rejects_what_it_cannot_run():
     for cfg, C2 in (((1, 32, 32, 32, 32, 3, 3, 2, 1, 1, 4), 32), ((1, 32, 14, 14, 32, 3, 3, 1, 1, 1, 4), 32),
                     ((1, 32, 32, 32, 32, 3, 3, 1, 1, 1, 4), 24), ((1, 256, 28, 28, 256, 3, 3, 1, 1, 1, 32), 256),
