@@ -8,10 +8,10 @@ is cycled between two uses of the same buffer (more than the 126 MB L2).
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--quick]
 
-Prints ONE JSON line.  `value` is GFLOP/s (2*MACs of Eq. (2) of the paper per second) with inputs
+Prints ONE short JSON line.  `value` is GFLOP/s (2*MACs of Eq. (2) of the paper per second) with inputs
 resident in HBM, the step replayed as a CUDA graph; `e2e` is the same metric through
-gconv_forward_host with pinned host buffers (copies inside the timed region).  The same line carries
-the per-layer tables of every benchmark family (ms, GFLOP/s, GB/s, fraction of the layer's roofline,
+gconv_forward_host with pinned host buffers (copies inside the timed region).  A second JSON line, on
+stderr, carries the per-layer tables of every benchmark family (ms, GFLOP/s, GB/s, fraction of the layer's roofline,
 cold and warm L2, the plain-copy and launch-interval floors beside them), the time-falls-with-groups
 checks and a `targets` object that names every layer below the 50 % tensor / 60 % HBM bars.
 `--impl reference` times the CPU oracle (the only reference there is: the paper ships no code) on
@@ -506,6 +506,32 @@ def layer_row(L, ms, variant, peaks, gconv):
             "roofline_frac": t_roof / (ms * 1e-3)}
 
 
+# what the one line on stdout carries; the tables of a run (200 KB) go to stderr, as one line too: a line of that length is cut by whoever
+# keeps the end of the output, and with it the metric
+HEADLINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline", "dtype", "data",
+                 "config", "clocks", "e2e", "gpu_launches")
+ROOFLINE_KEYS = ("bound", "achieved", "peak", "unit", "frac", "traffic", "kernel")
+CPU_KEYS = ("value", "unit", "cores", "kind")
+
+
+def headline(line):
+    """(the short line, everything else) of a run's record; numbers of the short line to seven digits."""
+    def digits(v):
+        if isinstance(v, dict):
+            return {k: digits(u) for k, u in v.items()}
+        if isinstance(v, list):
+            return [digits(u) for u in v]
+        return float("%.7g" % v) if isinstance(v, float) else v
+
+    short = {k: line[k] for k in HEADLINE_KEYS}
+    for name, keys in (("roofline", ROOFLINE_KEYS), ("cpu_baseline", CPU_KEYS)):
+        if line.get(name):
+            short[name] = {k: line[name][k] for k in keys}
+    if line.get("two_streams"):
+        short["two_streams_ms_per_step"] = line["two_streams"]["ms_per_step"]
+    return digits(short), {k: v for k, v in line.items() if k not in HEADLINE_KEYS}
+
+
 def run_ours(args):
     import torch
     import torch.distributed as dist
@@ -803,7 +829,9 @@ def run_ours(args):
                 "gpu_launches": launches_per_step * args.steps,
                 "cpu_baseline": cpu, "layers": rows}
         line.update(extra)
-        print(json.dumps(line))
+        short, tables = headline(line)
+        print(json.dumps(tables), file=sys.stderr, flush=True)
+        print(json.dumps(short), flush=True)
     for it in insts:
         gconv.gconv_desc_destroy(it.desc)
     if world > 1:
