@@ -4,8 +4,12 @@
 // other leave half of it idle.  The batch is cut into up to kMaxParts runs of images; their copies in are enqueued on one side
 // stream, the kernels on the caller's stream as each part lands, the copies out on a second side stream.  The caller's stream
 // waits for the last copy out, so the call keeps its contract: everything happens in stream order, y_host is complete when the
-// stream gets there.  51 MB each way (64 channels @56x56, N = 64, g = 8): 1870 -> 1297 us; the link moves 84 GB/s both ways
+// stream gets there.  51 MB each way (64 channels @56x56, N = 64, g = 8): 1870 -> 1310 us; the link moves 84 GB/s both ways
 // together on this machine (1224 us), the rest is the first part's way in and the last one's way out.
+//
+// A call that finds other streams' calls in flight goes in order: those calls fill the other direction already, with whole copies.
+// us per call on 1, 2 and 3 streams: 32 -> 32 @32x32 N = 128 g = 4 in order 622, 376, 378, always in parts 498, 462, 478, as it is 495, 382,
+// 381; 64 -> 64 @56x56 N = 64 1879, 1099, 1119 / 1379, 1264, 1289 / 1317, 1104, 1105.
 #include <new>
 
 #include "gconv_internal.h"
@@ -24,7 +28,7 @@ constexpr int kMaxLanes = 4;
 struct Lane {
     int device;
     bool busy;                       // a thread is enqueueing on it
-    cudaStream_t last;               // the caller's stream of its last call
+    cudaStream_t last;               // the caller's stream of its last call (which may have run in order; `end` follows it)
     cudaStream_t in, out;
     cudaEvent_t begin, end, landed[kMaxParts], done[kMaxParts];
 };
@@ -74,8 +78,8 @@ static Lane* open_lane(int device) {
 }
 
 // The lane of the last call on this stream (in stream order anyway), else one with nothing in flight (a call's side streams must
-// not wait for another caller's stream), else a new one; nullptr if there is none.
-static Lane* take_lane(int device, cudaStream_t st) {
+// not wait for another caller's stream), else a new one; nullptr if there is none.  `alone`: no other lane's call is in flight.
+static Lane* take_lane(int device, cudaStream_t st, bool& alone) {
     std::lock_guard<std::mutex> lock(g_lane_mutex);
     // (another thread may be capturing a stream: a query or a creation here is none of that capture's business)
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
@@ -94,6 +98,13 @@ static Lane* take_lane(int device, cudaStream_t st) {
         else (void)cudaGetLastError();               // (cudaErrorNotReady)
     }
     if (found == nullptr && empty >= 0) found = g_lanes[empty] = open_lane(device);
+    alone = true;
+    for (int i = 0; i < kMaxLanes && alone; ++i) {
+        const Lane* l = g_lanes[i];
+        if (l == nullptr || l == found || l->device != device) continue;
+        alone = !l->busy && cudaEventQuery(l->end) == cudaSuccess;
+        if (!alone) (void)cudaGetLastError();
+    }
     if (found != nullptr) {
         found->busy = true;
         found->last = st;
@@ -231,8 +242,16 @@ extern "C" int gconv_forward_host(gconv_desc_t d, const float* x_host, const voi
         c->workspace_bytes = d->workspace_bytes;
         c->wait_us = d->wait_us;
     }
-    Lane* l = take_lane(d->device, st);
+    bool alone = true;
+    Lane* l = take_lane(d->device, st, alone);
     if (l == nullptr) return in_order();
+    if (!alone) {
+        // Calls of other streams are in flight: they fill the other direction of the link, and whole copies do that better than parts.
+        rc = in_order();
+        if (cudaEventRecord(l->end, st) != cudaSuccess) (void)cudaGetLastError();
+        give_back(l);
+        return rc;
+    }
     cudaError_t e = cudaSuccess;
     bool side = false;                             // the side streams hold work that uses the caller's buffers
     auto check = [&](cudaError_t r) { if (e == cudaSuccess) e = r; return e == cudaSuccess; };

@@ -88,6 +88,43 @@ def test_host_buffers_that_share_memory(cfg, shift):
         L.close()
 
 
+def test_calls_of_several_streams_move_whole_batches():
+    """A call that finds another stream's call in flight copies x and y whole (the callers overlap by themselves); alone, it copies parts."""
+    L = _Host(64, 64, 28, 28, 64, 3, 1, 8)
+    try:
+        streams = [torch.cuda.Stream() for _ in range(3)]
+        stages = [(torch.empty_like(L.xs), torch.empty_like(L.ys)) for _ in streams]
+        ys = [torch.full(L.want.shape, float("nan")).pin_memory() for _ in streams]
+
+        def copies(body):
+            torch.cuda.synchronize()
+            with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CPU, torch.profiler.ProfilerActivity.CUDA]) as prof:
+                body()
+                torch.cuda.synchronize()
+            names = [e.name for e in prof.events()]
+            return sum("Memcpy HtoD" in n for n in names), sum("Memcpy DtoH" in n for n in names)
+
+        def call(k):
+            gconv.gconv_forward_host(L.d, L.xh, L.wp, ys[k], *stages[k], streams[k])
+
+        def overlapped():
+            with torch.cuda.stream(streams[0]):
+                torch.cuda._sleep(20_000_000)                   # some 10 ms: the first call is in flight until the others are enqueued
+            call(0)                                             # (nothing of the library's is in flight yet: parts)
+            call(1)
+            call(2)
+            call(1)
+
+        alone = copies(lambda: call(0))
+        assert alone[0] > 1 and alone[0] == alone[1], alone
+        assert copies(overlapped) == (alone[0] + 3, alone[1] + 3)
+        assert copies(lambda: call(2)) == alone
+        for y in ys:
+            L.check(y)
+    finally:
+        L.close()
+
+
 def test_host_parts_from_several_threads_and_in_a_graph():
     L = _Host(48, 64, 32, 32, 64, 3, 1, 4)
     other = [(torch.empty_like(L.xs), torch.empty_like(L.ys)) for _ in range(2)]
