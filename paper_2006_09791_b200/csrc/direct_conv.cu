@@ -52,47 +52,54 @@ __device__ __forceinline__ void ffma2(float2& d, float2 a, float2 b) {
 }
 
 // The tile's outputs one by one, taps outside the image left out: weights that are infinite or not a number must not meet the zeros that
-// are staged for the padding.  (Inlined, parameters by value, the branch marked as rare: as a called function it
-// cost the main path registers and spills, six layers of other filters N = 16 @224 244 -> 254 us; like this 244.5.)
-__device__ __forceinline__ void plain_tile(const Shape& s, const ConvCfg& c, const float* __restrict__ x, const float* __restrict__ wpk, float* __restrict__ y, int BM) {
+// are staged for the padding.  (Its parameters come a second time, as its own: values shared with the main path were moved ahead of the
+// branch and cost that path registers, 2 % on tiles of 16 filters by 64 pixels.)
+struct Plain {
+    int split, kblocks, groups, tiles_x, tiles_y, NI, TH, TW, BM;
+    int Kg, N, C_in, Cg, KH, KW, H, W, H_out, W_out, stride, stride_w, dilation, dilation_w, pad, pad_w;
+    const float* x;
+    const float* wpk;
+    float* y;
+};
+__device__ __forceinline__ void plain_tile(const Plain& t) {
     int b = (int)blockIdx.x;
-    const int rank = b % c.split; b /= c.split;
-    const int kb0 = b % c.kblocks * BM; b /= c.kblocks;
-    const int g = b % s.groups; b /= s.groups;
-    const int q0 = b % c.tiles_x * c.TW; b /= c.tiles_x;
-    const int p0 = b % c.tiles_y * c.TH, n0 = b / c.tiles_y * c.NI, pixels = c.NI * c.TH * c.TW, threads = (int)blockDim.x;
+    const int rank = b % t.split; b /= t.split;
+    const int kb0 = b % t.kblocks * t.BM; b /= t.kblocks;
+    const int g = b % t.groups; b /= t.groups;
+    const int q0 = b % t.tiles_x * t.TW; b /= t.tiles_x;
+    const int p0 = b % t.tiles_y * t.TH, n0 = b / t.tiles_y * t.NI, pixels = t.NI * t.TH * t.TW, threads = (int)blockDim.x;
 #pragma unroll 1
-    for (int i = rank * threads + (int)threadIdx.x; i < pixels * BM; i += c.split * threads) {
-        const int k = kb0 + i / pixels, pix = i % pixels, rem = pix % (c.TH * c.TW), n = n0 + pix / (c.TH * c.TW), p = p0 + rem / c.TW, q = q0 + rem % c.TW;
-        if (k >= s.Kg || n >= s.N || p >= s.H_out || q >= s.W_out) continue;
+    for (int i = rank * threads + (int)threadIdx.x; i < pixels * t.BM; i += t.split * threads) {
+        const int k = kb0 + i / pixels, pix = i % pixels, rem = pix % (t.TH * t.TW), n = n0 + pix / (t.TH * t.TW), p = p0 + rem / t.TW, q = q0 + rem % t.TW;
+        if (k >= t.Kg || n >= t.N || p >= t.H_out || q >= t.W_out) continue;
         float acc = 0.f;
 #pragma unroll 1
-        for (int ch = 0; ch < s.Cg; ++ch)
+        for (int ch = 0; ch < t.Cg; ++ch)
 #pragma unroll 1
-            for (int r = 0; r < s.KH; ++r) {
-                const int h = p * s.stride + r * s.dilation - s.pad;
-                if (h < 0 || h >= s.H) continue;
+            for (int r = 0; r < t.KH; ++r) {
+                const int h = p * t.stride + r * t.dilation - t.pad;
+                if (h < 0 || h >= t.H) continue;
 #pragma unroll 1
-                for (int t = 0; t < s.KW; ++t) {
-                    const int v = q * s.stride_w + t * s.dilation_w - s.pad_w;
-                    if (v < 0 || v >= s.W) continue;
-                    acc = fmaf(__ldg(x + (((size_t)n * s.C_in + (size_t)g * s.Cg + ch) * s.H + h) * s.W + v),
-                               __ldg(wpk + ((((size_t)g * s.Cg + ch) * s.KH + r) * s.KW + t) * s.Kg + k), acc);
+                for (int c = 0; c < t.KW; ++c) {
+                    const int v = q * t.stride_w + c * t.dilation_w - t.pad_w;
+                    if (v < 0 || v >= t.W) continue;
+                    acc = fmaf(__ldg(t.x + (((size_t)n * t.C_in + (size_t)g * t.Cg + ch) * t.H + h) * t.W + v),
+                               __ldg(t.wpk + ((((size_t)g * t.Cg + ch) * t.KH + r) * t.KW + c) * t.Kg + k), acc);
                 }
             }
-        y[(((size_t)n * s.groups + g) * s.Kg + k) * s.H_out * s.W_out + (size_t)p * s.W_out + q] = acc;
+        t.y[(((size_t)n * t.groups + g) * t.Kg + k) * t.H_out * t.W_out + (size_t)p * t.W_out + q] = acc;
     }
 }
 
 template <int TM, int TN>
 __global__ void __launch_bounds__(256, TM * TN > 64 ? 1 : 2)
 direct_conv_kernel(const Shape s, const ConvCfg c, const float* __restrict__ x, const uint32_t* __restrict__ packed,
-                   float* __restrict__ y, Status* status, uint32_t tag) {
+                   float* __restrict__ y, Status* status, uint32_t tag, const Plain plain) {
     extern __shared__ __align__(16) float conv_smem[];
     dependent_start();
     const uint32_t seen = __ldg(packed);
     if (__builtin_expect(seen != tag, 0)) {               // uniform across the grid
-        if (seen == (tag ^ kNonFiniteMark)) plain_tile(s, c, x, reinterpret_cast<const float*>(packed + kHeaderBytes / 4), y, c.WM * TM);
+        if (seen == (tag ^ kNonFiniteMark)) plain_tile(plain);
         else if (threadIdx.x == 0) record_status(status, GCONV_ERR_PACK_MISMATCH, (int)blockIdx.x);
         return;
     }
@@ -446,7 +453,9 @@ bool conv_config(const Shape& s, int sm_count, ConvCfg& best) {
 template <int TM, int TN>
 static cudaError_t launch_conv(const Shape& s, const ConvCfg& c, const float* x, const uint32_t* pk, float* y, Status* status,
                                uint32_t tag, const Launch& st) {
-    return launch_kernel<direct_conv_kernel<TM, TN>>(c.ctas, (unsigned)(32 * c.WM * c.WN), c.smem, st, (unsigned)c.split, s, c, x, pk, y, status, tag);
+    const Plain plain = {c.split, c.kblocks, s.groups, c.tiles_x, c.tiles_y, c.NI, c.TH, c.TW, c.WM * TM, s.Kg, s.N, s.C_in, s.Cg, s.KH, s.KW, s.H, s.W,
+                         s.H_out, s.W_out, s.stride, s.stride_w, s.dilation, s.dilation_w, s.pad, s.pad_w, x, reinterpret_cast<const float*>(pk + kHeaderBytes / 4), y};
+    return launch_kernel<direct_conv_kernel<TM, TN>>(c.ctas, (unsigned)(32 * c.WM * c.WN), c.smem, st, (unsigned)c.split, s, c, x, pk, y, status, tag, plain);
 }
 
 cudaError_t conv_forward(const Shape& s, const ConvCfg& c, const float* x, const void* packed, float* y, Status* status, uint32_t tag,
