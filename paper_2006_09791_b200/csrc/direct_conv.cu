@@ -393,8 +393,30 @@ double conv_cost(const Shape& s, const ConvCfg& c, int sm_count) {
     return full * wave(occ) + (rest > 0 ? wave(ceil(rest / sm_count)) : 0.0);
 }
 
+// Taps of an axis that meet the image, on average over the outputs.
+double taps_inside(int in, int out, int k, int stride, int pad, int dilation) {
+    long long inside = 0;
+    for (int r = 0; r < k; ++r) {
+        const long long first = pad - (long long)r * dilation;                  // outputs p with first <= p * stride < first + in
+        const long long lo = first <= 0 ? 0 : (first + stride - 1) / stride, hi = first + in <= 0 ? 0 : (first + in - 1) / stride + 1;
+        const long long end = hi < out ? hi : out;
+        inside += end > lo ? end - lo : 0;
+    }
+    return (double)inside / out;
+}
+
+// Estimated time of the one-thread-per-output kernel on groups of one filter, microseconds: a thread's own chain, or every output's taps
+// (most of a tap's cost where it meets the image, some of it where it does not).  A fit over 235 timed layers (21 % r.m.s.).
+double plain_us(const Shape& s) {
+    const double taps = (double)s.Cg * s.KH * s.KW, outputs = 1e-6 * s.N * s.C_out * ((double)s.H_out * s.W_out);
+    const double inside = s.Cg * taps_inside(s.H, s.H_out, s.KH, s.stride, s.pad, s.dilation) * taps_inside(s.W, s.W_out, s.KW, s.stride_w, s.pad_w, s.dilation_w);
+    const double chain = 0.048 * taps + 0.061 * inside, all = outputs * (9.1 + 0.32 * taps + 0.45 * inside);
+    return 2.9 + (chain > all ? chain : all);
+}
+
 }  // namespace
 
+// false: the one-thread-per-output kernel runs (no tile fits, or it is the faster one)
 bool conv_config(const Shape& s, int sm_count, ConvCfg& best) {
     bool found = false;
     double best_cost = 0.0;
@@ -440,7 +462,12 @@ bool conv_config(const Shape& s, int sm_count, ConvCfg& best) {
                 }
             }
     }
-    if (!found) return false;
+    // Groups of one filter leave the register tiles a single row and, with strides, dilations and small planes, a staged patch that is mostly
+    // halo: the one-thread-per-output kernel takes them where it is estimated to be the faster one (the estimate of the tiles is 20 ... 40 %
+    // low for single channels).  Staged -> that kernel: 121 channels @6x6 11x11 stride 3 dilation 3 N = 51 80.2 -> 4.2 us, 224 @14x14 5x5 stride 2 dilation 4
+    // N = 113 105.0 -> 33.1, 140 @28x6 1x7 dilation 3 N = 65 57.9 -> 18.1; but 22 @56x56 7x7 dilation 2 N = 105 159.6 against 264.6.  Over 235
+    // layers the choice is 3 % slower than the better kernel on average, the staged kernel everywhere 30 %.  (Two filters and more: staged.)
+    if (!found || (s.Kg == 1 && plain_us(s) < (s.Cg == 1 ? 1.2 : 0.9) * (best_cost / 1965.0 + 1.5))) return false;
     best.div_ph = make_fastdiv((uint32_t)best.PH);
     best.div_cc = make_fastdiv((uint32_t)best.CC);
     best.div_sw = make_fastdiv((uint32_t)s.stride_w);

@@ -1,8 +1,9 @@
 // Variant DIRECT_GENERIC: FP32 grouped convolution of any shape the descriptor accepts (any kernel size; stride, padding and
-// dilation per axis).  Nearly every shape runs on the staged kernel of direct_conv.cu; the kernel here, one thread per output
-// element straight from global memory, takes what no tile of that one holds (single-channel patches over 200 KB: filters
-// or dilations of hundreds of pixels).  Grouped convolution of Section II of the paper, summed in the (c, r, s) order of
-// the convolution stage of Algorithm 1.  Packed weights: [g][c][r][s][Kg], as for DIRECT_TILED.
+// dilation per axis).  Most shapes run on the staged kernel of direct_conv.cu; the kernel here, one thread per output element
+// straight from global memory, takes what no tile of that one holds (single-channel patches over 200 KB: filters or dilations of
+// hundreds of pixels) and the groups of one filter whose staged tiles would be mostly halo (conv_config).  Grouped convolution of
+// Section II of the paper, summed in the (c, r, s) order of the convolution stage of Algorithm 1.  Packed weights:
+// [g][c][r][s][Kg], as for DIRECT_TILED.
 #include "gconv_internal.h"
 
 namespace gconv {
@@ -18,6 +19,9 @@ cudaError_t generic_pack(const Shape& s, const float* w, void* packed, cudaStrea
 // The tag names the layout as well as the shape (a blob packed as a plain OIHW copy by an earlier build is refused).
 uint32_t generic_tag(const Shape& s) { return pack_tag(s, GCONV_VARIANT_DIRECT_GENERIC | (2 << 8)); }
 
+// What bounds it is a thread's chain of taps, or the instructions of all taps (index arithmetic, two bounds tests).  ONE (a filter a group):
+// the weights of a thread lie side by side.  (With the step of Kg floats in a register instead 146 depthwise layers took 8 % longer.)
+template <bool ONE>
 __global__ void __launch_bounds__(256)
 generic_forward_kernel(Shape s, const float* __restrict__ x, const uint32_t* __restrict__ packed,
                        float* __restrict__ y, Status* status, uint32_t tag) {
@@ -46,7 +50,8 @@ generic_forward_kernel(Shape s, const float* __restrict__ x, const uint32_t* __r
                 for (int ss = 0; ss < s.KW; ++ss) {
                     const int v = q * s.stride_w + ss * s.dilation_w - s.pad_w;
                     if (v < 0 || v >= s.W) continue;
-                    acc = fmaf(__ldg(xg + ((size_t)c * s.H + h) * s.W + v), __ldg(wk + (size_t)((c * s.KH + r) * s.KW + ss) * s.Kg), acc);
+                    const int tap = (c * s.KH + r) * s.KW + ss;
+                    acc = fmaf(__ldg(xg + ((size_t)c * s.H + h) * s.W + v), __ldg(wk + (ONE ? (size_t)tap : (size_t)tap * s.Kg)), acc);
                 }
             }
         }
@@ -61,7 +66,11 @@ cudaError_t generic_forward(const Shape& s, const ConvCfg* conv, const float* x,
     size_t want = (total + 255) / 256;
     size_t cap = (size_t)sm_count * 8 * 4;
     int blocks = (int)(want < cap ? want : cap);
-    return launch_kernel<generic_forward_kernel>((unsigned)blocks, 256, 0, st, 1, s, x, reinterpret_cast<const uint32_t*>(packed), y, status, tag);
+    // (not beside the previous kernel's tail: its blocks work from L1, whose size follows the kernel before it; 6 % on depthwise layers)
+    const Launch to = {st.st, false};
+    const uint32_t* pk = reinterpret_cast<const uint32_t*>(packed);
+    return s.Kg == 1 ? launch_kernel<generic_forward_kernel<true>>((unsigned)blocks, 256, 0, to, 1, s, x, pk, y, status, tag)
+                     : launch_kernel<generic_forward_kernel<false>>((unsigned)blocks, 256, 0, to, 1, s, x, pk, y, status, tag);
 }
 
 }  // namespace gconv

@@ -169,7 +169,7 @@ cudaError_t generic_pack(const Shape& s, const float* w, void* packed, cudaStrea
 cudaError_t generic_forward(const Shape& s, const ConvCfg* conv, const float* x, const void* packed, float* y, Status* status,
                             int sm_count, uint32_t tag, const Launch& st);
 
-bool conv_config(const Shape& s, int sm_count, ConvCfg& c);   // false: no tile fits (huge filters or dilations)
+bool conv_config(const Shape& s, int sm_count, ConvCfg& c);   // false: the one-thread-per-output kernel runs
 cudaError_t conv_forward(const Shape& s, const ConvCfg& c, const float* x, const void* packed, float* y, Status* status, uint32_t tag,
                          const Launch& st);
 

@@ -86,7 +86,7 @@ def test_staged_fp32_buffers_in_64_bits(probe):
     rows = probe(huge + drawn)
     bad = [s for s, r in zip(huge + drawn, rows) if r is None or r[3] == 0]
     assert not bad, (len(bad), bad[:5])
-    assert sum(r[3] == 1 for r in rows) > 700, sum(r[3] == 1 for r in rows)
+    assert sum(r[3] == 1 for r in rows) > 600, sum(r[3] == 1 for r in rows)
     # more output pixels than 31 bits count: still staged
     assert probe([(70000, 1, 180, 180, 1, 7, 7, 1, 1, 3, 3, 1, 1, 1)])[0][3] == 1
 
@@ -95,3 +95,11 @@ def test_host_batches_are_cut_for_the_variant_that_runs(probe):
     """A batch whose tensor-core layout allows no parts is cut once the descriptor runs the generic variant."""
     rows = probe([_square(8, 576, 16, 16, 2304, 1, 1, 3), _square(92, 6144, 20, 20, 512, 3, 1, 32), _square(27, 384, 42, 42, 32, 3, 1, 2)])
     assert [r[4] for r in rows] == [0, 0, 0] and [r[5] for r in rows] == [4, 5, 5]
+
+
+def test_groups_of_one_filter_take_the_faster_fp32_kernel(probe):
+    """Patches that are mostly halo: one thread per output; wide planes, several filters: staged."""
+    plain = [(51, 121, 6, 6, 121, 11, 11, 3, 3, 15, 15, 3, 3, 121), (113, 224, 14, 14, 224, 5, 5, 2, 2, 8, 8, 4, 4, 224), (65, 140, 28, 6, 140, 1, 7, 1, 1, 0, 9, 3, 3, 140),
+             (125, 158, 14, 14, 79, 1, 7, 2, 2, 0, 3, 1, 1, 79)]
+    staged = [(105, 22, 56, 56, 22, 7, 7, 1, 1, 6, 6, 2, 2, 22), (4, 64, 29, 29, 128, 7, 7, 1, 1, 3, 3, 1, 1, 64), (2, 6, 19, 21, 6, 7, 7, 1, 1, 3, 3, 1, 1, 6)]
+    assert [r[3] for r in probe(plain + staged)] == [-1] * 4 + [1] * 3

@@ -37,6 +37,9 @@ CASES = [  # N, C_in, H, W, C_out, (filter), (stride), (pad), (dilation), groups
     # column strides far beyond the width: whole column phases of a staged row would be millions of columns
     (1, 1, 5000, 1, 1, (3, 1), (1, 3000000), (0, 0), (1, 1), 1), (2, 8, 30, 5, 8, (3, 3), (1, 2147483647), (1, 1), (1, 1), 1),
     (2, 6, 9, 40, 4, (3, 3), (2, 50), (1, 1), (1, 1), 2),
+    # groups of one filter whose patches are mostly halo: the one-thread-per-output kernel, one channel a group and two
+    (3, 21, 6, 6, 21, (11, 11), (3, 3), (15, 15), (3, 3), 21), (5, 30, 14, 14, 30, (5, 5), (2, 2), (8, 8), (4, 4), 30),
+    (7, 14, 28, 6, 14, (1, 7), (1, 1), (0, 9), (1, 3), 14), (6, 20, 7, 7, 10, (7, 7), (2, 2), (9, 9), (3, 3), 10),
 ]
 
 
