@@ -1810,7 +1810,10 @@ size_t igemm_scratch_bytes(const Shape& s_any) {
 // 12.7 -> 6.7, 256 -> 256 @13x13 N = 13 g = 2 14.2 -> 12.9; but 64 -> 64 @14x14 N = 1 (48 channels spared) 5.9 -> 6.4 and, on row boxes,
 // whose stages are the quickest, 128 -> 128 @20x20 N = 2 (96 spared) 6.6 -> 7.4 against 256 -> 256 @28x28 N = 1 (192 spared)
 // 10.1 -> 9.3: the lines lie between.  16x16 and 8x8 planes: 128 -> 128 @16x16 (96 spared) N = 1, 4 tiles, 6.8 -> 6.2, N = 6, 24 tiles, 7.1 -> 7.5.
-// Stride-2 row tiles gain at 32 channels already (64 -> 128 @56x56 N = 1 8.5 -> 6.2).
+// Stride 2: row tiles of two segments gain at 32 channels already (64 -> 128 @56x56 N = 1 8.5 -> 6.2), those of one segment, whose whole tiles
+// have instantiations of their own, from 192 on (256 -> 512 @20x12 g = 4 N = 3 5.1 -> 8.0 with 32, 128 -> 192 @24x16 N = 1 6.1 -> 6.6 with 96, 192 ->
+// 192 @36x16 N = 1 7.9 -> 8.2 with 160, 256 -> 64 @36x24 N = 1 10.0 -> 7.2 with 224); the gather producer's pair tiles from 64 on (16 channels a group
+// @7x7 ... 30x30 1.15 ... 1.45 times as long, 32 -> 64 @9x27 g = 4 N = 21 8.4 -> 9.7, 64 -> 128 @27x19 g = 8 N = 2 13.6 -> 11.5).
 static int max_split(int tiles) { return tiles <= 15 ? 8 : (tiles <= 22 ? 6 : (tiles <= 26 ? 5 : (tiles <= 33 ? 4 : (tiles <= 45 ? 3 : (tiles <= 74 ? 2 : 1))))); }
 static void split_channels(IgemmCfg& c) {
     c.spl = 0;
@@ -1823,7 +1826,7 @@ static void split_channels(IgemmCfg& c) {
     S = (c.chunks + per - 1) / per;                  // every rank has work
     // channels a CTA has to be spared, above (0: tilings whose whole tiles run the generic instantiation)
     const bool s1 = !c.sub_h && !c.sub_w;
-    const int least = c.soft == 1 ? 96 : (s1 && c.Kt == 64 && c.rowbox ? 160 : (s1 && c.Kt == 64 && c.nr == 1 ? (c.num_tiles <= 15 ? 96 : 160) : 0));
+    const int least = c.soft == 1 ? 96 : (c.soft == 2 && c.pair) ? 64 : (c.s2h && c.Kt == 64 && c.SR == 1) ? 192 : (s1 && c.Kt == 64 && c.rowbox ? 160 : (s1 && c.Kt == 64 && c.nr == 1 ? (c.num_tiles <= 15 ? 96 : 160) : 0));
     if ((c.chunks - per) * c.CK * (c.pair ? 2 : 1) < least) return;
     if (S < 2 || (uint32_t)c.stages * c.stage_bytes < (uint32_t)(c.pair ? 2 : 1) * (uint32_t)c.Kt * 512u) return;
     c.spl = 1;

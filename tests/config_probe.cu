@@ -1,7 +1,8 @@
 // Reads descriptors (one per line: N C_in H W C_out KH KW stride_h stride_w pad_h pad_w dilation_h dilation_w groups) and prints what the
 // library's host code makes of each: the variant, whether an instantiation runs its configuration, the workspace, and for the staged FP32
 // kernel whether its shared memory holds what the kernel puts there (-1: the one-thread-per-output kernel runs), the parts a batch of host
-// buffers is cut into, and those after the descriptor has been set to the generic variant.  Host code only.
+// buffers is cut into, and those after the descriptor has been set to the generic variant, and of the tensor-core configuration: CTAs that
+// share a tile's channels, whether its tiles are row boxes, and filters a tile (0 where the variant does not apply).  Host code only.
 #include <stdio.h>
 
 #include "../paper_2006_09791_b200/csrc/gconv_internal.h"
@@ -33,8 +34,10 @@ int main() {
         const int staged = gconv::conv_config(d->s, 148, c) ? staging_fits(d->s, c) : -1;
         const int variant = d->variant, parts = gconv::host_parts(d);
         gconv_desc_set_variant(d, GCONV_VARIANT_DIRECT_GENERIC);
-        printf("%d %d %zu %d %d %d\n", variant, !tc || gconv::igemm_runnable(d->s, 0, 148) ? 1 : 0, tc ? gconv::igemm_scratch_bytes(d->s) : (size_t)0, staged, parts,
-               gconv::host_parts(d));
+        gconv::IgemmCfg ig = {};
+        if (tc) ig = gconv::igemm_config(d->s, 148);
+        printf("%d %d %zu %d %d %d %d %d %d\n", variant, !tc || gconv::igemm_runnable(d->s, 0, 148) ? 1 : 0, tc ? gconv::igemm_scratch_bytes(d->s) : (size_t)0, staged, parts,
+               gconv::host_parts(d), ig.spl ? ig.split : 0, ig.rowbox, ig.Kt);
         gconv_desc_destroy(d);
     }
 }

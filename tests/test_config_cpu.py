@@ -103,3 +103,10 @@ def test_groups_of_one_filter_take_the_faster_fp32_kernel(probe):
              (125, 158, 14, 14, 79, 1, 7, 2, 2, 0, 3, 1, 1, 79)]
     staged = [(105, 22, 56, 56, 22, 7, 7, 1, 1, 6, 6, 2, 2, 22), (4, 64, 29, 29, 128, 7, 7, 1, 1, 3, 3, 1, 1, 64), (2, 6, 19, 21, 6, 7, 7, 1, 1, 3, 3, 1, 1, 6)]
     assert [r[3] for r in probe(plain + staged)] == [-1] * 4 + [1] * 3
+
+
+def test_stride_2_splits_only_where_they_pay(probe):
+    """Channels a CTA is spared: too few on row tiles of one segment and on the gather producer's pair tiles, enough, and row tiles of two segments."""
+    whole = [(3, 256, 20, 12, 512, 3, 2, 4), (1, 192, 36, 16, 192, 3, 2, 1), (11, 128, 16, 18, 512, 3, 2, 8), (21, 128, 9, 27, 256, 3, 2, 4)]
+    split = [(1, 256, 36, 24, 64, 3, 2, 1), (1, 64, 56, 56, 128, 3, 2, 1), (2, 512, 27, 19, 1024, 3, 2, 8), (1, 768, 5, 5, 768, 3, 2, 1)]
+    assert [r[6] > 0 for r in probe([_square(*s) for s in whole + split])] == [False] * 4 + [True] * 4
