@@ -110,3 +110,9 @@ def test_stride_2_splits_only_where_they_pay(probe):
     whole = [(3, 256, 20, 12, 512, 3, 2, 4), (1, 192, 36, 16, 192, 3, 2, 1), (11, 128, 16, 18, 512, 3, 2, 8), (21, 128, 9, 27, 256, 3, 2, 4)]
     split = [(1, 256, 36, 24, 64, 3, 2, 1), (1, 64, 56, 56, 128, 3, 2, 1), (2, 512, 27, 19, 1024, 3, 2, 8), (1, 768, 5, 5, 768, 3, 2, 1)]
     assert [r[6] > 0 for r in probe([_square(*s) for s in whole + split])] == [False] * 4 + [True] * 4
+
+
+def test_pointwise_stride_2_filter_tiles_follow_the_tiles_there_are(probe):
+    """Even rows only, a tile four segments of one row each: on 8- and 16-wide planes more tiles than pixels / 128, so wider filter tiles."""
+    rows = probe([_square(30, 256, 8, 8, 512, 1, 2, 1, 0), _square(32, 1024, 16, 16, 128, 1, 2, 2, 0), _square(64, 256, 56, 56, 512, 1, 2, 1, 0)])
+    assert [r[8] for r in rows] == [128, 64, 256] and all(r[7] for r in rows)
