@@ -2081,15 +2081,25 @@ static IgemmCfg igemm_config_c2(const Shape& s_any, int sm_count, int C2) {
     // (the second segment of a row shifted left to end at column W).  Every vertical tap is then a whole number of
     // segments away, so one staged block (tile + a row above and below, one 5-D TMA box) serves all three taps, and
     // each segment contains the horizontal neighbours of the columns it stores (no exchange between warps).  Taken
-    // however many lanes of a segment stay empty: the flat tiling copies every tap by itself, exchanges edge lanes between warps and
-    // runs the generic instantiation.  Flat -> row boxes: 64 -> 64 @40x40 N = 64 42.9 -> 20.0 us (g = 1), 38.2 -> 14.0 us (g = 8);
+    // while the empty lanes do not cost more: the flat tiling copies every tap by itself, exchanges edge lanes between warps and
+    // runs the generic instantiation, 2.5 times as long a tile, but on narrow planes needs up to eight times fewer tiles.  Flat -> row boxes: 64 -> 64 @40x40 N = 64 42.9 -> 20.0 us (g = 1), 38.2 -> 14.0 us (g = 8);
     // 256 -> 256 @12x12 N = 64, 3/8 of the lanes in use, 74.0 -> 39.5 us (g = 1), 24.1 -> 10.9 us (g = 8); 128 -> 128 @9x8 N = 8, a
     // quarter in use, g = 8 7.7 -> 3.0 us; pointwise 256 -> 256 @40x40 stride 2 81.3 -> 58.8 us.  Only stride 2 on 4- and 8-wide planes
     // (no stride-2 row tiles there) is faster flat: 128 -> 256 @9x8 N = 64 g = 8 13.1 against 21.9 us.
+    // Tall planes 4 and 8 wide that fill the chip several times over are flat (3x3): 128 -> 256 @77x4 N = 122 g = 2 row boxes 4.0 times as long, 64 ->
+    // 128 @146x8 N = 26 2.0 times, 256 -> 256 @13x4 N = 36 1.3; up to a ratio of waves of 3.2 row boxes win (64 -> 64 @11x8 N = 91 0.58 at 3.0, 32 ->
+    // 32 @49x4 N = 70 0.80 at 3.1; over 207 shapes 5 % faster on average than row boxes everywhere).
     c.rowbox = 0;
     c.SR = 0;
-    if (!c.seg_mode && s.W <= (c.pw ? 64 : 62) && !(s.stride == 2 && s.W <= 8 && !c.row_skip)) {
-        const int sr = s.W <= 32 ? 1 : 2;
+    const int sr = s.W <= 32 ? 1 : 2;
+    bool fewer_flat = false;
+    if (!c.seg_mode && !fuse && !c.pw && s.stride == 1) {
+        const bool two = 2 * c.Np <= 256 && 3u * (uint32_t)c.Cg * (uint32_t)c.Np * 4u <= 40u * 1024u;        // (CTAs an SM holds, see below)
+        const double per_row_tile = (double)c.groups * c.NT * s.N / (kLayoutSMs * (two ? 2 : 1));
+        const double boxes = per_row_tile * ((s.H + 4 / sr - 1) / (4 / sr)), flat = per_row_tile * c.RB;
+        fewer_flat = (boxes > 1.0 ? boxes : 1.0) > 3.2 * (flat > 1.0 ? flat : 1.0);
+    }
+    if (!c.seg_mode && s.W <= (c.pw ? 64 : 62) && !(s.stride == 2 && s.W <= 8 && !c.row_skip) && !fewer_flat) {
         c.rowbox = 1;
         c.SR = sr;
         c.R = 4 / sr;                                // rows per tile

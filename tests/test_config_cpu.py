@@ -116,3 +116,9 @@ def test_pointwise_stride_2_filter_tiles_follow_the_tiles_there_are(probe):
     """Even rows only, a tile four segments of one row each: on 8- and 16-wide planes more tiles than pixels / 128, so wider filter tiles."""
     rows = probe([_square(30, 256, 8, 8, 512, 1, 2, 1, 0), _square(32, 1024, 16, 16, 128, 1, 2, 2, 0), _square(64, 256, 56, 56, 512, 1, 2, 1, 0)])
     assert [r[8] for r in rows] == [128, 64, 256] and all(r[7] for r in rows)
+
+
+def test_tall_narrow_planes_are_flat_where_row_boxes_take_many_more_waves(probe):
+    flat = [(122, 128, 77, 4, 256, 3, 1, 2), (26, 64, 146, 8, 128, 3, 1, 1), (36, 256, 13, 4, 256, 3, 1, 1)]
+    boxes = [(91, 64, 11, 8, 128, 3, 1, 1), (70, 32, 49, 4, 32, 3, 1, 1), (2, 32, 18, 4, 32, 3, 1, 1), (64, 256, 12, 12, 256, 3, 1, 1)]
+    assert [r[7] for r in probe([_square(*s) for s in flat + boxes])] == [0] * 3 + [1] * 4
