@@ -30,3 +30,11 @@ def test_sparse_row_boxes(cfg):
     N, C, H, W, K, k, stride, g = cfg
     err, used = check_layer(Layer("rowbox", N, C, H, W, K, k, k, stride, k // 2, 1, g), seed=13)
     assert used == gconv.GCONV_VARIANT_IGEMM_TF32
+
+
+# tall planes 4 and 8 wide whose row-box tiles would take several times the waves: flat tiles (rows straddle the warps' quarters)
+@pytest.mark.parametrize("cfg", [(36, 256, 13, 4, 256, 1), (26, 64, 146, 8, 128, 1), (60, 96, 77, 4, 32, 4)])
+def test_tall_narrow_planes(cfg):
+    N, Ci, H, W, Co, g = cfg
+    err, used = check_layer(Layer("tall", N, Ci, H, W, Co, groups=g), seed=23)
+    assert used == gconv.GCONV_VARIANT_IGEMM_TF32
