@@ -19,7 +19,7 @@
 // Measured against the kernels it replaced (one thread per output; a fixed 4-pixel tile for 3x3), N = 16: 3 -> 64 @224x224
 // 7x7 stride 2 1310 -> 113 us (34 TFLOP/s, 45 % of the FP32 peak), 64 -> 64 @56x56 dilation 2, 4 groups 461 -> 39 us,
 // 64 -> 128 @28x28 5x5 stride 2, 4 groups 138 -> 29 us, 3 -> 32 @224x224 3x3 stride 2 32 -> 23 us; 512 -> 512 @4x4 3x3 (N = 6)
-// 3197 -> 37 us.  What is left on the large ones: the FP32 pipe is active 72 % of the time (the packed FMAs, and as many
+// 3197 -> 37 us.  What is left on the large ones: the FP32 pipe is active 60 % of the time (the packed FMAs, and as many
 // moves that pair their operands as shared-memory loads), and the last wave of CTAs is partly empty.
 #include <cooperative_groups.h>
 #include <math.h>

@@ -462,7 +462,7 @@ DwPlan dw_plan(const Shape& s, int sm_count) {
     const bool k3 = s.KH == 3, s2 = s.stride == 2;
     const int fewest = s.W == 28 ? (k3 ? 12288 : (s2 ? 6144 : 4096))
                                  : s.W == 14 ? (k3 ? 12288 : (s2 ? 6144 : 2048)) : (s2 ? (k3 ? 24576 : 12288) : (k3 ? 2048 : 6144));
-    p.planes = dw_plane_supported(s) && !(s.KH == 3 && s.stride == 1 && s.W == 28) &&
+    p.planes = dw_plane_supported(s) &&
                (double)s.N * s.C_in * s.H > (double)fewest * s.W;
     if (p.planes) p.batches = dw_plane_config(s, sm_count);
     else p.strips = dw_config(s, sm_count);

@@ -291,7 +291,7 @@ bool dw_plane_supported(const Shape& s) {
     if (!s.square() || !(s.Cg == 1 && s.Kg == 1) || s.dilation != 1 || !(s.stride == 1 || s.stride == 2)) return false;
     const bool k3 = s.KH == 3 && s.KW == 3 && s.pad == 1, k5 = s.KH == 5 && s.KW == 5 && s.pad == 2;
     if (!(k3 || k5)) return false;
-    if (!(s.W == 7 || s.W == 14 || s.W == 28)) return false;
+    if (!(s.W == 7 || s.W == 14 || (s.W == 28 && !(k3 && s.stride == 1)))) return false;   // (28 wide, 3x3 stride 1: the same on both kernels)
     const long long per_plane = (long long)s.H * s.W + (long long)s.H_out * s.W_out;
     if (per_plane * 4 * 8 > 50 * 1024) return false;              // a batch of four planes, in and out, twice
     return (unsigned long long)s.N * s.C_in < (1ull << 31) / 4;
@@ -355,10 +355,11 @@ cudaError_t dw_plane_forward(const Shape& s, const DwPlaneCfg& c, const float* x
         if (s.W == 7 && s.H == 7 && S == 1) return launch_plane<K, 1, 7, true>(s, c, x, pk, y, status, tag, st); \
         if (s.W == 7) return launch_plane<K, S, 7>(s, c, x, pk, y, status, tag, st); \
         if (s.W == 14) return launch_plane<K, S, 14>(s, c, x, pk, y, status, tag, st); \
-        return launch_plane<K, S, 28>(s, c, x, pk, y, status, tag, st); \
+        if constexpr (K == 3 && S == 1) return cudaErrorInvalidValue;   /* 28 wide: on the strips */ \
+        else return launch_plane<K, S, 28>(s, c, x, pk, y, status, tag, st); \
     } while (0)
     if (s.KH == 3) {
-        if (s.stride == 1) GCONV_PLANE_W(3, 1);   // (28 wide: on the strips, see dw_plan)
+        if (s.stride == 1) GCONV_PLANE_W(3, 1);
         else GCONV_PLANE_W(3, 2);
     } else {
         if (s.stride == 1) GCONV_PLANE_W(5, 1);

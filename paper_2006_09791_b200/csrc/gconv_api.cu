@@ -39,7 +39,8 @@ int select_variant(const Shape& s) {
 }
 
 // What the descriptor's variant keeps from call to call: the staged FP32 kernel's tile (a search over a few hundred choices), the
-// depthwise kernels' strips and batches.
+// depthwise kernels' strips and batches.  148: the SMs of a B200 (a descriptor is made without a device, and its choices are those a
+// saved blob was packed for).
 void choose_tile(gconv_desc* d) {
     d->has_conv = false;
     if (d->variant == GCONV_VARIANT_DIRECT_GENERIC || (d->variant == GCONV_VARIANT_DIRECT_TILED && tiled_takes_conv(d->s)))

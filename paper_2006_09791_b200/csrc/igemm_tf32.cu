@@ -1587,6 +1587,9 @@ struct IgemmGeom {
 // segment tiling fills its lanes whatever the width (12x12 planes: 36 of 40 lanes instead of 12 of 32).
 // Small planes that 28 divides and 32 does not (14x14, 7x8) and small batches of larger ones (28x28) are cut into rows of 28 instead: one
 // box a stage.  512 -> 512 @14x14 N = 64 21.3 us in rows of 28, 22.2 in segments; 512 -> 256 @28x28 N = 4 14.0 and 17.3, N = 64 42.3 and 33.2.
+// One image or a few gain whatever the plane (12 ... 20 % on 56 to 1008 pixels at N = 1), batches only where rows of 28 need hardly more tiles
+// (196 pixels 5 %, 420 3 %; 784 pixels lose 12 ... 16 %, the line at 128 x 148 pixels; small planes that leave a tile half empty lose up to 27 %).
+// Over 215 layers (13 plane sizes, N = 1 ... 128) this line is 5 % behind the better of the two on average, segments everywhere 7, rows of 28 everywhere 6.
 static bool pw_rows_of_28(const Shape& s) {
     const long long hw = (long long)s.H * s.W;
     return s.KH == 1 && s.KW == 1 && s.stride == 1 && hw % 28 == 0 && hw % 32 != 0 && (hw < 400 || s.N * hw < 128ll * kLayoutSMs);
@@ -1997,9 +2000,9 @@ static IgemmCfg igemm_config_c2(const Shape& s_any, int sm_count, int C2) {
     c.csplit = 0;
     c.wait_us = kDefaultWaitUs;
     c.dbg_skip = -1;
-    // Pointwise: one vertical tap (a third of the stages and MMAs), one accumulator per filter (N = Kt), filter tiles of
-    // up to 128.  Stride 2 computes every pixel and stores the even ones (no stride-2 row tiles: those are built around
-    // nine staged rows).
+    // Pointwise: one vertical tap (a third of the stages and MMAs), one accumulator per filter (N = Kt), filter tiles of up to
+    // 256.  Stride 2 reads the even rows only (row_skip) or a copy of the pixels it needs (one_row); what is left of the odd rows
+    // or columns is computed and not stored (no stride-2 row tiles: those are built around nine staged rows).
     const bool one_row = pw_one_row(s_any);              // (with stride 2 only the pixels the layer reads are there)
     c.sub_h = s_any.stride == 2 && !one_row ? 1 : 0;
     c.sub_w = s_any.stride_w == 2 && !one_row ? 1 : 0;
