@@ -109,7 +109,7 @@ def test_calls_of_several_streams_move_whole_batches():
 
         def overlapped():
             with torch.cuda.stream(streams[0]):
-                torch.cuda._sleep(20_000_000)                   # some 10 ms: the first call is in flight until the others are enqueued
+                torch.cuda._sleep(400_000_000)                  # 0.2 s: the first call is in flight until the others are enqueued
             call(0)                                             # (nothing of the library's is in flight yet: parts)
             call(1)
             call(2)

@@ -575,6 +575,8 @@ BLOCK_SHAPES = [
     (2, 32, 32, 32, 4, 32), (40, 32, 32, 32, 4, 32), (130, 32, 32, 32, 16, 48), (3, 64, 16, 16, 2, 64), (96, 64, 16, 16, 8, 128),
     (64, 128, 8, 8, 8, 128), (9, 64, 56, 56, 16, 64), (20, 128, 28, 28, 32, 64), (33, 96, 20, 24, 3, 80), (7, 64, 30, 60, 8, 16),
     (5, 32, 12, 56, 1, 32, 64), (1, 32, 8, 8, 32, 256), (12, 64, 16, 16, 2, 96, 128),
+    # planes that leave most lanes of a row box empty
+    (5, 32, 9, 4, 4, 32), (40, 64, 11, 12, 2, 48), (4, 32, 13, 20, 8, 64), (9, 64, 10, 40, 4, 32), (3, 128, 7, 8, 16, 64),
 ]
 
 
