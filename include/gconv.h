@@ -22,9 +22,15 @@
  *     GCONV_OK (0) on success.
  *   - "device" pointers are CUDA device pointers of the current device, "host" pointers are host
  *     memory.  The caller owns every buffer (the workspace of the few layers that need one included)
- *     and the stream; the library owns only the descriptor and a 16-byte device status block it
- *     allocates on the first pack/forward call of a descriptor.  No other device memory is ever
- *     allocated by the library.
+ *     and the stream; the library owns the descriptor, a 16-byte device status block it allocates on the
+ *     first pack/forward call of a descriptor, host memory of a descriptor (plans, kept from its first
+ *     forward on, freed with it), and, once gconv_forward_host has overlapped a call, up to four sets of two
+ *     streams and twelve events for the process, closed with the last descriptor that used them.  No other
+ *     device memory is ever allocated by the library.
+ *   - Results depend on the sizes and the variant, not on time or address: a call repeated gives the same
+ *     bits.  The order of the FP32 sums is part of the tiling, which follows the batch too: one image alone,
+ *     in a batch, or in a batch that gconv_forward_host cuts may differ in the last bits (and, as the tensor
+ *     cores round the inputs of the next layer, by as much as that rounding after it), within the tolerance.
  *   - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).  pack and
  *     forward only enqueue work on it and return without synchronising.
  *   - Device pointers must be 16-byte aligned (GCONV_ERR_ALIGNMENT otherwise).
@@ -58,7 +64,7 @@ enum gconv_status {
  * max|y - y_ref| / max|y_ref| <= 1e-5 for the FP32 variants, <= 5e-3 for the TF32 variant. */
 enum gconv_variant_id {
     GCONV_VARIANT_AUTO = 0,           /* let the selector choose (default) */
-    GCONV_VARIANT_DIRECT_GENERIC = 1, /* FP32 FFMA, any shape: staged register tiles */
+    GCONV_VARIANT_DIRECT_GENERIC = 1, /* FP32 FFMA, any shape: staged register tiles, or one thread per output where those are mostly halo */
     GCONV_VARIANT_DIRECT_TILED = 2,   /* FP32 FFMA, 3x3, dilation 1: register tiles; depthwise 3x3 (pad 1) and 5x5
                                          (pad 2) on streams of row strips or batches of small planes */
     GCONV_VARIANT_IGEMM_TF32 = 3      /* TF32 tcgen05 implicit GEMM per (merged) group; 3x3 with pad = dilation or 1x1 with pad 0,
@@ -129,7 +135,8 @@ int gconv_desc_set_variant(gconv_desc_t desc, int variant);
  * descriptor's variant reads, prefixed by a 64-byte header that names shape and variant.
  *   w_ochw    device, fp32 [C_out, Cg, KH, KW], read only.
  *   w_packed  device, gconv_packed_bytes(desc) bytes, written.  The blob is position independent
- *             and may be copied, saved and reloaded.
+ *             and may be copied, saved and reloaded by the library build that packed it; a build whose
+ *             layout differs refuses it on the device (GCONV_ERR_PACK_MISMATCH).
  * One kernel launch on `stream` (FP32 variants: the header is cleared before it).  Errors: GCONV_ERR_NULL, GCONV_ERR_ALIGNMENT,
  * GCONV_ERR_CUDA.
  */
@@ -142,7 +149,8 @@ int gconv_pack_weights(gconv_desc_t desc, const float *w_ochw, void *w_packed, v
  *   x_nchw    device, fp32 [N, C_in, H, W], read only; must not overlap y.
  *   w_packed  device, produced by gconv_pack_weights on a descriptor of the same shape and variant.
  *   y_nchw    device, fp32 [N, C_out, H_out, W_out], every element written.
- * Kernel launches only, on `stream`; allocates nothing; deterministic (no atomics on y).  A w_packed made for
+ * Kernel launches only, on `stream`; allocates no device memory after the descriptor's first call (that one works out the
+ * plan and allocates the status block); deterministic (no atomics on y).  A w_packed made for
  * another shape or variant -- or under a descriptor whose batch, plane size or stride led to another packed layout --
  * is detected on the device: y is left unwritten and gconv_last_status reports GCONV_ERR_PACK_MISMATCH.
  * A few layers need a workspace (see gconv_workspace_bytes); without one attached the call enqueues nothing and
@@ -154,7 +162,8 @@ int gconv_forward(gconv_desc_t desc, const float *x_nchw, const void *w_packed, 
  * Workspace (the role of Algorithm 1's input-reshaping stage, Section III-B: a rearranged copy of the padded input).
  * The tensor-core variant stages its input with bulk tensor copies, whose rows must be multiples of 16 bytes.  Layers
  * whose width is not a multiple of 4 therefore either build their stages with copy warps (no workspace) or, where
- * that path does not apply, compute on a zero-padded copy of x kept in a caller-owned device workspace:
+ * that path does not apply, compute on a copy of x -- zero-padded rows, or for pointwise layers the pixels that are read as
+ * one row a plane -- kept in a caller-owned device workspace:
  *   gconv_workspace_bytes     bytes the descriptor's current variant needs; 0 for every layer whose width is a
  *                             multiple of 4, for the FP32 variants, and for the layers of this kind that the copy
  *                             warps serve (gconv_forward_launches reports 1 for them, 2 when a workspace is used).
@@ -170,9 +179,11 @@ int gconv_desc_set_workspace(gconv_desc_t desc, void *workspace, size_t bytes);
  * gconv_forward_host -- the same operation (Section II) for callers whose activations live in host memory:
  * copies x to the device, runs gconv_forward and copies y back, all enqueued on `stream` in order.
  * Batches of a few MB and more are cut into parts whose copies and kernels overlap on streams the library keeps; `stream`
- * still orders the whole call (work before it is waited for, what follows it finds y_host complete).
+ * still orders the whole call (work before it is waited for, what follows it finds y_host complete).  A call that finds calls of
+ * other streams in flight copies whole batches instead: those calls overlap with it already.
  *   x_host    host, fp32 [N, C_in, H, W] (pinned memory makes the copies asynchronous).
- *   y_host    host, fp32 [N, C_out, H_out, W_out], written when the stream reaches that point.
+ *   y_host    host, fp32 [N, C_out, H_out, W_out], written when the stream reaches that point; it may share memory with
+ *             x_host (the whole input is then read before any output is written).
  *   x_stage, y_stage   device staging buffers of the sizes of x and y, caller-owned.
  *   w_packed  device, as for gconv_forward.
  * Errors as gconv_forward.
@@ -218,8 +229,7 @@ int gconv_forward_host_static(gconv_desc_t desc, const float *x_host, const void
  *   y2[n, k2, p, q] = sum_{o < C_out} w2[k2, o] * y[n, o, p, q],   y = the descriptor's grouped convolution of x
  *
  * gconv_block_supported  1 if the pair (descriptor, C2) can run fused, else 0: 3x3, pad 1, stride 1, dilation 1,
- *                        W a multiple of 4 and at most 62 or equal to 64 wide planes only where the grouped kernel
- *                        needs no edge exchange, merged group width a multiple of 8 with at most 64 filters per
+ *                        W a multiple of 4 and at most 60, or 64 where the grouped kernel needs no edge exchange, merged group width a multiple of 8 with at most 64 filters per
  *                        group, C2 a multiple of 16 from 16 to 256 with 2 * 3 * (filters per merged group) + C2 <= 512,
  *                        and the resident pointwise weights (C_out * C2 * 4 bytes) must leave room for two input
  *                        stages.  "Supported" is not "faster than two launches": fusing pays on large planes
